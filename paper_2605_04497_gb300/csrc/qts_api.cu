@@ -3,6 +3,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <new>
 
 #include "qts_device.cuh"
 #include "qts_internal.h"
@@ -70,6 +71,7 @@ void release_device(qts_ensemble* e) {
     e->device_bytes = 0;
     release_dfs(e);
     release_batch_tables(e);
+    release_blocks(e);
 }
 
 void release_batch_tables(qts_ensemble* e) {
@@ -168,6 +170,48 @@ qts_status ensure_batch_tables(qts_ensemble* e) {
     std::vector<Rec32>().swap(P.rec32);
     e->bready = true;
     return QTS_OK;
+}
+
+// Block tables: built from the host copy of the model; `grad` adds the adjoint's
+// part (the records are the same either way, so they are kept).
+qts_status ensure_blocks(qts_ensemble* e, bool grad) {
+    if (e->blk_ready && (!grad || e->blk_grad_ready)) return QTS_OK;
+    if (grad && e->n_nodes >= ((int64_t)1 << 31)) return fail(QTS_ERR_UNSUPPORTED, "gradients of 2^31 nodes or more");
+    BlockHost H;
+    try {
+        build_blocks(e, grad, &H);
+    } catch (const std::bad_alloc&) {
+        return fail(QTS_ERR_OOM, "host allocation of the block tables");
+    }
+    if (grad && H.n_slots >= ((int64_t)1 << 32)) return fail(QTS_ERR_UNSUPPORTED, "too many adjoint sums");
+    int64_t tot = 0;
+    qts_status st = QTS_OK;
+    if (!e->blk_ready) st = up(&e->blkdev.rec, H.rec, &tot, "upload block tables");
+    if (grad) {
+        if (st == QTS_OK) st = up(&e->blkdev.ent, H.ent, &tot, "upload block tables");
+        e->blkdev.n_ent = (int64_t)H.ent.size();
+        if (st == QTS_OK) st = up(&e->blkdev.bias_leaf, H.bias_leaf, &tot, "upload block tables");
+        if (st == QTS_OK) st = up(&e->blkdev.bias_z, H.bias_z, &tot, "upload block tables");
+    }
+    if (st != QTS_OK) {
+        release_blocks(e);
+        return st;
+    }
+    e->blk = std::move(H.buckets);
+    e->n_blocks = H.n_blocks;
+    e->n_blk_slots = H.n_slots;
+    e->blk_ready = true;
+    e->blk_grad_ready = e->blk_grad_ready || grad;
+    return QTS_OK;
+}
+
+void release_blocks(qts_ensemble* e) {
+    BlockDev& T = e->blkdev;
+    for (void* p : {(void*)T.rec, (void*)T.ent, (void*)T.bias_leaf, (void*)T.bias_z}) cudaFree(p);
+    T = BlockDev();
+    e->blk.clear();
+    e->n_blocks = e->n_blk_slots = 0;
+    e->blk_ready = e->blk_grad_ready = false;
 }
 
 qts_status ensure_workspace(qts_ensemble* e, size_t bytes) {
@@ -350,8 +394,16 @@ qts_status qts_shap_values(qts_ensemble* e, const float* X, int64_t M, int32_t F
     if (M == 0) return QTS_OK;
     if (!phi) return fail(QTS_ERR_ARG, "phi is NULL");
     cudaStream_t s = (cudaStream_t)stream;
-    // FP32 runs on the pair tables (built on the first call that needs them)
+    // FP32 runs on the block tables, or for a few samples on the pair tables
+    // (either built on the first call that needs them)
     const bool fp64 = (e->flags & QTS_FLAG_FP64) != 0;
+    if (!fp64 && M > kFewRows) {
+        st = ensure_blocks(e, false);
+        if (st != QTS_OK) return st;
+        cudaError_t ce = launch_phi_init(phi, M, F, e->prep.bias, s);
+        if (ce == cudaSuccess) ce = launch_fwd_blocks(e, X, M, F, n_quad, phi, s);
+        return ce == cudaSuccess ? QTS_OK : cuda_fail(ce, "forward kernel launch");
+    }
     if (!fp64) {
         st = ensure_batch_tables(e);
         if (st != QTS_OK) return st;

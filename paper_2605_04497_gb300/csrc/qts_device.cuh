@@ -134,7 +134,7 @@ __device__ __forceinline__ bool satisfies(float x, float lo, float hi, uint32_t 
 namespace qts {
 
 // Block-level path streaming.  The block's path range [p0, p1) of one bucket
-// (D elements + 1 header record per path) is copied into two shared staging
+// (`stride` records per path or block of leaves) is copied into two shared staging
 // buffers of `sub` paths each by bulk copies, double-buffered on two
 // mbarriers; visit(first_path_index, count, records) runs on every thread for
 // each staged sub-chunk.  Thread 0 does the bounded wait and broadcasts the
@@ -142,8 +142,8 @@ namespace qts {
 // reporting QTS_ERR_TIMEOUT and waiting, bounded, for the copies in flight) if
 // a copy did not complete.  Must be called by all threads; `bars` must have
 // been initialised by mbar_init(.., 1) and a __syncthreads.
-template <typename Rec, int D, typename Visit>
-__device__ __forceinline__ bool stream_chunks(const Rec* __restrict__ rec, int64_t p0, int64_t p1, int sub,
+template <typename Rec, typename Visit>
+__device__ __forceinline__ bool stream_chunks(const Rec* __restrict__ rec, int stride, int64_t p0, int64_t p1, int sub,
                                               Rec* st0, Rec* st1, uint64_t* bars, uint32_t* phase_base,
                                               int* s_flag, int* status, Visit&& visit) {
     const int nsub = (int)((p1 - p0 + sub - 1) / sub);
@@ -152,10 +152,10 @@ __device__ __forceinline__ bool stream_chunks(const Rec* __restrict__ rec, int64
     auto issue = [&](int c) {
         const int64_t q0 = p0 + (int64_t)c * sub;
         const int cnt = (int)imin64(sub, p1 - q0);
-        const uint32_t bytes = (uint32_t)cnt * (D + 1) * (uint32_t)sizeof(Rec);
+        const uint32_t bytes = (uint32_t)cnt * stride * (uint32_t)sizeof(Rec);
         uint64_t* bar = &bars[c & 1];
         mbar_arrive_expect_tx(bar, bytes);
-        bulk_g2s((c & 1) ? (void*)st1 : (void*)st0, rec + q0 * (D + 1), bytes, bar);
+        bulk_g2s((c & 1) ? (void*)st1 : (void*)st0, rec + q0 * stride, bytes, bar);
     };
     if (threadIdx.x == 0)
         for (int c = 0; c < 2 && c < nsub; ++c) issue(c);
@@ -192,16 +192,23 @@ __device__ __forceinline__ bool stream_chunks(const Rec* __restrict__ rec, int64
 
 // Lane = sample: warp w calls body(global_path_index, records) for paths w,
 // w + nwarps, ... of each staged sub-chunk (every path, when every_warp).
+template <typename Rec, typename Body>
+__device__ __forceinline__ bool stream_records(const Rec* __restrict__ rec, int stride, int64_t p0, int64_t p1,
+                                               int sub, Rec* st0, Rec* st1, uint64_t* bars, uint32_t* phase_base,
+                                               int* s_flag, int* status, Body&& body, bool every_warp = false) {
+    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    return stream_chunks<Rec>(rec, stride, p0, p1, sub, st0, st1, bars, phase_base, s_flag, status,
+                              [&](int64_t q0, int cnt, const Rec* buf) {
+                                  const int i0 = every_warp ? 0 : warp, di = every_warp ? 1 : nwarps;
+                                  for (int i = i0; i < cnt; i += di) body(q0 + i, buf + i * stride);
+                              });
+}
+
 template <typename Rec, int D, typename Body>
 __device__ __forceinline__ bool stream_paths(const Rec* __restrict__ rec, int64_t p0, int64_t p1, int sub,
                                              Rec* st0, Rec* st1, uint64_t* bars, uint32_t* phase_base,
                                              int* s_flag, int* status, Body&& body, bool every_warp = false) {
-    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    return stream_chunks<Rec, D>(rec, p0, p1, sub, st0, st1, bars, phase_base, s_flag, status,
-                                 [&](int64_t q0, int cnt, const Rec* buf) {
-                                     const int i0 = every_warp ? 0 : warp, di = every_warp ? 1 : nwarps;
-                                     for (int i = i0; i < cnt; i += di) body(q0 + i, buf + i * (D + 1));
-                                 });
+    return stream_records<Rec>(rec, D + 1, p0, p1, sub, st0, st1, bars, phase_base, s_flag, status, body, every_warp);
 }
 
 // Lane = (path, sample), for calls with few samples: warp w takes `group`

@@ -134,6 +134,33 @@ struct DevTables {
     int64_t bytes = 0;
 };
 
+// Block tables of the FP32 first-order and adjoint passes (layout: qts_blocks.h).
+struct BlockBucket {  // all blocks of one width and height
+    int D = 0, h = 0;
+    int dmax = 0;           // most unique features on a path of theirs
+    int64_t n = 0;
+    int64_t rec_off = 0;    // first record
+    int64_t slot_off = 0;   // first adjoint sum (n * (D + blk_slots(h)) of them)
+};
+struct BlockEntry {  // one term of a gradient: += coef * the block's sum
+    uint32_t slot;   // index of the sum among all blocks' slots
+    uint32_t target; // node << 1 | (1: d_leaf, 0: d_z)
+    double coef;
+};
+struct BlockHost {
+    std::vector<BlockBucket> buckets;
+    std::vector<Rec32> rec;
+    std::vector<BlockEntry> ent;       // adjoint only, as the rest
+    std::vector<double> bias_leaf, bias_z;  // per node: d E[f] / d leaf value, d z
+    int64_t n_blocks = 0, n_slots = 0;
+};
+struct BlockDev {
+    Rec32* rec = nullptr;
+    BlockEntry* ent = nullptr;
+    int64_t n_ent = 0;
+    double *bias_leaf = nullptr, *bias_z = nullptr;
+};
+
 // Launch tuning of one bucket width.
 struct Tune {
     int warps = 4;        // warps per block (samples are shared, paths split)
@@ -195,6 +222,12 @@ struct qts_ensemble {
     qts::Prepared bprep;
     qts::DevTables bdev;
     bool bready = false;
+    // block tables of the FP32 first-order and adjoint passes, built on the
+    // first call that needs them (the adjoint's part on the first such call)
+    std::vector<qts::BlockBucket> blk;
+    qts::BlockDev blkdev;
+    int64_t n_blocks = 0, n_blk_slots = 0;
+    bool blk_ready = false, blk_grad_ready = false;
     // per-width launch tuning (index = bucket width)
     qts::Tune tune[qts::kMaxD + 1];
     bool tuned = false;
@@ -212,6 +245,10 @@ void release_device(qts_ensemble* e);
 void release_dfs(qts_ensemble* e);      // drop the depth-first program (rebuilt on demand)
 qts_status ensure_batch_tables(qts_ensemble* e);  // build the pair tables of the batched pass
 void release_batch_tables(qts_ensemble* e);
+// build the block tables, with grad those of the adjoint too
+void build_blocks(const qts_ensemble* e, bool grad, BlockHost* out);
+qts_status ensure_blocks(qts_ensemble* e, bool grad);
+void release_blocks(qts_ensemble* e);
 int num_sms();
 void batch_forget(const qts_ensemble* e);  // drop cached batched graphs using e
 
@@ -252,6 +289,9 @@ cudaError_t launch_phi_init(double* phi, int64_t M, int F, double bias, cudaStre
 cudaError_t launch_wait_selftest(int* status, cudaStream_t st);
 cudaError_t launch_fwd_bucket(const qts_ensemble* e, const Bucket& b, const float* X, int64_t M,
                               int F, const QuadF& q, const QuadD& qd, double* phi, const Tune& tn,
+                              cudaStream_t st);
+// first-order values of more than kFewRows samples on the block tables
+cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* phi,
                               cudaStream_t st);
 // pairs: b is a bucket of the sibling-pair tables (e->bprep), else of e->prep
 cudaError_t launch_int_bucket(const qts_ensemble* e, const Bucket& b, bool pairs, const float* X, int64_t M,
