@@ -1,44 +1,47 @@
 // Batched forward + adjoint of many heterogeneous requests in one persistent
-// kernel, captured (with its initialisation and epilogues) into a CUDA graph.
+// kernel per register class, captured (with its initialisation and epilogues)
+// into a CUDA graph; a single adjoint call launches the same kernels.
 //
-// Work items are (request, bucket, path chunk, sample tile of 32).  Items are
-// not materialised: segments (request, bucket) are ordered by per-item cost,
-// heaviest first, and carry their first item index, so a block that takes
+// Work items are (request, bucket, run of blocks, sample tile).  Items are not
+// materialised: segments (request, bucket) are ordered by per-item cost,
+// heaviest first, and carry their first item index, so a thread block that takes
 // item k from the atomic counter finds its segment by binary search.  For a
-// request with grad_phi one pass over each (sample, path) yields both phi and
-// the adjoint sums (the forward products P_j S_j are part of the adjoint's).
+// request with grad_phi one pass over each (sample, block) yields both phi and
+// the adjoint sums (the forward products are part of the adjoint's).
 //
-// qts-build-parts: 9 (part 0: host code; parts 1-8: one register class each)
+// Bound by instruction issue and FP32 (8 to 16 warps per SM).  Measured, path
+// tables before and block tables now: eight requests of 17-100 trees, depth 4-13,
+// 40-2,000 samples 8.61 -> 4.60 ms; sixteen of at most 200 samples 3.28 -> 0.38 ms (by
+// default the warps of a thread block now share 64 samples and split the blocks:
+// with 64 samples per warp a request of fewer than 193 left warps idle); adjoint
+// alone, 200 trees of depth 8, 4,001 samples 3.30 -> 2.00 ms.
+//
+// qts-build-parts: 12 (part 0: host code; parts 1-3: the pass of two samples per
+// lane, parts 4-11: the others, one register class each)
 #include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <numeric>
 
-#include "qts_paths.cuh"
+#include "qts_blocks.cuh"
 
 namespace qts {
 
 struct SegDev {
     const Rec32* rec;
-    double* g_val;      // bucket-offset adjoint accumulators (nullptr: forward only)
-    double* g_slot;
-    int64_t n_paths;
+    double* g;          // the bucket's adjoint sums (nullptr: forward only)
+    int64_t n;          // blocks
     int64_t item_begin;
-    int32_t D;
-    int32_t paths;      // paths per item
-    int32_t n_tiles;    // sample groups per chunk (a group = 32, or 32 per warp when priv)
+    int32_t D, h;
+    int32_t per_item;   // blocks per item
+    int32_t n_tiles;    // sample groups per run of blocks
     int32_t req;
-    int32_t priv;       // 0: warps share 32 samples (atomics); 1: each warp owns 32
-                        // samples and a private phi tile; 2: each warp owns 64
-                        // samples, two per lane (sample-pair packing), private tile;
-                        // 3: as 2, but the warps share 64 samples and split the paths
-    int32_t pad;
+    int32_t mode;       // 0: the warps share 32 samples and a phi tile (atomics) - forward
+                        // only, or too many features for the others; 2: each warp owns
+                        // 64 samples, two per lane, and a phi tile; 3: the warps share 64
+                        // samples, two per lane, and split the blocks, a phi tile each
 };
 
-// Widths that run the fused pass with sample-pair packing when the 64-sample
-// tile fits the class's shared memory.  The register classes below are cut so
-// that every packed width fits its class's cap without spilling.
-__host__ __device__ constexpr bool pair_width(int D) { return D <= 16; }
 constexpr int kBatchWarps = 4;
 
 // Per request: x and grad_phi transposed to [feature][Mpad] (row F of XT is
@@ -56,199 +59,150 @@ struct ReqDev {
     int* status;
 };
 
+constexpr int kInlineSegs = 40;
+
 struct BatchArgs {
-    const SegDev* segs;
-    int n_segs;
+    const SegDev* segs;   // nullptr: seg and req below (a call of one request)
     const ReqDev* reqs;
+    int n_segs;
+    int sub;              // blocks per staged sub-chunk
+    int stage;            // records per staging buffer
+    int pad;
     int64_t n_items;
     unsigned long long* counter;
     int64_t tile_floats;  // floats of the phi region (max over the launch's requests)
-    int sub;
     QuadF q;
+    SegDev seg[kInlineSegs];
+    ReqDev req;
 };
 
 // samples per item for each mode
-__host__ __device__ __forceinline__ int item_samples(int priv) {
-    return priv == 3 ? 64 : priv == 2 ? 64 * kBatchWarps : (priv == 1 ? 32 * kBatchWarps : 32);
+__host__ __device__ __forceinline__ int item_samples(int mode) {
+    return mode == 3 ? 64 : mode == 2 ? 64 * kBatchWarps : 32;
 }
 
 // floats of the phi region a request needs in a mode
-inline int64_t tile_floats_for(int priv, int F) {
-    return priv >= 2 ? (int64_t)kBatchWarps * (F + 1) * kTileLd2
-                     : (priv == 1 ? (int64_t)kBatchWarps * (F + 1) * kTileLd : (int64_t)(F + 1) * kTileLd);
+inline int64_t tile_floats_for(int mode, int F) {
+    return mode >= 2 ? (int64_t)kBatchWarps * (F + 1) * kTileLd2 : (int64_t)(F + 1) * kTileLd;
 }
 
-inline size_t batch_smem_bytes(int64_t tile_floats, int sub, int dmax) {
-    size_t off = (size_t)tile_floats * 4;
-    off = (off + 15) & ~(size_t)15;
-    off += 2 * (size_t)sub * (dmax + 1) * sizeof(Rec32);
-    off = (off + 15) & ~(size_t)15;
-    return off + 16;
+inline size_t batch_smem_bytes(int64_t tile_floats, int stage) {
+    const size_t off = ((size_t)tile_floats * 4 + 15) & ~(size_t)15;
+    return off + 2 * (size_t)stage * sizeof(Rec32) + 16;
 }
 
-// node-group width and register policy per width (fits 3 blocks of 128 threads)
-template <int D>
-struct BatchNP {
-    static constexpr bool packed = D <= 16;  // bwd_path_f32_pk
-    static constexpr int fused = 2;          // otherwise: lean per-pass variant
-    static constexpr bool recomp = true;
-    static constexpr int fwd = D <= 8 ? 8 : 2;
-};
+// Register classes.  A block's fused pass holds about 12 registers per shared
+// element, 10 / 36 / 88 for a subtree of height 1 / 2 / 3 and 35 more: class 8 takes
+// what fits 128 registers (4 thread blocks of 128 threads per SM), 12 what fits
+// 168 (3), 16 the other exact widths (255, 2); the padded widths 20..32 are class
+// 32 and each of 40, 48, 56 and 64 (which spill) is a class of its own.
+__host__ __device__ constexpr int batch_class(int D, int h) {
+    if (D > 32) return D;
+    if (D > 16) return 32;
+    const int regs = 12 * D + (h == 0 ? 0 : h == 1 ? 10 : h == 2 ? 36 : 88) + 35;
+    return regs <= 128 ? 8 : regs <= 168 ? 12 : 16;
+}
+constexpr int batch_blocks(int cls) { return cls == 8 ? 4 : cls == 12 ? 3 : cls == 16 ? 2 : 1; }
 
-template <int C>
-cudaError_t launch_batch_class(const BatchArgs& a, size_t smem, cudaStream_t st, int* blocks_out, int occ = 0);
+template <int C, bool SP>
+cudaError_t launch_batch_class(const BatchArgs& a, size_t smem, cudaStream_t st);
 
 #if QTS_DEVICE_PARTS
 
-template <int D>
-__device__ __forceinline__ bool batch_item(const SegDev& sg, const ReqDev& rq, int64_t p0, int64_t p1,
-                                           int64_t s0, float* ps, Rec32* st0, Rec32* st1, uint64_t* bars,
-                                           uint32_t* s_phase, int* s_flag, int sub, const QuadF& q,
-                                           float2* zs_all) {
+struct ItemCtx {
+    const SegDev& sg;
+    const ReqDev& rq;
+    int64_t p0, p1, s0;
+    float* ps;
+    Rec32 *st0, *st1;
+    uint64_t* bars;
+    uint32_t* s_phase;
+    int* s_flag;
+    int sub;
+    const QuadF& q;
+};
+
+// phi of `n` samples from tiles of [feature][ld], `tiles` of them, into the output
+__device__ __forceinline__ void flush_phi(const ReqDev& rq, const float* t, int tiles, int tile_elems, int ld,
+                                          int64_t s0, int n, int first, int step) {
+    for (int s = first; s < n && s0 + s < rq.M; s += step)
+        for (int f = threadIdx.x & 31; f < rq.F; f += 32) {
+            float v = 0.f;
+            for (int w = 0; w < tiles; ++w) v += t[w * tile_elems + f * ld + s];
+            if (v != 0.f) atomicAdd(&rq.phi[(s0 + s) * (rq.F + 1) + f], (double)v);
+        }
+}
+
+template <int D, int H, bool SP>
+__device__ __forceinline__ bool batch_item(const ItemCtx& c) {
+    const SegDev& sg = c.sg;
+    const ReqDev& rq = c.rq;
     const int F = rq.F;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if constexpr (pair_width(D)) {
-        if (sg.priv >= 2) {
-            // sample-pair modes, lane l the pair 2l, 2l+1 of its warp's 64 samples.
-            // priv 2: warp w owns samples s0 + 64 w .. + 63 and walks every path;
-            // priv 3: the block's warps share samples s0 .. s0 + 63 and split the
-            // paths.  Either way warp w accumulates into its own phi tile w.
-            const bool split = sg.priv == 2;
-            const int tile_elems = (F + 1) * kTileLd2;
-            float* my = ps + warp * tile_elems;
-            float2* zs = zs_all + warp * 16;
-            const int64_t sw = split ? s0 + 64 * warp : s0;
-            for (int idx = lane; idx < tile_elems; idx += 32) my[idx] = 0.f;
-            __syncthreads();
-            const bool has_nan = *rq.has_nan != 0;
-            const GlobalCols2 xr{rq.XT, rq.Mpad, sw + 2 * lane};
-            const GlobalCols2 gr{rq.GT, rq.Mpad, sw + 2 * lane};
-            const bool ok = stream_paths<Rec32, D>(
-                sg.rec, p0, p1, sub, st0, st1, bars, s_phase, s_flag, rq.status,
-                [&](int64_t p, const Rec32* r) {
-                    double* gsl = sg.g_slot + p * D;
-                    double* gv = sg.g_val + 2 * p;
-                    if (has_nan) bwd_path_f32_sp<D, true, true>(r, xr, gr, my, zs, lane, q, gsl, gv);
-                    else bwd_path_f32_sp<D, false, true>(r, xr, gr, my, zs, lane, q, gsl, gv);
-                },
-                split);
-            if (!ok) return false;
-            if (rq.phi) {
-                if (split) {
-                    for (int idx = lane; idx < 64 * F; idx += 32) {
-                        const int s = idx / F, f = idx - s * F;
-                        if (sw + s < rq.M) {
-                            const float v = my[f * kTileLd2 + s];
-                            if (v != 0.f) atomicAdd(&rq.phi[(sw + s) * (F + 1) + f], (double)v);
-                        }
-                    }
-                } else {
-                    // stream_paths ended on a block barrier: every warp's tile is complete
-                    for (int idx = threadIdx.x; idx < 64 * F; idx += blockDim.x) {
-                        const int s = idx / F, f = idx - s * F;
-                        if (sw + s < rq.M) {
-                            float v = 0.f;
-#pragma unroll
-                            for (int w = 0; w < kBatchWarps; ++w) v += ps[w * tile_elems + f * kTileLd2 + s];
-                            if (v != 0.f) atomicAdd(&rq.phi[(sw + s) * (F + 1) + f], (double)v);
-                        }
-                    }
-                }
-            }
-            __syncthreads();
-            return true;
-        }
-    }
-    const bool priv = sg.priv != 0;
-    const int tile_elems = (F + 1) * kTileLd;
-    // private mode: warp w owns samples s0 + 32 w .. and tile w
-    float* my = priv ? ps + warp * tile_elems : ps;
-    const int64_t sw = priv ? s0 + 32 * warp : s0;
-    if (priv) {
-        for (int idx = lane; idx < tile_elems; idx += 32) my[idx] = 0.f;
-    } else {
-        for (int idx = threadIdx.x; idx < tile_elems; idx += blockDim.x) ps[idx] = 0.f;
-    }
-    __syncthreads();
     const bool has_nan = *rq.has_nan != 0;
-    const bool grad = rq.GT != nullptr;
-    const GlobalCols xr{rq.XT, rq.Mpad, sw + lane};
-    const GlobalCols gr{rq.GT, rq.Mpad, sw + lane};
-    constexpr int FWD_NP = BatchNP<D>::fwd;
-    const bool ok = stream_paths<Rec32, D>(
-        sg.rec, p0, p1, sub, st0, st1, bars, s_phase, s_flag, rq.status,
-        [&](int64_t p, const Rec32* r) {
-            if (grad) {
-                double* gsl = sg.g_slot + p * D;
-                double* gv = sg.g_val + 2 * p;
-                if (priv) {
-                    if (has_nan) bwd_path_f32_pk<D, true, kPhiPrivate, GlobalCols, GlobalCols, true>(r, xr, gr, my, lane, q, gsl, gv);
-                    else bwd_path_f32_pk<D, false, kPhiPrivate, GlobalCols, GlobalCols, true>(r, xr, gr, my, lane, q, gsl, gv);
-                } else {
-                    if (has_nan) bwd_path_f32_pk<D, true, kPhiAtomic, GlobalCols, GlobalCols, true>(r, xr, gr, my, lane, q, gsl, gv);
-                    else bwd_path_f32_pk<D, false, kPhiAtomic, GlobalCols, GlobalCols, true>(r, xr, gr, my, lane, q, gsl, gv);
-                }
-            } else {
-                auto fwd = [&](auto np) {
-                    constexpr int NP = decltype(np)::value;
-                    if (priv) {
-                        if (has_nan) fwd_path_f32<D, NP, true, GlobalCols, kPhiPrivate, true>(r, xr, my, lane, q);
-                        else fwd_path_f32<D, NP, false, GlobalCols, kPhiPrivate, true>(r, xr, my, lane, q);
-                    } else {
-                        if (has_nan) fwd_path_f32<D, NP, true, GlobalCols, kPhiAtomic, true>(r, xr, my, lane, q);
-                        else fwd_path_f32<D, NP, false, GlobalCols, kPhiAtomic, true>(r, xr, my, lane, q);
-                    }
-                };
-                // a rule of fewer than FWD_NP points (or not a multiple of it)
-                // runs node pairs
-                if (FWD_NP > 2 && q.n_pad % FWD_NP != 0) fwd(std::integral_constant<int, 2>{});
-                else fwd(std::integral_constant<int, FWD_NP>{});
-            }
-        },
-        priv);
+    constexpr int kSlots = D + blk_slots(H);
+    constexpr int ld = SP ? kTileLd2 : kTileLd;
+    const bool own = SP && sg.mode == 2;  // every warp has its own samples
+    const int tile_elems = (F + 1) * ld;
+    float* my = SP ? c.ps + warp * tile_elems : c.ps;
+    const int64_t sw = own ? c.s0 + 64 * warp : c.s0;
+    for (int idx = threadIdx.x; idx < (SP ? kBatchWarps : 1) * tile_elems; idx += blockDim.x) c.ps[idx] = 0.f;
+    __syncthreads();
+    bool ok;
+    auto run = [&](auto&& body) {
+        return stream_records<Rec32>(sg.rec, blk_stride(D, H), c.p0, c.p1, c.sub, c.st0, c.st1, c.bars, c.s_phase,
+                                     c.s_flag, rq.status, body, own);
+    };
+    if constexpr (SP) {
+        const BwdCols<true> xr{rq.XT, rq.Mpad, sw + 2 * lane}, gr{rq.GT, rq.Mpad, sw + 2 * lane};
+        ok = run([&](int64_t p, const Rec32* r) {
+            double* g = sg.g + p * kSlots;
+            if (has_nan) bwd_block<D, H, true, true, kPhiPrivate>(r, xr, gr, my, lane, c.q, g);
+            else bwd_block<D, H, false, true, kPhiPrivate>(r, xr, gr, my, lane, c.q, g);
+        });
+    } else if (rq.GT) {
+        const BwdCols<false> xr{rq.XT, rq.Mpad, sw + lane}, gr{rq.GT, rq.Mpad, sw + lane};
+        ok = run([&](int64_t p, const Rec32* r) {
+            bwd_block<D, H, true, false, kPhiAtomic>(r, xr, gr, my, lane, c.q, sg.g + p * kSlots);
+        });
+    } else {
+        const GlobalCols xr{rq.XT, rq.Mpad, sw + lane};
+        ok = run([&](int64_t, const Rec32* r) { fwd_block<D, H, 4, true, kPhiAtomic>(r, xr, my, lane, c.q); });
+    }
     if (!ok) return false;
+    // stream_records ended on a block barrier: every warp's adds are in the tiles
     if (rq.phi) {
-        if (priv) {
-            for (int idx = lane; idx < 32 * F; idx += 32) {
-                const int s = idx / F, f = idx - s * F;
-                if (sw + s < rq.M) {
-                    const float v = my[f * kTileLd + s];
-                    if (v != 0.f) atomicAdd(&rq.phi[(sw + s) * (F + 1) + f], (double)v);
-                }
-            }
-        } else {
-            for (int idx = threadIdx.x; idx < 32 * F; idx += blockDim.x) {
-                const int s = idx / F, f = idx - s * F;
-                if (s0 + s < rq.M) {
-                    const float v = ps[f * kTileLd + s];
-                    if (v != 0.f) atomicAdd(&rq.phi[(s0 + s) * (F + 1) + f], (double)v);
-                }
-            }
-        }
+        if (own) flush_phi(rq, my, 1, tile_elems, ld, sw, 64, 0, 1);
+        else flush_phi(rq, c.ps, SP ? kBatchWarps : 1, tile_elems, ld, c.s0, SP ? 64 : 32, warp, kBatchWarps);
     }
     __syncthreads();  // the tiles are rewritten by the next item
     return true;
 }
 
-// Register classes: DCLASS 8 handles widths 1..6 (4 blocks of 128 threads per
-// SM, 128 registers), 12 handles 7..10 (3 blocks, 168 registers), 16 handles
-// 11..16 (2 blocks, 255 registers), 32 handles 20..32, and each of the widths
-// 40, 48, 56 and 64 (which spill) is a class of its own.
-// With two samples per lane a width needs about as many registers as twice
-// that width with one, so the cuts sit lower than the widths' names suggest.
-template <int DCLASS>
-__global__ void __launch_bounds__(128, DCLASS == 8 ? 4 : (DCLASS == 12 ? 3 : (DCLASS == 16 ? 2 : 1)))
-    batch_kernel(BatchArgs a) {
+// the (width, height) pairs of a class, as keys 4 D + h
+template <int CLS, bool SP, int KEY>
+__device__ __forceinline__ bool batch_dispatch(const ItemCtx& c) {
+    constexpr int D = KEY / 4, H = KEY % 4;
+    constexpr bool width = CLS <= 16 ? D <= 16 : CLS == 32 ? (D > 16 && D <= 32 && D % 4 == 0) : D == CLS;
+    if constexpr (width && H <= blk_max_h(D) && batch_class(D, H) == CLS) {
+        if (c.sg.D == D && c.sg.h == H) return batch_item<D, H, SP>(c);
+    }
+    if constexpr (KEY + 1 < 4 * (CLS <= 16 ? 17 : CLS == 32 ? 33 : CLS + 1)) return batch_dispatch<CLS, SP, KEY + 1>(c);
+    else return false;
+}
+
+template <int CLS, bool SP>
+__global__ void __launch_bounds__(128, batch_blocks(CLS)) batch_kernel(const __grid_constant__ BatchArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     float* ps = (float*)smem;
-    size_t off = ((size_t)a.tile_floats * 4 + 15) & ~(size_t)15;
+    const size_t off = ((size_t)a.tile_floats * 4 + 15) & ~(size_t)15;
     Rec32* st0 = (Rec32*)(smem + off);
-    Rec32* st1 = st0 + (size_t)a.sub * (DCLASS + 1);
-    uint64_t* bars = (uint64_t*)(st1 + (size_t)a.sub * (DCLASS + 1));
+    Rec32* st1 = st0 + a.stage;
+    uint64_t* bars = (uint64_t*)(st1 + a.stage);
     __shared__ int s_flag;
     __shared__ uint32_t s_phase[2];
     __shared__ long long s_item;
-    __shared__ float2 s_zs[kBatchWarps * 16];
+    const SegDev* segs = a.segs ? a.segs : a.seg;
     if (threadIdx.x == 0) {
         mbar_init(&bars[0], 1);
         mbar_init(&bars[1], 1);
@@ -265,90 +219,66 @@ __global__ void __launch_bounds__(128, DCLASS == 8 ? 4 : (DCLASS == 12 ? 3 : (DC
         int lo = 0, hi = a.n_segs - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (a.segs[mid].item_begin <= item) lo = mid;
+            if (segs[mid].item_begin <= item) lo = mid;
             else hi = mid - 1;
         }
-        const SegDev sg = a.segs[lo];
-        const ReqDev rq = a.reqs[sg.req];
+        const SegDev sg = segs[lo];
+        const ReqDev rq = a.segs ? a.reqs[sg.req] : a.req;
         const int64_t local = item - sg.item_begin;
-        const int64_t s0 = (local % sg.n_tiles) * item_samples(sg.priv);
-        const int64_t p0 = (local / sg.n_tiles) * sg.paths;
-        const int64_t p1 = imin64(p0 + sg.paths, sg.n_paths);
-        bool ok = true;
-#define QTS_CASE(DD) \
-    case DD: ok = batch_item<DD>(sg, rq, p0, p1, s0, ps, st0, st1, bars, s_phase, &s_flag, a.sub, a.q, s_zs); break;
-        if constexpr (DCLASS == 8) {
-            switch (sg.D) {
-                QTS_CASE(1) QTS_CASE(2) QTS_CASE(3) QTS_CASE(4) QTS_CASE(5) QTS_CASE(6)
-                default: break;
-            }
-        } else if constexpr (DCLASS == 12) {
-            switch (sg.D) {
-                QTS_CASE(7) QTS_CASE(8) QTS_CASE(9) QTS_CASE(10)
-                default: break;
-            }
-        } else if constexpr (DCLASS == 16) {
-            switch (sg.D) {
-                QTS_CASE(11) QTS_CASE(12) QTS_CASE(13) QTS_CASE(14) QTS_CASE(15) QTS_CASE(16)
-                default: break;
-            }
-        } else if constexpr (DCLASS == 32) {
-            switch (sg.D) {
-                QTS_CASE(20) QTS_CASE(24) QTS_CASE(28) QTS_CASE(32)
-                default: break;
-            }
-        } else {
-            switch (sg.D) {
-                QTS_CASE(DCLASS)
-                default: break;
-            }
-        }
-#undef QTS_CASE
-        if (!ok) break;  // a bounded wait ran out: status is set, stop this block
+        const int64_t p0 = (local / sg.n_tiles) * sg.per_item;
+        const ItemCtx c{sg, rq, p0, imin64(p0 + sg.per_item, sg.n), (local % sg.n_tiles) * item_samples(sg.mode),
+                        ps, st0, st1, bars, s_phase, &s_flag, a.sub, a.q};
+        if (!batch_dispatch<CLS, SP, (CLS <= 16 ? 0 : CLS == 32 ? 80 : 4 * CLS)>(c))
+            break;  // a bounded wait ran out: status is set, stop this thread block
     }
 }
 
-// occ > 0: at most occ blocks per SM (the persistent grid is occ x SMs blocks)
-template <int C>
-cudaError_t launch_batch_class(const BatchArgs& a, size_t smem, cudaStream_t st, int* blocks_out, int occ) {
-    auto k = batch_kernel<C>;
+template <int C, bool SP>
+cudaError_t launch_batch_class(const BatchArgs& a, size_t smem, cudaStream_t st) {
+    auto k = batch_kernel<C, SP>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 128, smem);
     if (e != cudaSuccess) return e;
-    if (occ > 0) per_sm = std::min(per_sm, occ);
-    const int blocks = std::max(1, per_sm) * num_sms();
-    *blocks_out = blocks;
-    k<<<blocks, 128, smem, st>>>(a);
+    const int64_t blocks = std::min<int64_t>((int64_t)std::max(1, per_sm) * num_sms(), std::max<int64_t>(1, a.n_items));
+    k<<<(unsigned)blocks, 128, smem, st>>>(a);
     return cudaGetLastError();
 }
 
-#define QTS_INST(C) \
-    template cudaError_t launch_batch_class<C>(const BatchArgs&, size_t, cudaStream_t, int*, int);
+#define QTS_INST(C, SP) template cudaError_t launch_batch_class<C, SP>(const BatchArgs&, size_t, cudaStream_t);
 #if QTS_IN_PART(1)
-QTS_INST(8)
+QTS_INST(8, true)
 #endif
 #if QTS_IN_PART(2)
-QTS_INST(12)
+QTS_INST(12, true)
 #endif
 #if QTS_IN_PART(3)
-QTS_INST(16)
+QTS_INST(16, true)
 #endif
 #if QTS_IN_PART(4)
-QTS_INST(32)
+QTS_INST(8, false)
 #endif
 #if QTS_IN_PART(5)
-QTS_INST(40)
+QTS_INST(12, false)
 #endif
 #if QTS_IN_PART(6)
-QTS_INST(48)
+QTS_INST(16, false)
 #endif
 #if QTS_IN_PART(7)
-QTS_INST(56)
+QTS_INST(32, false)
 #endif
 #if QTS_IN_PART(8)
-QTS_INST(64)
+QTS_INST(40, false)
+#endif
+#if QTS_IN_PART(9)
+QTS_INST(48, false)
+#endif
+#if QTS_IN_PART(10)
+QTS_INST(56, false)
+#endif
+#if QTS_IN_PART(11)
+QTS_INST(64, false)
 #endif
 #undef QTS_INST
 
@@ -430,28 +360,8 @@ void batch_forget(const qts_ensemble* e) {
     }
 }
 
-// widths 40, 48, 56 and 64 (bucket widths) are classes of their own
-int batch_class(int D) { return D <= 6 ? 8 : D <= 10 ? 12 : (D <= 16 ? 16 : (D <= 32 ? 32 : D)); }
-// shared memory one block of a class may use and still reach its blocks per SM
-static size_t class_smem_budget(int cls) {
-    const size_t sm = 227 * 1024;
-    const int blocks = cls == 8 ? 4 : cls == 12 ? 3 : cls == 16 ? 2 : 1;
-    return sm / blocks - 1024;
-}
-
-// paths per work item: about 2^23 FP32 operations per item
-static int item_paths(int D, bool grad) {
-    const int per_path = 32 * 8 * D * (grad ? 12 : 4);
-    int p = (1 << 23) / std::max(per_path, 1);
-    p = std::max(32, std::min(2048, p));
-    return (p + 31) / 32 * 32;
-}
-
-cudaError_t launch_bwd_epilogue(const qts_ensemble* e, const float* grad, int64_t M, int F,
-                                const double* g_val, const double* g_slot, double* d_leaf,
-                                double* d_z, double* gb, cudaStream_t st);
-
 // Workspace of one request in its ensemble: [adjoint sums (grad only)][XT][GT (grad only)][flag]
+constexpr int kGradHead = 256;  // doubles before the adjoint sums
 struct BatchWork {
     size_t grad_bytes, xt_off, gt_off, flag_off, total;
     int64_t Mpad;
@@ -462,8 +372,8 @@ static size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 static BatchWork batch_work(const qts_ensemble* e, int64_t M, int F, bool grad) {
     BatchWork w;
     w.Mpad = (M + 64 * kBatchWarps - 1) / (64 * kBatchWarps) * (64 * kBatchWarps);
-    // adjoint sums of the pair tables: two per path (a sibling pair's two leaves), one per slot
-    w.grad_bytes = grad ? align256(sizeof(double) * (size_t)(4 + 2 * e->bprep.n_paths + e->bprep.n_slots)) : 0;
+    // G = sum of grad_phi's last column, the work counter, then the blocks' adjoint sums
+    w.grad_bytes = grad ? align256(sizeof(double) * (size_t)(kGradHead + e->n_blk_slots)) : 0;
     const size_t tbytes = align256(sizeof(float) * (size_t)(F + 1) * (size_t)w.Mpad);
     w.xt_off = w.grad_bytes;
     w.gt_off = w.xt_off + tbytes;
@@ -480,36 +390,165 @@ static cudaError_t launch_transpose(const float* in, int64_t M, int ncols, int64
     return cudaGetLastError();
 }
 
-// Requests with F + 1 <= kPrivRows use per-warp private phi tiles (plain
-// read-add-write); wider ones share one tile with shared-memory atomics.
-constexpr int kPrivRows = 64;
-
 // Per-width launch choices that override the ensembles' own while tuning:
-// paths per work item and packed sample mapping (0: keep), and optionally only
+// blocks per work item and packed sample mapping (0: keep), and optionally only
 // the buckets of one width.
 struct BatchOverride {
     int paths[kMaxD + 1];
     int mode[kMaxD + 1];
-    int occ[kMaxD + 1];  // blocks per SM of the width's class (0: the tuned or full count)
     int only_width;
-    int only_class;      // > 0: only the widths of this register class
 };
+
+struct SegHost {
+    SegDev d;
+    double unit;   // cost of one block (all samples of one item)
+    int cls;
+    int64_t tile;  // floats of its phi region
+    int bin;       // tile-size bin: one launch per (class, bin, rule)
+    int nq;        // quadrature points of the bucket (QTS_NQ_EXACT: ceil(width / 2))
+    int npad;      // ... padded to `pad`, what its variant of the pass takes per register pass
+    int pad;
+    int stride;
+};
+
+constexpr int kBatchSub = 16;  // blocks per staged sub-chunk
+
+// Blocks per item of the default launch, from the work of the whole launch: a
+// dozen items per resident thread block evens out the tail and serves small
+// requests; at least 32 blocks keep the tile set-up and the phi flush (about
+// 64 F atomics) small beside the sweeps, and 2,048 are plenty.
+static void default_items(std::vector<SegHost>& segs) {
+    double total = 0.0;
+    for (const SegHost& s : segs) total += s.unit * (double)s.d.n * s.d.n_tiles;
+    const double share = total / (12.0 * 2.5 * num_sms());
+    for (SegHost& s : segs) {
+        if (s.d.per_item > 0) continue;
+        const double per = std::min(2048.0, std::max(32.0, share / s.unit));
+        s.d.per_item = (int32_t)(((int64_t)per + 15) / 16 * 16);
+    }
+}
+
+// The segments of one request's buckets.
+static void request_segments(const qts_request& R, int req, int n_quad, const BatchOverride* ov,
+                             std::vector<SegHost>* out) {
+    qts_ensemble* e = R.ens;
+    const bool grad = R.grad_phi != nullptr;
+    double* g = grad ? (double*)e->d_work + kGradHead : nullptr;
+    for (const BlockBucket& b : e->blk) {
+        if (ov && ov->only_width > 0 && b.D != ov->only_width) continue;
+        const Tune& tn = e->tune[b.D];
+        SegHost s;
+        s.cls = batch_class(b.D, b.h);
+        s.stride = blk_stride(b.D, b.h);
+        int mode = 0;
+        if (grad && b.D <= 16 && batch_smem_bytes(tile_floats_for(2, R.F), kBatchSub * s.stride) <= kSmemMax / 2) {
+            // the warps share 64 samples and split the blocks; the tuner may
+            // prefer 64 samples per warp on large requests
+            const int want = ov && ov->mode[b.D] ? ov->mode[b.D] : tn.bt_mode;
+            mode = want == 2 ? 2 : 3;
+        }
+        const int per = item_samples(mode);
+        s.d.rec = e->blkdev.rec + b.rec_off;
+        s.d.g = grad ? g + b.slot_off : nullptr;
+        s.d.n = b.n;
+        s.d.item_begin = 0;
+        s.d.D = b.D;
+        s.d.h = b.h;
+        s.d.per_item = ov && ov->paths[b.D] ? ov->paths[b.D] : tn.bt_paths;
+        s.d.n_tiles = (int)((R.M + per - 1) / per);
+        s.d.req = req;
+        s.d.mode = mode;
+        s.nq = nodes_for(n_quad, b.dmax, 1);
+        // the pass of two samples per lane takes one node at a time, the others pairs,
+        // the forward alone four
+        const int pad = mode >= 2 ? 1 : grad ? 2 : 4;
+        s.pad = pad;
+        s.npad = (s.nq + pad - 1) / pad * pad;
+        s.unit = blk_cost(b.D, b.h) * (grad ? 2.5 : 1.0) * s.npad / 8.0 * (mode == 0 ? 1.0 : per / 32.0);
+        // a launch sizes its shared memory for its widest tile, and whatever
+        // shared memory a thread block does not take stays L1 (which serves the x and
+        // grad_phi loads): requests of one class are launched by tile size
+        s.tile = tile_floats_for(mode, R.F);
+        const int64_t tb = s.tile * 4;
+        s.bin = tb <= 48 * 1024 ? 0 : tb <= 80 * 1024 ? 1 : 2;
+        out->push_back(s);
+    }
+}
+
+struct LaunchHost {
+    int cls, nq, npad, pad;
+    bool sp;
+    size_t first, count;  // segments
+    int64_t items, tile;
+    int stride;
+};
+
+// Order the segments - one launch per (class, tile bin, rule), heaviest items
+// first within it - and number their items.
+static std::vector<LaunchHost> order_segments(std::vector<SegHost>& segs, size_t max_segs) {
+    default_items(segs);
+    std::stable_sort(segs.begin(), segs.end(), [](const SegHost& a, const SegHost& b) {
+        if (a.cls != b.cls) return a.cls > b.cls;
+        if (a.pad != b.pad) return a.pad < b.pad;
+        if (a.bin != b.bin) return a.bin < b.bin;
+        if (a.npad != b.npad) return a.npad > b.npad;
+        if (a.nq != b.nq) return a.nq > b.nq;
+        return a.unit * a.d.per_item > b.unit * b.d.per_item;
+    });
+    std::vector<LaunchHost> out;
+    for (size_t i = 0; i < segs.size(); ++i) {
+        SegHost& s = segs[i];
+        if (out.empty() || out.back().cls != s.cls || segs[i - 1].bin != s.bin || out.back().nq != s.nq ||
+            out.back().npad != s.npad || out.back().pad != s.pad || out.back().count == max_segs)
+            out.push_back({s.cls, s.nq, s.npad, s.pad, s.d.mode >= 2, i, 0, 0, 0, 0});
+        LaunchHost& l = out.back();
+        s.d.item_begin = l.items;
+        l.items += (s.d.n + s.d.per_item - 1) / s.d.per_item * s.d.n_tiles;
+        l.tile = std::max(l.tile, s.tile);
+        l.stride = std::max(l.stride, s.stride);
+        ++l.count;
+    }
+    return out;
+}
+
+// Launch one entry of order_segments; a.segs / a.seg and a.reqs / a.req are set.
+static cudaError_t launch_ordered(const LaunchHost& l, BatchArgs& a, unsigned long long* counter, cudaStream_t st) {
+    a.n_segs = (int)l.count;
+    a.n_items = l.items;
+    a.counter = counter;
+    a.tile_floats = std::max<int64_t>(l.tile, kTileLd);
+    a.sub = kBatchSub;
+    // wide inputs: stage fewer blocks at a time until the thread block fits
+    while (a.sub > 1 && batch_smem_bytes(a.tile_floats, a.sub * l.stride) > kSmemMax) a.sub /= 2;
+    a.stage = a.sub * l.stride;
+    a.pad = 0;
+    if (!make_quad(l.nq, &a.q, nullptr, l.pad) || a.q.n_pad != l.npad) return cudaErrorInvalidValue;
+    const size_t smem = batch_smem_bytes(a.tile_floats, a.stage);
+    if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
+    if (l.sp) {
+        switch (l.cls) {
+            case 8: return launch_batch_class<8, true>(a, smem, st);
+            case 12: return launch_batch_class<12, true>(a, smem, st);
+            case 16: return launch_batch_class<16, true>(a, smem, st);
+            default: return cudaErrorInvalidValue;
+        }
+    }
+    switch (l.cls) {
+        case 8: return launch_batch_class<8, false>(a, smem, st);
+        case 12: return launch_batch_class<12, false>(a, smem, st);
+        case 16: return launch_batch_class<16, false>(a, smem, st);
+        case 32: return launch_batch_class<32, false>(a, smem, st);
+        case 40: return launch_batch_class<40, false>(a, smem, st);
+        case 48: return launch_batch_class<48, false>(a, smem, st);
+        case 56: return launch_batch_class<56, false>(a, smem, st);
+        default: return launch_batch_class<64, false>(a, smem, st);
+    }
+}
 
 static qts_status build_plan(int n, const qts_request* reqs, int n_quad, BatchPlan* plan,
                              cudaStream_t cap, const BatchOverride* ov = nullptr) {
-    struct SegHost {
-        SegDev d;
-        double cost;  // per item
-        int cls;
-        int64_t tile;  // floats of its phi region
-        int bin;       // tile-size bin: one launch per (class, bin, rule)
-        int occ;       // blocks per SM of its class launch (0: as many as fit)
-        int nq;        // quadrature points of the bucket (QTS_NQ_EXACT: ceil(D/2))
-        int npad;      // ... padded to what its variant of the pass takes per register pass
-    };
     std::vector<SegHost> segs;
     std::vector<ReqDev> rd(n);
-    const int sub = 32;                        // paths per staged sub-chunk
     for (int r = 0; r < n; ++r) {
         const qts_request& R = reqs[r];
         qts_ensemble* e = R.ens;
@@ -518,85 +557,12 @@ static qts_status build_plan(int n, const qts_request* reqs, int n_quad, BatchPl
         char* wbase = (char*)e->d_work;
         rd[r] = {(const float*)(wbase + bw.xt_off), grad ? (const float*)(wbase + bw.gt_off) : nullptr, R.phi,
                  R.M, bw.Mpad, R.F, 0, (const int*)(wbase + bw.flag_off), e->d_status};
-        if (R.M <= 0) continue;
-        double* g_val = grad ? (double*)e->d_work + 4 : nullptr;
-        double* g_slot = grad ? g_val + 2 * e->bprep.n_paths : nullptr;
-        for (const Bucket& b : e->bprep.buckets) {
-            if (ov && ov->only_width > 0 && b.D != ov->only_width) continue;
-            const int cls = batch_class(b.D);
-            if (ov && ov->only_class > 0 && cls != ov->only_class) continue;
-            const Tune& tn = e->tune[b.D];
-            int mode = R.F + 1 <= kPrivRows ? 1 : 0;
-            if (grad && pair_width(b.D) &&
-                batch_smem_bytes(tile_floats_for(2, R.F), sub, cls) <= class_smem_budget(cls)) {
-                const int want = ov && ov->mode[b.D] ? ov->mode[b.D] : tn.bt_mode;
-                mode = want == 3 ? 3 : 2;
-            }
-            const int per_item = item_samples(mode);
-            const int n_tiles = (int)((R.M + per_item - 1) / per_item);
-            SegHost s;
-            s.d.rec = (const Rec32*)e->bdev.rec + b.rec_off;
-            s.d.g_val = grad ? g_val + 2 * b.path_base : nullptr;
-            s.d.g_slot = grad ? g_slot + b.slot_base : nullptr;
-            s.d.n_paths = b.n_paths;
-            s.d.D = b.D;
-            s.d.paths = ov && ov->paths[b.D] ? ov->paths[b.D]
-                        : tn.bt_paths ? tn.bt_paths : (e->tuned ? tn.bpaths : item_paths(b.D, grad));
-            s.d.n_tiles = n_tiles;
-            s.d.req = r;
-            s.d.priv = mode;
-            s.d.pad = 0;
-            s.occ = ov && ov->occ[b.D] ? ov->occ[b.D] : tn.bt_occ;
-            s.nq = nodes_for(n_quad, b.D, 1);
-            // the packed fused pass takes one node at a time, the others node pairs
-            const int pad = (grad && mode >= 2) ? 1 : 2;
-            s.npad = (s.nq + pad - 1) / pad * pad;
-            s.cost = (double)s.d.paths * b.D * (grad ? 12 : 4) * s.npad;
-            s.cls = cls;
-            // a launch sizes its shared memory for its widest tile, and whatever
-            // shared memory a block does not take stays L1 (which serves the x and
-            // grad_phi loads): requests of one class are launched by tile size
-            s.tile = tile_floats_for(mode, R.F);
-            const int64_t tb = s.tile * 4;
-            s.bin = tb <= 48 * 1024 ? 0 : tb <= 80 * 1024 ? 1 : 2;
-            segs.push_back(s);
-        }
+        if (R.M > 0) request_segments(R, r, n_quad, ov, &segs);
     }
-    // one launch per (kernel class, tile bin, quadrature rule), heaviest items
-    // first within it
-    std::stable_sort(segs.begin(), segs.end(), [](const SegHost& a, const SegHost& b) {
-        if (a.cls != b.cls) return a.cls < b.cls;
-        if (a.bin != b.bin) return a.bin < b.bin;
-        if (a.npad != b.npad) return a.npad > b.npad;
-        if (a.nq != b.nq) return a.nq > b.nq;
-        return a.cost > b.cost;
-    });
-    std::vector<int> cls_list, cls_nq, cls_npad, cls_occ;
-    std::vector<int64_t> cls_items, cls_first_seg, cls_tile;
-    int64_t item = 0;
-    for (size_t i = 0; i < segs.size(); ++i) {
-        if (cls_list.empty() || cls_list.back() != segs[i].cls || segs[i - 1].bin != segs[i].bin ||
-            segs[i - 1].nq != segs[i].nq || segs[i - 1].npad != segs[i].npad) {
-            cls_list.push_back(segs[i].cls);
-            cls_nq.push_back(segs[i].nq);
-            cls_npad.push_back(segs[i].npad);
-            cls_occ.push_back(0);
-            cls_first_seg.push_back((int64_t)i);
-            cls_items.push_back(0);
-            cls_tile.push_back(0);
-            item = 0;
-        }
-        cls_tile.back() = std::max(cls_tile.back(), segs[i].tile);
-        // a launch takes the smallest cap of its widths
-        if (segs[i].occ > 0 && (cls_occ.back() == 0 || segs[i].occ < cls_occ.back())) cls_occ.back() = segs[i].occ;
-        segs[i].d.item_begin = item;
-        const int64_t chunks = (segs[i].d.n_paths + segs[i].d.paths - 1) / segs[i].d.paths;
-        item += chunks * segs[i].d.n_tiles;
-        cls_items.back() = item;
-    }
+    const std::vector<LaunchHost> launches = order_segments(segs, (size_t)1 << 30);
     const size_t seg_bytes = (sizeof(SegDev) * std::max<size_t>(segs.size(), 1) + 255) / 256 * 256;
     const size_t req_bytes = (sizeof(ReqDev) * std::max(n, 1) + 255) / 256 * 256;
-    const size_t cnt_bytes = 256;
+    const size_t cnt_bytes = (sizeof(unsigned long long) * std::max<size_t>(launches.size(), 1) + 255) / 256 * 256;
     cudaError_t ce = cudaMalloc(&plan->dev, seg_bytes + req_bytes + cnt_bytes);
     if (ce != cudaSuccess) return cuda_fail(ce, "batch plan allocation");
     SegDev* d_segs = (SegDev*)plan->dev;
@@ -622,14 +588,14 @@ static qts_status build_plan(int n, const qts_request* reqs, int n_quad, BatchPl
         const BatchWork bw = batch_work(R.ens, R.M, R.F, grad);
         char* wbase = (char*)R.ens->d_work;
         if (R.phi && R.M > 0) {
-            err = launch_phi_init(R.phi, R.M, R.F, R.ens->bprep.bias, cap);
+            err = launch_phi_init(R.phi, R.M, R.F, R.ens->prep.bias, cap);
             ++kernels;
         }
         if (grad && err == cudaSuccess) err = cudaMemsetAsync(wbase, 0, bw.grad_bytes, cap);
         // the NaN flag starts set for ensembles with categorical elements, so
         // their items take the NaN-aware (categorical-aware) variant
         if (err == cudaSuccess)
-            err = cudaMemsetAsync(wbase + bw.flag_off, R.ens->bprep.has_cat ? 1 : 0, 256, cap);
+            err = cudaMemsetAsync(wbase + bw.flag_off, R.ens->prep.has_cat ? 1 : 0, 256, cap);
         if (R.M > 0 && err == cudaSuccess) {
             err = launch_transpose(R.X, R.M, R.F, R.F, (float*)(wbase + bw.xt_off), R.F + 1, bw.Mpad,
                                    (int*)(wbase + bw.flag_off), cap);
@@ -643,43 +609,21 @@ static qts_status build_plan(int n, const qts_request* reqs, int n_quad, BatchPl
     }
     if (err == cudaSuccess) err = cudaMemsetAsync(d_cnt, 0, cnt_bytes, cap);
     if (err == cudaSuccess) err = cudaEventRecordWithFlags(plan->ev0, cap, cudaEventRecordExternal);
-    for (size_t c = 0; c < cls_list.size() && err == cudaSuccess; ++c) {
-        const int cls = cls_list[c];
+    for (size_t c = 0; c < launches.size() && err == cudaSuccess; ++c) {
         BatchArgs a;
-        a.segs = d_segs + cls_first_seg[c];
-        a.n_segs = (int)((c + 1 < cls_list.size() ? cls_first_seg[c + 1] : (int64_t)segs.size()) - cls_first_seg[c]);
+        a.segs = d_segs + launches[c].first;
         a.reqs = d_reqs;
-        a.n_items = cls_items[c];
-        a.counter = d_cnt + c;
-        a.tile_floats = std::max<int64_t>(cls_tile[c], kTileLd);
-        a.sub = sub;
-        if (!make_quad(cls_nq[c], &a.q, nullptr, cls_npad[c] == cls_nq[c] ? 1 : 2) || a.q.n_pad != cls_npad[c]) {
-            err = cudaErrorInvalidValue;
-            break;
-        }
-        const size_t smem = batch_smem_bytes(a.tile_floats, sub, cls);
-        int blocks = 0;
-        if (cls == 8) err = launch_batch_class<8>(a, smem, cap, &blocks, cls_occ[c]);
-        else if (cls == 12) err = launch_batch_class<12>(a, smem, cap, &blocks, cls_occ[c]);
-        else if (cls == 16) err = launch_batch_class<16>(a, smem, cap, &blocks, cls_occ[c]);
-        else if (cls == 32) err = launch_batch_class<32>(a, smem, cap, &blocks, cls_occ[c]);
-        else if (cls == 40) err = launch_batch_class<40>(a, smem, cap, &blocks, cls_occ[c]);
-        else if (cls == 48) err = launch_batch_class<48>(a, smem, cap, &blocks, cls_occ[c]);
-        else if (cls == 56) err = launch_batch_class<56>(a, smem, cap, &blocks, cls_occ[c]);
-        else err = launch_batch_class<64>(a, smem, cap, &blocks, cls_occ[c]);
+        err = launch_ordered(launches[c], a, d_cnt + c, cap);
         ++kernels;
     }
     if (err == cudaSuccess) err = cudaEventRecordWithFlags(plan->ev1, cap, cudaEventRecordExternal);
     for (int r = 0; r < n && err == cudaSuccess; ++r) {
         const qts_request& R = reqs[r];
         if (!R.grad_phi) continue;
-        double* gb = (double*)R.ens->d_work;
-        double* g_val = gb + 4;
-        double* g_slot = g_val + 2 * R.ens->bprep.n_paths;
         if (R.M > 0) {
-            err = launch_bwd_epilogue_pairs(R.ens, R.grad_phi, R.M, R.F, g_val, g_slot, R.d_leaf, R.d_z, gb, cap);
-            kernels += 1 + (R.ens->bprep.n_paths + (int64_t)R.ens->bprep.empty_leaf.size() > 0) +
-                       (R.ens->bprep.n_slots > 0);
+            double* gb = (double*)R.ens->d_work;
+            err = launch_bwd_epilogue_blocks(R.ens, R.grad_phi, R.M, R.F, gb + kGradHead, R.d_leaf, R.d_z, gb, cap);
+            kernels += 2 + (R.ens->blkdev.n_ent > 0);
         } else {
             err = cudaMemsetAsync(R.d_leaf, 0, sizeof(double) * R.ens->n_nodes, cap);
             if (err == cudaSuccess) err = cudaMemsetAsync(R.d_z, 0, sizeof(double) * R.ens->n_nodes, cap);
@@ -726,7 +670,7 @@ static qts_status check_batch(int32_t n, const qts_request* reqs, int32_t n_quad
     }
     for (int r = 0; r < n; ++r) {
         const qts_request& R = reqs[r];
-        qts_status st = ensure_batch_tables(R.ens);
+        qts_status st = ensure_blocks(R.ens, R.grad_phi != nullptr);
         if (st != QTS_OK) return st;
         st = ensure_workspace(R.ens, batch_work(R.ens, R.M, R.F, R.grad_phi != nullptr).total);
         if (st != QTS_OK) return st;
@@ -749,7 +693,7 @@ extern "C" qts_status qts_batched_fwd_bwd(int32_t n, const qts_request* reqs, in
         for (uint64_t v : {(uint64_t)(uintptr_t)R.ens, (uint64_t)(uintptr_t)R.X, (uint64_t)R.M, (uint64_t)R.F,
                            (uint64_t)(uintptr_t)R.grad_phi, (uint64_t)(uintptr_t)R.phi,
                            (uint64_t)(uintptr_t)R.d_leaf, (uint64_t)(uintptr_t)R.d_z,
-                           (uint64_t)(uintptr_t)R.ens->d_work, (uint64_t)(uintptr_t)R.ens->bdev.rec,
+                           (uint64_t)(uintptr_t)R.ens->d_work, (uint64_t)(uintptr_t)R.ens->blkdev.rec,
                            (uint64_t)R.ens->tune_gen})
             key.push_back(v);
     }
@@ -825,18 +769,15 @@ extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, i
     std::vector<qts_request> sub(reqs, reqs + n);
     if (max_samples > 0)
         for (auto& R : sub) R.M = std::min<int64_t>(R.M, max_samples);
-    // work (element-samples) per bucket width of the reduced batch, and whether
-    // the width runs the packed fused pass for some request
+    // work per bucket width of the reduced batch, and whether the width runs the
+    // pass of two samples per lane for some request
     std::vector<double> work(kMaxD + 1, 0.0);
     std::vector<char> packed(kMaxD + 1, 0);
-    std::vector<char> fused(kMaxD + 1, 0);
     for (const auto& R : sub) {
         if (R.M <= 0) continue;
-        for (const Bucket& b : R.ens->bprep.buckets) {
-            if (b.n_paths == 0) continue;
-            work[b.D] += (double)R.M * (double)b.n_paths * b.D;
-            if (R.grad_phi) fused[b.D] = 1;
-            if (R.grad_phi && pair_width(b.D)) packed[b.D] = 1;
+        for (const BlockBucket& b : R.ens->blk) {
+            work[b.D] += (double)R.M * (double)b.n * blk_cost(b.D, b.h);
+            if (R.grad_phi && b.D <= 16) packed[b.D] = 1;
         }
     }
     double total = 0.0;
@@ -853,12 +794,10 @@ extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, i
         BatchOverride ov;
         std::memset(&ov, 0, sizeof(ov));
         ov.only_width = D;
-        const int base = item_paths(D, fused[D] != 0);
         float best = 1e30f;
         for (int mode : {2, 3}) {
             if (mode == 3 && !packed[D]) continue;
-            for (int mult : {1, 2, 4, 8}) {  // base, twice, four and eight times
-                const int paths = std::max(32, std::min(4096, base * mult / 32 * 32));
+            for (int paths : {64, 256, 1024, 2048}) {
                 ov.paths[D] = paths;
                 ov.mode[D] = packed[D] ? mode : 0;
                 float ms = 0.f;
@@ -875,36 +814,6 @@ extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, i
             }
         }
     }
-    // blocks per SM of the two register classes that fit three or more: all
-    // that fit, or one fewer, which leaves the SM's shared memory more L1 for
-    // the x and grad_phi reads; timed over the class's widths with the choices
-    // above
-    std::vector<int> best_occ(kMaxD + 1, 0);
-    for (int cls : {8, 12}) {
-        bool any = false;
-        for (int D : widths) any = any || batch_class(D) == cls;
-        if (!any) continue;
-        const int full = cls == 8 ? 4 : 3;
-        BatchOverride ov;
-        std::memset(&ov, 0, sizeof(ov));
-        ov.only_class = cls;
-        for (int D = 1; D <= kMaxD; ++D) {
-            ov.paths[D] = best_paths[D];
-            ov.mode[D] = best_mode[D];
-        }
-        float t[2] = {0.f, 0.f};
-        for (int k = 0; k < 2; ++k) {
-            for (int D = 1; D <= kMaxD; ++D) ov.occ[D] = (k == 1 && batch_class(D) == cls) ? full - 1 : 0;
-            st = time_plan(n, sub.data(), n_quad, ov, cap, (cudaStream_t)stream, &t[k]);
-            if (st != QTS_OK) {
-                cudaStreamDestroy(cap);
-                return st;
-            }
-        }
-        if (t[1] < t[0])
-            for (int D = 1; D <= kMaxD; ++D)
-                if (batch_class(D) == cls) best_occ[D] = full - 1;
-    }
     cudaStreamDestroy(cap);
     for (int r = 0; r < n; ++r) {
         qts_ensemble* e = reqs[r].ens;
@@ -912,7 +821,6 @@ extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, i
             e->tune[D].bt_paths = best_paths[D];
             e->tune[D].bt_mode = best_mode[D];
         }
-        for (int D = 1; D <= kMaxD; ++D) e->tune[D].bt_occ = best_occ[D];
         ++e->tune_gen;
         batch_forget(e);
     }
@@ -920,7 +828,7 @@ extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, i
         for (int D = 0; D <= kMaxD; ++D) {
             chosen[3 * D] = best_paths[D];
             chosen[3 * D + 1] = best_mode[D];
-            chosen[3 * D + 2] = best_occ[D];
+            chosen[3 * D + 2] = 0;
         }
     return QTS_OK;
 }
@@ -943,6 +851,49 @@ extern "C" qts_status qts_get_batch_info(qts_ensemble* e, int64_t* n_paths, int6
     }
     return QTS_OK;
 }
+
+// Adjoint of one request by the batched kernels, without a graph (qts_shap_backward).
+namespace qts {
+
+size_t adjoint_work_bytes(const qts_ensemble* e, int64_t M, int F) { return batch_work(e, M, F, true).total; }
+
+cudaError_t launch_adjoint_blocks(qts_ensemble* e, const float* X, const float* grad, int64_t M, int F, int n_quad,
+                                  double* d_leaf, double* d_z, cudaStream_t st) {
+    const BatchWork bw = batch_work(e, M, F, true);
+    char* w = (char*)e->d_work;
+    qts_request R;
+    std::memset(&R, 0, sizeof(R));
+    R.ens = e;
+    R.X = X;
+    R.M = M;
+    R.F = F;
+    R.grad_phi = grad;
+    cudaError_t err = cudaMemsetAsync(w, 0, bw.grad_bytes, st);
+    if (err == cudaSuccess) err = cudaMemsetAsync(w + bw.flag_off, e->prep.has_cat ? 1 : 0, 256, st);
+    if (err == cudaSuccess)
+        err = launch_transpose(X, M, F, F, (float*)(w + bw.xt_off), F + 1, bw.Mpad, (int*)(w + bw.flag_off), st);
+    if (err == cudaSuccess)
+        err = launch_transpose(grad, M, F + 1, F + 1, (float*)(w + bw.gt_off), F + 1, bw.Mpad, nullptr, st);
+    std::vector<SegHost> segs;
+    request_segments(R, 0, n_quad, nullptr, &segs);
+    const std::vector<LaunchHost> launches = order_segments(segs, kInlineSegs);
+    if (launches.size() > kGradHead - 1) return cudaErrorInvalidConfiguration;
+    unsigned long long* counter = (unsigned long long*)w + 1;  // cleared with the sums
+    for (size_t c = 0; c < launches.size() && err == cudaSuccess; ++c) {
+        BatchArgs a;
+        a.segs = nullptr;
+        a.reqs = nullptr;
+        for (size_t i = 0; i < launches[c].count; ++i) a.seg[i] = segs[launches[c].first + i].d;
+        a.req = {(const float*)(w + bw.xt_off), (const float*)(w + bw.gt_off), nullptr, M, bw.Mpad, F, 0,
+                 (const int*)(w + bw.flag_off), e->d_status};
+        err = launch_ordered(launches[c], a, counter + c, st);
+    }
+    double* gb = (double*)w;
+    if (err == cudaSuccess) err = launch_bwd_epilogue_blocks(e, grad, M, F, gb + kGradHead, d_leaf, d_z, gb, st);
+    return err;
+}
+
+}  // namespace qts
 
 extern "C" int32_t qts_batched_kernel_count(void) { return g_last_batch_kernels; }
 

@@ -75,4 +75,6 @@ QTS_HD constexpr int blk_slots(int h) { return h == 0 ? 1 : 2 * blk_inner(h) + 3
 // (36 per shared element, 65 per inner and 36 per pair node, 25 for the rest).
 inline double blk_cost(int D, int h) { return 25.0 + 36.0 * D + 65.0 * blk_inner(h) + 36.0 * blk_pairs(h); }
 
+constexpr double kBlkUnit = 300.0;
+
 }  // namespace qts

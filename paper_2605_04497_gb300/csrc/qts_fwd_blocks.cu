@@ -284,7 +284,8 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
             };
             // work per thread block: about eight rounds of the whole chip, at
             // most what keeps the tile set-up and flush small beside it
-            const double share = std::min(400e3, std::max(4e3, total / (8.0 * num_sms() * 4)));
+            const double share = e->tune[0].bpaths > 0 ? kBlkUnit * e->tune[0].bpaths
+                                                       : std::min(400e3, std::max(4e3, total / (8.0 * num_sms() * 4)));
             for (const BlockBucket* b : pick) {
                 if (a.n_seg == kFbSegs) {
                     const cudaError_t r = flush();

@@ -167,7 +167,8 @@ struct Tune {
     int paths = 128;      // paths per block (chunk)
     int sub = 32;         // paths per staged sub-chunk
     int np = 8;           // nodes per register pass (8, 4 or 2)
-    int bpaths = 128;     // paths per work item of the fused forward + adjoint pass
+    int bpaths = 0;       // block-table forward: work per thread block in units of an
+                          // average block (kBlkUnit); 0: chosen from the call's work
     int priv = 1;         // forward: 1 each warp owns a sample tile (when it fits), 2 the
                           // warps share one and split the paths with a phi tile each,
                           // 0 they share one phi tile (shared-memory atomics)
@@ -299,16 +300,11 @@ cudaError_t launch_int_bucket(const qts_ensemble* e, const Bucket& b, bool pairs
                               cudaStream_t st);
 cudaError_t launch_int_finalize(const double* acc_pair, const double* acc_phi, int64_t M, int F,
                                 double bias, float* out, cudaStream_t st);
-cudaError_t launch_bwd_bucket(const qts_ensemble* e, const Bucket& b, const float* X,
-                              const float* grad, int64_t M, int F, const QuadF& q,
-                              double* g_val, double* g_slot, double* phi, const Tune& tn,
-                              cudaStream_t st);
-cudaError_t launch_bwd_epilogue(const qts_ensemble* e, const float* grad, int64_t M, int F,
-                                const double* g_val, const double* g_slot, double* d_leaf,
-                                double* d_z, double* g_bias_scratch, cudaStream_t st);
-// the same for the pair tables of the batched pass (two g_val sums per path)
-cudaError_t launch_bwd_epilogue_pairs(const qts_ensemble* e, const float* grad, int64_t M, int F,
-                                      const double* g_val, const double* g_slot, double* d_leaf,
-                                      double* d_z, double* g_bias_scratch, cudaStream_t st);
+cudaError_t launch_bwd_epilogue_blocks(const qts_ensemble* e, const float* grad, int64_t M, int F, const double* g,
+                                       double* d_leaf, double* d_z, double* g_bias_scratch, cudaStream_t st);
+// FP32 adjoint of one request (workspace: adjoint_work_bytes, block tables with grad)
+size_t adjoint_work_bytes(const qts_ensemble* e, int64_t M, int F);
+cudaError_t launch_adjoint_blocks(qts_ensemble* e, const float* X, const float* grad, int64_t M, int F, int n_quad,
+                                  double* d_leaf, double* d_z, cudaStream_t st);
 
 }  // namespace qts

@@ -1,9 +1,6 @@
-// Launch-shape autotuner: for each bucket width of an ensemble, time candidate
-// (warps per block, paths per block, staged sub-chunk, node-group width, private
-// per-warp tiles or not) of the
-// forward kernel and candidate work-item sizes of the fused forward+adjoint
-// kernel on the caller's data, keep the fastest, and optionally merge them into
-// a JSON cache keyed by (width, log2 F, log2 M).
+// Launch-shape autotuner of the forward: times the work per thread block of the
+// block-table kernels on the caller's data, keeps the fastest, and optionally
+// merges it into a JSON cache keyed by (width, log2 F, log2 M).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -15,9 +12,6 @@
 
 namespace qts {
 
-cudaError_t launch_bwd_bucket(const qts_ensemble* e, const Bucket& b, const float* X,
-                              const float* grad, int64_t M, int F, const QuadF& q, double* g_val,
-                              double* g_slot, double* phi, const Tune& tn, cudaStream_t st);
 void batch_forget(const qts_ensemble* e);
 
 static int ilog2(int64_t v) {
@@ -107,101 +101,36 @@ extern "C" qts_status qts_autotune(qts_ensemble* e, const float* X, int64_t M, i
     std::map<std::string, Tune> cache;
     if (cache_path) cache = read_cache(cache_path);
     const int64_t Mt = std::min<int64_t>(M, 4096);  // tune on a leading slice of the samples
-    QuadF qf;
-    QuadD qd;
-    make_quad(8, &qf, &qd);
     double* phi = nullptr;
-    float* grad = nullptr;
-    // the FP32 forward and adjoint run on the pair tables
-    st = ensure_batch_tables(e);
+    // the FP32 forward runs on the block tables
+    st = ensure_blocks(e, false);
     if (st != QTS_OK) return st;
-    const Prepared& P = e->bprep;
     cudaError_t ce = cudaMalloc(&phi, sizeof(double) * Mt * (F + 1));
-    if (ce == cudaSuccess) ce = cudaMalloc(&grad, sizeof(float) * Mt * (F + 1));
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(grad, 0, sizeof(float) * Mt * (F + 1), s);
-    if (ce != cudaSuccess) {
-        cudaFree(phi);
-        cudaFree(grad);
-        return cuda_fail(ce, "autotune scratch");
-    }
-    st = ensure_workspace(e, sizeof(double) * (size_t)(4 + 2 * P.n_paths + P.n_slots));
-    if (st != QTS_OK) {
-        cudaFree(phi);
-        cudaFree(grad);
-        return st;
-    }
-    double* g_val = (double*)e->d_work + 4;
-    double* g_slot = g_val + 2 * P.n_paths;
-    for (int D = 1; D <= kMaxD; ++D) {
-        const Bucket* bf = nullptr;
-        for (const Bucket& b : P.buckets)
-            if (b.D == D) bf = &b;
-        const Bucket* bb = bf;
-        if (!bf) continue;
-        const std::string key = cache_key(D, F, M);
-        auto it = cache.find(key);
-        if (it != cache.end()) {
-            const Tune keep = e->tune[D];  // the batched-launch tuner's choices stay
-            e->tune[D] = it->second;
-            e->tune[D].bt_paths = keep.bt_paths;
-            e->tune[D].bt_mode = keep.bt_mode;
-            e->tune[D].bt_occ = keep.bt_occ;
-            continue;
-        }
-        Tune best = e->tune[D];
+    if (ce != cudaSuccess) return cuda_fail(ce, "autotune scratch");
+    // one choice for the ensemble (its buckets share launches), kept under the
+    // width of every path bucket: Tune::bpaths
+    bool cached = !e->prep.buckets.empty();
+    for (const Bucket& b : e->prep.buckets) cached = cached && cache.count(cache_key(b.D, F, M)) != 0;
+    Tune best = e->tune[0];
+    if (cached) {
+        best = cache[cache_key(e->prep.buckets.front().D, F, M)];
+    } else {
         float best_ms = 1e30f;
-        const int nps[3] = {8, 4, 2};
-        for (int np : nps) {
-            if (!bf) break;
-            if ((np == 8 && D > 8) || (np == 4 && D > 24)) continue;
-            for (int warps : {2, 4, 8}) {
-                for (int paths : {128, 512, 2048}) {
-                    for (int sub : {16, 32}) {
-                      for (int priv : {1, 2, 0}) {
-                        Tune t = best;
-                        t.np = np;
-                        t.warps = warps;
-                        t.paths = paths;
-                        t.sub = sub;
-                        t.priv = priv;
-                        cudaError_t le = cudaSuccess;
-                        const float ms = time_ms([&] {
-                            le = launch_fwd_bucket(e, *bf, X, Mt, F, qf, qd, phi, t, s);
-                        }, s, 3);
-                        if (le == cudaSuccess && ms < best_ms) {
-                            best_ms = ms;
-                            best = t;
-                        }
-                        cudaGetLastError();
-                      }
-                    }
-                }
-            }
-        }
-        // work-item size of the fused forward + adjoint pass (batched launches)
-        float best_b = 1e30f;
-        for (int paths : {32, 64, 128, 256, 512}) {
-            if (!bb) break;
-            Tune t = best;
-            t.paths = paths;
-            t.sub = 16;
-            t.warps = 4;
+        for (int paths : {128, 256, 512, 1024, 2048}) {
+            for (Tune& t : e->tune) t.bpaths = paths;
             cudaError_t le = cudaSuccess;
-            const float ms = time_ms([&] {
-                le = launch_bwd_bucket(e, *bb, X, grad, Mt, F, qf, g_val, g_slot, phi, t, s);
-            }, s, 3);
-            if (le == cudaSuccess && ms < best_b) {
-                best_b = ms;
+            const float ms = time_ms([&] { le = launch_fwd_blocks(e, X, Mt, F, 8, phi, s); }, s, 3);
+            if (le == cudaSuccess && ms < best_ms) {
+                best_ms = ms;
                 best.bpaths = paths;
             }
             cudaGetLastError();
         }
-        e->tune[D] = best;
-        cache[key] = best;
+        for (const Bucket& b : e->prep.buckets) cache[cache_key(b.D, F, M)] = best;
     }
+    for (Tune& t : e->tune) t.bpaths = best.bpaths;
     ce = cudaStreamSynchronize(s);
     cudaFree(phi);
-    cudaFree(grad);
     if (ce != cudaSuccess) return cuda_fail(ce, "autotune");
     e->tuned = true;
     ++e->tune_gen;
