@@ -185,7 +185,10 @@ qts_status ensure_blocks(qts_ensemble* e, bool grad) {
     if (grad && H.n_slots >= ((int64_t)1 << 32)) return fail(QTS_ERR_UNSUPPORTED, "too many adjoint sums");
     int64_t tot = 0;
     qts_status st = QTS_OK;
-    if (!e->blk_ready) st = up(&e->blkdev.rec, H.rec, &tot, "upload block tables");
+    if (!e->blk_ready) {
+        st = up(&e->blkdev.rec, H.rec, &tot, "upload block tables");
+        if (st == QTS_OK && !H.dbl.empty()) st = up(&e->blkdev.dbl, H.dbl, &tot, "upload block tables");
+    }
     if (grad) {
         if (st == QTS_OK) st = up(&e->blkdev.ent, H.ent, &tot, "upload block tables");
         e->blkdev.n_ent = (int64_t)H.ent.size();
@@ -206,7 +209,7 @@ qts_status ensure_blocks(qts_ensemble* e, bool grad) {
 
 void release_blocks(qts_ensemble* e) {
     BlockDev& T = e->blkdev;
-    for (void* p : {(void*)T.rec, (void*)T.ent, (void*)T.bias_leaf, (void*)T.bias_z}) cudaFree(p);
+    for (void* p : {(void*)T.rec, (void*)T.dbl, (void*)T.ent, (void*)T.bias_leaf, (void*)T.bias_z}) cudaFree(p);
     T = BlockDev();
     e->blk.clear();
     e->n_blocks = e->n_blk_slots = 0;
@@ -393,32 +396,15 @@ qts_status qts_shap_values(qts_ensemble* e, const float* X, int64_t M, int32_t F
     if (M == 0) return QTS_OK;
     if (!phi) return fail(QTS_ERR_ARG, "phi is NULL");
     cudaStream_t s = (cudaStream_t)stream;
-    // FP32 runs on the block tables, or for a few samples on the pair tables
-    // (either built on the first call that needs them)
-    const bool fp64 = (e->flags & QTS_FLAG_FP64) != 0;
-    if (!fp64 && M > kFewRows) {
-        st = ensure_blocks(e, false);
-        if (st != QTS_OK) return st;
-        cudaError_t ce = launch_phi_init(phi, M, F, e->prep.bias, s);
-        if (ce == cudaSuccess) ce = launch_fwd_blocks(e, X, M, F, n_quad, phi, s);
-        return ce == cudaSuccess ? QTS_OK : cuda_fail(ce, "forward kernel launch");
-    }
-    if (!fp64) {
-        st = ensure_batch_tables(e);
-        if (st != QTS_OK) return st;
-    }
-    const Prepared& P = fp64 ? e->prep : e->bprep;
-    cudaError_t ce = launch_phi_init(phi, M, F, P.bias, s);
+    // the block tables (built on the first call that needs them)
+    st = ensure_blocks(e, false);
+    if (st != QTS_OK) return st;
+    cudaError_t ce = launch_phi_init(phi, M, F, e->prep.bias, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "phi init launch");
-    for (const Bucket& b : P.buckets) {
-        // the bucket's rule, padded to whole node pairs (QTS_NQ_EXACT: ceil(D/2) points)
-        QuadF qf;
-        QuadD qd;
-        if (!make_quad(nodes_for(n_quad, b.D, 1), &qf, &qd, 2)) return fail(QTS_ERR_ARG, "quadrature rule");
-        ce = launch_fwd_bucket(e, b, X, M, F, qf, qd, phi, e->tune[b.D], s);
-        if (ce != cudaSuccess) return cuda_fail(ce, "forward kernel launch");
-    }
-    return QTS_OK;
+    if (e->flags & QTS_FLAG_FP64) ce = launch_fwd64(e, X, M, F, n_quad, phi, s);
+    else if (M <= kFewRows) ce = launch_fwd_few(e, X, M, F, n_quad, phi, s);
+    else ce = launch_fwd_blocks(e, X, M, F, n_quad, phi, s);
+    return ce == cudaSuccess ? QTS_OK : cuda_fail(ce, "forward kernel launch");
 }
 
 qts_status qts_selftest_wait_timeout(qts_ensemble* e, qts_stream_t stream) {

@@ -39,6 +39,7 @@ constexpr int kKeys = (kMaxD + 1) * (kBlkMaxH + 1);
 
 struct Part {  // one thread's share of one bucket
     std::vector<Rec32> rec;
+    std::vector<double> dbl;
     std::vector<BlockEntry> ent;
     std::vector<uint32_t> ent_count;  // per block
     int64_t n = 0;
@@ -62,8 +63,10 @@ struct Walker {
 
     // scratch of the block under construction
     std::vector<Rec32> rec;
+    std::vector<double> dbl;
     std::vector<BlockEntry> ent;
-    int H = 0, slot0 = 0, dmax = 0;
+    int H = 0, slot0 = 0, dmax = 0;  // slot0: the block's width
+    bool fp64 = false;
 
     Edge edge(int64_t g, int side) const {
         const int32_t c = side == 0 ? e->left[g] : e->right[g];
@@ -153,14 +156,20 @@ struct Walker {
             // neutral; a leaf goes down the left edges to a pair's left leaf
             const bool leaf = v >= 0 && is_leaf(v);
             const float val = leaf ? e->leaf[base + v] : 0.f;
+            double* q = &dbl[blk_dbl(slot0, H, n)];
             r[1] = word_rec(e->n_features, INFINITY, -INFINITY, INFINITY, true, true);
             if (levels > 1) {
                 r[0] = four(1.f, 1.f, 0.f, 0.f);
+                q[0] = 1.0;
+                q[1] = 0.0;
                 place(leaf ? v : -1, 2 * n, levels - 1);
                 place(-1, 2 * n + 1, levels - 1);
             } else {
                 r[0] = four(val, 0.f, 1.f, 0.f);
                 r[2] = four(val, val, 0.f, 0.f);
+                q[0] = q[4] = val;
+                q[1] = q[3] = 0.0;
+                q[2] = 1.0;
                 if (leaf) {
                     dmax = std::max(dmax, (int)uniq[v]);
                     if (grad) {
@@ -176,12 +185,13 @@ struct Walker {
         const Elem prev = merged(f);
         r[1] = word_rec(f, e->thr[g], prev.lo, prev.hi, prev.nan_ok != 0, e->defl[g] != 0);
         float z[2], val[2] = {0.f, 0.f};
-        double vz = 0.0;
+        double zd[2], vz = 0.0;
         for (int side = 0; side < 2; ++side) {
             const Edge x = edge(g, side);
             const int32_t c = (int32_t)(x.child - base);
             const double ze = prev.z * x.w;
             z[side] = (float)ze;
+            zd[side] = ze;
             path.push_back(x);
             if (levels > 1) {
                 if (grad) chain(f, slot + side, 1.0);
@@ -198,11 +208,19 @@ struct Walker {
             }
             path.pop_back();
         }
+        double* q = &dbl[blk_dbl(slot0, H, n)];
         if (levels > 1) {
             r[0] = four(z[0], z[0], z[1], z[1]);
+            q[0] = zd[0];
+            q[1] = zd[1];
         } else {
             r[0] = four(val[0], val[1], z[0], z[1]);
             r[2] = four((float)vz, (float)vz, 0.f, 0.f);
+            q[0] = val[0];
+            q[1] = val[1];
+            q[2] = zd[0];
+            q[3] = zd[1];
+            q[4] = vz;
         }
     }
 
@@ -218,6 +236,9 @@ struct Walker {
         dmax = h == 0 ? uniq[v] : 0;
         ent.clear();
         rec.resize((size_t)(blk_stride(0, h) - blk_head(0)));
+        dbl.assign((size_t)blk_doubles(width, h), 1.0);
+        dbl[0] = h == 0 ? (double)e->leaf[g] : 1.0;
+        for (int j = 0; j < D; ++j) dbl[1 + j] = merged(pre[j]).z;
         if (h > 0) place(v, 1, h);
         Part& P = part[width * (kBlkMaxH + 1) + h];
         P.rec.push_back(four(h == 0 ? e->leaf[g] : 1.f, 0.f, 0.f, 0.f));
@@ -235,6 +256,7 @@ struct Walker {
             P.rec.push_back(r);
         }
         P.rec.insert(P.rec.end(), rec.begin(), rec.end());
+        if (fp64) P.dbl.insert(P.dbl.end(), dbl.begin(), dbl.end());
         if (grad) {
             for (int j = 0; j < D; ++j) chain(pre[j], j, 1.0);
             if (h == 0) add(g, true, slot0, 1.0);
@@ -367,23 +389,26 @@ void build_blocks(const qts_ensemble* e, bool grad, BlockHost* out) {
     run(nth, [&](int k) {
         w[k].e = e;
         w[k].grad = grad;
+        w[k].fp64 = (e->flags & QTS_FLAG_FP64) != 0;
         for (int t = cut[k]; t < cut[k + 1]; ++t) w[k].tree(t);
     });
     // bucket sizes and each thread's place in them
     *out = BlockHost();
-    int64_t n_rec = 0, n_ent = 0, n_slot = 0, n_blk = 0;
-    struct Place { int64_t rec, ent, slot; };
+    int64_t n_rec = 0, n_dbl = 0, n_ent = 0, n_slot = 0, n_blk = 0;
+    struct Place { int64_t rec, dbl, ent, slot; };
     std::vector<Place> at((size_t)nth * kKeys);
     for (int key = 0; key < kKeys; ++key) {
         BlockBucket b;
         b.D = key / (kBlkMaxH + 1);
         b.h = key % (kBlkMaxH + 1);
         b.rec_off = n_rec;
+        b.dbl_off = n_dbl;
         b.slot_off = n_slot;
         for (int k = 0; k < nth; ++k) {
             const Part& p = w[k].part[key];
-            at[(size_t)k * kKeys + key] = {n_rec, n_ent, n_slot + b.n * (b.D + blk_slots(b.h))};
+            at[(size_t)k * kKeys + key] = {n_rec, n_dbl, n_ent, n_slot + b.n * (b.D + blk_slots(b.h))};
             n_rec += (int64_t)p.rec.size();
+            n_dbl += (int64_t)p.dbl.size();
             n_ent += (int64_t)p.ent.size();
             b.n += p.n;
             b.dmax = std::max(b.dmax, p.dmax);
@@ -396,6 +421,7 @@ void build_blocks(const qts_ensemble* e, bool grad, BlockHost* out) {
     out->n_blocks = n_blk;
     out->n_slots = n_slot;
     out->rec.resize((size_t)n_rec);
+    out->dbl.resize((size_t)n_dbl);
     if (grad) {
         out->ent.resize((size_t)n_ent);
     }
@@ -405,6 +431,7 @@ void build_blocks(const qts_ensemble* e, bool grad, BlockHost* out) {
             const Place& a = at[(size_t)k * kKeys + key];
             if (p.n == 0) continue;
             std::memcpy(out->rec.data() + a.rec, p.rec.data(), p.rec.size() * sizeof(Rec32));
+            if (!p.dbl.empty()) std::memcpy(out->dbl.data() + a.dbl, p.dbl.data(), p.dbl.size() * sizeof(double));
             if (!grad) continue;
             const int64_t stride = key / (kBlkMaxH + 1) + blk_slots(key % (kBlkMaxH + 1));
             const BlockEntry* src = p.ent.data();

@@ -37,6 +37,10 @@
 // stored as pairs.  [lo, hi) is what the splits above leave of the feature's range
 // (all of it but at r); word: the feature, kNanOk and kDefLeft.
 //
+// FP64 ensembles keep the FP64 weights beside the records, per block: val (h = 0),
+// z of the D elements, zL and zR of the inner nodes, {valL, valR, zL, zR, vz} of the
+// pair nodes.
+//
 // Adjoint sums of a block ("slots"): the z-gradients of its D elements, of every
 // inner node's two edges, then per pair node Q and for each leaf K (dL/dval = z Q
 // + K, dL/dz = val Q).  h = 0: the D z-gradients and the leaf value's gradient.
@@ -70,6 +74,12 @@ QTS_HD constexpr int blk_rec(int h, int n) {
 }
 QTS_HD constexpr int blk_slot(int h, int n) { return blk_rec(h, n); }
 QTS_HD constexpr int blk_slots(int h) { return h == 0 ? 1 : 2 * blk_inner(h) + 3 * blk_pairs(h); }
+
+// FP64 values of a block, and the offset of node n's among them
+QTS_HD constexpr int blk_doubles(int D, int h) { return 1 + D + 2 * blk_inner(h) + 5 * blk_pairs(h); }
+QTS_HD constexpr int blk_dbl(int D, int h, int n) {
+    return 1 + D + (n <= blk_inner(h) ? 2 * (n - 1) : 2 * blk_inner(h) + 5 * (n - 1 - blk_inner(h)));
+}
 
 // Relative cost of a block: about the instructions per warp of the forward pass
 // (36 per shared element, 65 per inner and 36 per pair node, 25 for the rest).

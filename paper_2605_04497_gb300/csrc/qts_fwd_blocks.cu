@@ -53,7 +53,7 @@ struct FbArgs {
 
 // Register classes by width; each runs NP quadrature nodes per pass.
 __host__ __device__ constexpr int fb_class(int D) { return D <= 5 ? 0 : D <= 8 ? 1 : D <= 12 ? 2 : D <= 16 ? 3 : 4; }
-constexpr int kFbClasses = 5;
+[[maybe_unused]] constexpr int kFbClasses = 5;
 // nodes per pass of a class for a rule of n_pad points (padded to pairs)
 static inline int fb_np(int cls, int n_pad) {
     int np = cls == 0 ? 8 : cls <= 3 ? 4 : 2;
@@ -223,6 +223,22 @@ QTS_INST(4, 2)
 static size_t fb_smem(int F, int nphi, int stage) {
     const size_t tiles = ((size_t)(1 + nphi) * (F + 1) * kTileLd * 4 + 15) & ~(size_t)15;
     return tiles + 2 * (size_t)stage * sizeof(Rec32) + 2 * sizeof(uint64_t);
+}
+
+// phi[:, :F] = 0, phi[:, F] = E[f]
+__global__ void phi_init_kernel(double* phi, int64_t M, int F, double bias) {
+    const int64_t n = M * (F + 1);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        phi[i] = (i % (F + 1) == F) ? bias : 0.0;
+}
+
+cudaError_t launch_phi_init(double* phi, int64_t M, int F, double bias, cudaStream_t st) {
+    if (M <= 0) return cudaSuccess;
+    const int64_t n = M * (F + 1);
+    const int blocks = (int)std::min<int64_t>((n + 255) / 256, 4 * 152);
+    phi_init_kernel<<<blocks, 256, 0, st>>>(phi, M, F, bias);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* phi,

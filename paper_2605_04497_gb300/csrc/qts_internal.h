@@ -140,6 +140,7 @@ struct BlockBucket {  // all blocks of one width and height
     int dmax = 0;           // most unique features on a path of theirs
     int64_t n = 0;
     int64_t rec_off = 0;    // first record
+    int64_t dbl_off = 0;    // first FP64 value (QTS_FLAG_FP64; n * blk_doubles(D, h) of them)
     int64_t slot_off = 0;   // first adjoint sum (n * (D + blk_slots(h)) of them)
 };
 struct BlockEntry {  // one term of a gradient: += coef * the block's sum
@@ -150,12 +151,14 @@ struct BlockEntry {  // one term of a gradient: += coef * the block's sum
 struct BlockHost {
     std::vector<BlockBucket> buckets;
     std::vector<Rec32> rec;
+    std::vector<double> dbl;           // QTS_FLAG_FP64: weights and leaf values in FP64
     std::vector<BlockEntry> ent;       // adjoint only, as the rest
     std::vector<double> bias_leaf, bias_z;  // per node: d E[f] / d leaf value, d z
     int64_t n_blocks = 0, n_slots = 0;
 };
 struct BlockDev {
     Rec32* rec = nullptr;
+    double* dbl = nullptr;
     BlockEntry* ent = nullptr;
     int64_t n_ent = 0;
     double *bias_leaf = nullptr, *bias_z = nullptr;
@@ -288,12 +291,13 @@ qts_status check_call(qts_ensemble* e, const float* X, int64_t M, int32_t F, int
 
 cudaError_t launch_phi_init(double* phi, int64_t M, int F, double bias, cudaStream_t st);
 cudaError_t launch_wait_selftest(int* status, cudaStream_t st);
-cudaError_t launch_fwd_bucket(const qts_ensemble* e, const Bucket& b, const float* X, int64_t M,
-                              int F, const QuadF& q, const QuadD& qd, double* phi, const Tune& tn,
-                              cudaStream_t st);
-// first-order values of more than kFewRows samples on the block tables
+// first-order values on the block tables: FP32 (any M), FP32 for M <= kFewRows, FP64
 cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* phi,
                               cudaStream_t st);
+cudaError_t launch_fwd_few(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* phi,
+                           cudaStream_t st);
+cudaError_t launch_fwd64(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* phi,
+                         cudaStream_t st);
 // pairs: b is a bucket of the sibling-pair tables (e->bprep), else of e->prep
 cudaError_t launch_int_bucket(const qts_ensemble* e, const Bucket& b, bool pairs, const float* X, int64_t M,
                               int F, const QuadF& q, double* acc_pair, double* acc_phi,

@@ -9,12 +9,15 @@
 namespace qts {
 
 // How a path adds its phi contributions to the shared tile.
-enum PhiMode : int { kPhiNone = 0, kPhiAtomic = 1, kPhiPrivate = 2 };
+// kPhiAtomicNz skips zeros: lanes that hold different blocks meet at the zero
+// row of absent elements, where atomics would serialise.
+enum PhiMode : int { kPhiAtomic = 1, kPhiPrivate = 2, kPhiAtomicNz = 3 };
 
 template <int MODE>
 __device__ __forceinline__ void phi_add(float* ps, int idx, float v) {
     if constexpr (MODE == kPhiAtomic) atomicAdd(&ps[idx], v);
     else if constexpr (MODE == kPhiPrivate) ps[idx] += v;  // tile owned by this warp
+    else if (v != 0.f) atomicAdd(&ps[idx], v);
 }
 
 // Per-lane reads of one sample's values by feature index.
@@ -29,123 +32,6 @@ struct GlobalCols {  // transposed global copy [feature][ld]; this lane's sample
     int64_t s;
     __device__ __forceinline__ float operator()(int f) const { return __ldg(t + (int64_t)f * ld + s); }
 };
-
-// ====================================================== first order ======
-//
-// c_i = sum_m w_m val prod_{j<i} a_j(t_m) prod_{j>i} a_j(t_m), a_j(t) = z_j + t (o_j - z_j),
-// by a prefix product seeded with w_m val and a suffix product (no division),
-// two quadrature nodes per f32x2 register pair; phi[f_i] += (o_i - z_i) c_i
-// (Thm 1 with S = {i}, Eq. shap_as_weighted_banzhafs).
-
-
-template <int D, int NP, bool HAS_NAN, typename XR, int PHI = kPhiAtomic, bool PAIRS = false>
-__device__ __forceinline__ void fwd_path_f32(const Rec32* __restrict__ r, const XR& xr, float* ps, int lane,
-                                             const QuadF& q) {
-    constexpr int K = NP / 2;  // node pairs per pass
-    const float val = r[0].z;
-    const bool pair = PAIRS && (r[D].bits & kPairElem) != 0;
-    float dd[D], zz[D];
-    int ff[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-        const Rec32 e = r[1 + j];
-        const int f = feat_of(e.bits);
-        const float x = xr(f);
-        const bool o = satisfies<HAS_NAN>(x, e.lo, e.hi, e.bits);
-        dd[j] = (o ? 1.f : 0.f) - e.z;
-        if (j == D - 1 && pair) dd[j] = pair_d(x, e, r[0]);
-        zz[j] = e.z;
-        ff[j] = f;
-    }
-    float cacc[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) cacc[j] = 0.f;
-    const int npass = q.n_pad / NP;
-    for (int pass = 0; pass < npass; ++pass) {
-        float2 T[K], P[D][K], A[D][K], S[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int m = pass * NP + 2 * k;
-            T[k] = f2(q.t[m], q.t[m + 1]);
-            P[0][k] = f2(q.w[m] * val, q.w[m + 1] * val);
-        }
-        // prefix products P_j = w val prod_{l<j} a_l
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                A[j][k] = fma2(T[k], f2s(dd[j]), f2s(zz[j]));
-                if (j + 1 < D) P[j + 1][k] = mul2(P[j][k], A[j][k]);
-            }
-        }
-        // suffix products, combined on the way down
-#pragma unroll
-        for (int k = 0; k < K; ++k) S[k] = f2s(1.f);
-#pragma unroll
-        for (int j = D - 1; j >= 0; --j) {
-            float2 acc = mul2(P[j][0], S[0]);
-#pragma unroll
-            for (int k = 1; k < K; ++k) acc = fma2(P[j][k], S[k], acc);
-            if (j > 0) {
-#pragma unroll
-                for (int k = 0; k < K; ++k) S[k] = mul2(S[k], A[j][k]);
-            }
-            cacc[j] += acc.x + acc.y;
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < D; ++j) phi_add<PHI>(ps, ff[j] * kTileLd + lane, dd[j] * cacc[j]);
-}
-
-
-// ps: the block's FP64 accumulator tile [feature][kTileLd] (column = lane), or,
-// with global_F = F > 0 (the tile does not fit shared memory), this lane's row
-// of the FP64 output itself; lanes past the last sample pass live = false.
-template <int D, bool HAS_NAN>
-__device__ __forceinline__ void fwd_path_f64(const Rec64* __restrict__ r, const float* __restrict__ xs,
-                                             double* ps, int lane, const QuadD& q, int global_F = 0,
-                                             bool live = true) {
-    const double val = r[0].z;
-    double dd[D], zz[D], cacc[D];
-    int ff[D];
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-        const Rec64 e = r[1 + j];
-        const int f = feat_of(e.bits);
-        const float x = xs[f * kTileLd + lane];
-        const bool o = satisfies<HAS_NAN>(x, e.lo, e.hi, e.bits);
-        dd[j] = (o ? 1.0 : 0.0) - e.z;
-        zz[j] = e.z;
-        ff[j] = f;
-        cacc[j] = 0.0;
-    }
-    for (int m = 0; m < q.n; ++m) {
-        const double t = q.t[m];
-        double A[D], P[D];
-        P[0] = q.w[m] * val;
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-            A[j] = fma(t, dd[j], zz[j]);
-            if (j + 1 < D) P[j + 1] = P[j] * A[j];
-        }
-        double S = 1.0;
-#pragma unroll
-        for (int j = D - 1; j >= 0; --j) {
-            cacc[j] += P[j] * S;
-            S *= A[j];
-        }
-    }
-    if (!live) return;
-    if (global_F == 0) {
-#pragma unroll
-        for (int j = 0; j < D; ++j) atomicAdd(&ps[ff[j] * kTileLd + lane], dd[j] * cacc[j]);
-    } else {
-#pragma unroll
-        for (int j = 0; j < D; ++j)
-            if (ff[j] < global_F) atomicAdd(&ps[ff[j]], dd[j] * cacc[j]);  // padding elements carry feature F
-    }
-}
-
 
 // =========================================================== adjoint =====
 
