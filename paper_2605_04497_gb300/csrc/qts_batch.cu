@@ -11,7 +11,9 @@
 //
 // Bound by instruction issue and FP32 (8 to 16 warps per SM).  Measured, path
 // tables before and block tables now: eight requests of 17-100 trees, depth 4-13,
-// 40-2,000 samples 8.61 -> 4.60 ms; sixteen of at most 200 samples 3.28 -> 0.38 ms (by
+// 40-2,000 samples 8.61 -> 4.60 ms (4.16 with the classes' kernels as parallel
+// branches); sixteen of at most 200 samples 3.28 -> 0.38 ms (0.17 with one launch for
+// all requests' preparation and epilogue; by
 // default the warps of a thread block now share 64 samples and split the blocks:
 // with 64 samples per warp a request of fewer than 193 left warps idle); adjoint
 // alone, 200 trees of depth 8, 4,001 samples 3.30 -> 2.00 ms.
@@ -54,7 +56,7 @@ struct ReqDev {
     int64_t M;
     int64_t Mpad;
     int32_t F;
-    int32_t pad;
+    int32_t cat;        // categorical elements: always the NaN-aware variant
     const int* has_nan;
     int* status;
 };
@@ -139,7 +141,7 @@ __device__ __forceinline__ bool batch_item(const ItemCtx& c) {
     const ReqDev& rq = c.rq;
     const int F = rq.F;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool has_nan = *rq.has_nan != 0;
+    const bool has_nan = *rq.has_nan != 0 || rq.cat != 0;
     constexpr int kSlots = D + blk_slots(H);
     constexpr int ld = SP ? kTileLd2 : kTileLd;
     const bool own = SP && sg.mode == 2;  // every warp has its own samples
@@ -290,29 +292,149 @@ QTS_INST(64, false)
 
 #if QTS_HOST_PART
 
-// out[c * Mpad + s] = in[s * ld + c] for c < ncols, s < M; zero elsewhere
-// (rows up to nrows, columns up to Mpad).
-__global__ void transpose_pad_kernel(const float* __restrict__ in, int64_t M, int ncols, int64_t ld,
-                                     float* __restrict__ out, int nrows, int64_t Mpad, int* has_nan) {
+// Everything a call does around its persistent kernels, for all requests at
+// once: each thread block finds its request and its part of that request's work by
+// its index (a call of sixteen small requests spent two thirds of its time in
+// about a hundred launches of 3 us each).
+struct ReqWork {
+    const float* X;
+    const float* G;       // nullptr: forward only
+    float *XT, *GT;       // transposed copies
+    double* phi;          // or nullptr
+    double *gb, *g;       // G = sum of grad_phi's last column; adjoint sums
+    int* flag;            // some x is NaN
+    const BlockEntry* ent;
+    const double *bias_leaf, *bias_z;
+    double *d_leaf, *d_z;
+    double bias;
+    int64_t M, Mpad, n_g, n_ent, n_nodes;
+    int64_t begin, bias_begin, ent_begin;  // first thread block in the three kernels
+    int32_t F;
+    int32_t pad;
+};
+constexpr int kInitChunk = 8192;    // doubles per thread block set to zero or E[f]
+constexpr int kNodeChunk = 4096;    // nodes per thread block of batch_bias_kernel
+constexpr int kEntryChunk = 4096;   // entries per thread block of batch_entries_kernel
+
+inline int64_t chunks_of(int64_t n, int64_t c) { return (n + c - 1) / c; }
+// thread blocks of batch_prepare_kernel for one request: transposed copies of X and
+// G, phi, adjoint sums, G's last column
+__host__ __device__ inline int64_t prepare_tiles(const ReqWork& w) { return w.Mpad / 32 * ((w.F + 32) / 32); }
+inline int64_t prepare_blocks(const ReqWork& w) {
+    return prepare_tiles(w) * (w.G ? 2 : 1) + (w.phi ? chunks_of(w.M * (w.F + 1), kInitChunk) : 0) +
+           (w.G ? chunks_of(w.n_g, kInitChunk) + 1 : 0);
+}
+
+// out[c * Mpad + s] = in[s * ld + c] for c < ncols, s < M; zero elsewhere (up to
+// row nrows - 1, column Mpad - 1).
+__device__ __forceinline__ void transpose_tile(const float* __restrict__ in, int64_t M, int ncols, int64_t ld,
+                                               float* __restrict__ out, int nrows, int64_t Mpad, int* has_nan,
+                                               int64_t s0, int c0) {
     __shared__ float tile[32][33];
-    const int64_t s0 = (int64_t)blockIdx.x * 32;
-    const int c0 = blockIdx.y * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     int nan_seen = 0;
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+    for (int r = ty; r < 32; r += 8) {
         const int64_t s = s0 + r;
-        const int c = c0 + threadIdx.x;
+        const int c = c0 + tx;
         float v = 0.f;
         if (s < M && c < ncols) v = in[s * ld + c];
         nan_seen |= (v != v);
-        tile[r][threadIdx.x] = v;
+        tile[r][tx] = v;
     }
     __syncthreads();
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+    for (int r = ty; r < 32; r += 8) {
         const int c = c0 + r;
-        const int64_t s = s0 + threadIdx.x;
-        if (c < nrows && s < Mpad) out[(int64_t)c * Mpad + s] = tile[threadIdx.x][r];
+        const int64_t s = s0 + tx;
+        if (c < nrows && s < Mpad) out[(int64_t)c * Mpad + s] = tile[tx][r];
     }
     if (has_nan && nan_seen) atomicOr(has_nan, 1);
+}
+
+template <int64_t ReqWork::*BEGIN>
+__device__ __forceinline__ const ReqWork& find_work(const ReqWork* w, int n) {
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (w[mid].*BEGIN <= (int64_t)blockIdx.x) lo = mid;
+        else hi = mid - 1;
+    }
+    return w[lo];
+}
+
+struct WorkArgs {
+    const ReqWork* many;  // nullptr: one
+    int n;
+    ReqWork one;
+};
+
+__global__ void __launch_bounds__(256) batch_prepare_kernel(const __grid_constant__ WorkArgs a) {
+    const ReqWork& w = a.many ? find_work<&ReqWork::begin>(a.many, a.n) : a.one;
+    int64_t k = (int64_t)blockIdx.x - w.begin;
+    const int64_t tiles = prepare_tiles(w);
+    const int rows = (w.F + 32) / 32;
+    if (k < tiles) {
+        transpose_tile(w.X, w.M, w.F, w.F, w.XT, w.F + 1, w.Mpad, w.flag, k / rows * 32, (int)(k % rows) * 32);
+        return;
+    }
+    k -= tiles;
+    if (w.G) {
+        if (k < tiles) {
+            transpose_tile(w.G, w.M, w.F + 1, w.F + 1, w.GT, w.F + 1, w.Mpad, nullptr, k / rows * 32,
+                           (int)(k % rows) * 32);
+            return;
+        }
+        k -= tiles;
+    }
+    if (w.phi) {
+        const int64_t n = w.M * (w.F + 1), c = (n + kInitChunk - 1) / kInitChunk;
+        if (k < c) {
+            const int64_t end = imin64(n, (k + 1) * kInitChunk);
+            for (int64_t i = k * kInitChunk + threadIdx.x; i < end; i += blockDim.x)
+                w.phi[i] = (i % (w.F + 1) == w.F) ? w.bias : 0.0;
+            return;
+        }
+        k -= c;
+    }
+    const int64_t c = (w.n_g + kInitChunk - 1) / kInitChunk;
+    if (k < c) {
+        const int64_t end = imin64(w.n_g, (k + 1) * kInitChunk);
+        for (int64_t i = k * kInitChunk + threadIdx.x; i < end; i += blockDim.x) w.g[i] = 0.0;
+        return;
+    }
+    double acc = 0.0;
+    for (int64_t s = threadIdx.x; s < w.M; s += blockDim.x) acc += (double)w.G[s * (w.F + 1) + w.F];
+    for (int off = 16; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    __shared__ double part[8];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int i = 0; i < 8; ++i) t += part[i];
+        *w.gb = t;
+    }
+}
+
+// Both gradients start at their share of E[f]'s, G times a constant per node, ...
+__global__ void __launch_bounds__(256) batch_bias_kernel(const __grid_constant__ WorkArgs a) {
+    const ReqWork& w = a.many ? find_work<&ReqWork::bias_begin>(a.many, a.n) : a.one;
+    const int64_t k = (int64_t)blockIdx.x - w.bias_begin;
+    const double G = *w.gb;
+    const int64_t end = imin64(w.n_nodes, (k + 1) * kNodeChunk);
+    for (int64_t i = k * kNodeChunk + threadIdx.x; i < end; i += blockDim.x) {
+        w.d_leaf[i] = G * w.bias_leaf[i];
+        w.d_z[i] = G * w.bias_z[i];
+    }
+}
+
+// ... then every block's sums are chained to its leaves and edges.
+__global__ void __launch_bounds__(256) batch_entries_kernel(const __grid_constant__ WorkArgs a) {
+    const ReqWork& w = a.many ? find_work<&ReqWork::ent_begin>(a.many, a.n) : a.one;
+    const int64_t k = (int64_t)blockIdx.x - w.ent_begin;
+    const int64_t end = imin64(w.n_ent, (k + 1) * kEntryChunk);
+    for (int64_t i = k * kEntryChunk + threadIdx.x; i < end; i += blockDim.x) {
+        const BlockEntry e = w.ent[i];
+        atomicAdd(((e.target & 1u) ? w.d_leaf : w.d_z) + (e.target >> 1), e.coef * w.g[e.slot]);
+    }
 }
 
 // ------------------------------------------------------------- host side --
@@ -382,12 +504,52 @@ static BatchWork batch_work(const qts_ensemble* e, int64_t M, int F, bool grad) 
     return w;
 }
 
-static cudaError_t launch_transpose(const float* in, int64_t M, int ncols, int64_t ld, float* out, int nrows,
-                                    int64_t Mpad, int* has_nan, cudaStream_t st) {
-    if (Mpad == 0) return cudaSuccess;
-    dim3 grid((unsigned)(Mpad / 32), (unsigned)((nrows + 31) / 32));
-    transpose_pad_kernel<<<grid, dim3(32, 8), 0, st>>>(in, M, ncols, ld, out, nrows, Mpad, has_nan);
-    return cudaGetLastError();
+static ReqWork request_work(const qts_request& R) {
+    qts_ensemble* e = R.ens;
+    const BatchWork bw = batch_work(e, R.M, R.F, R.grad_phi != nullptr);
+    char* base = (char*)e->d_work;
+    ReqWork w;
+    std::memset(&w, 0, sizeof(w));
+    w.X = R.X;
+    w.G = R.grad_phi;
+    w.XT = (float*)(base + bw.xt_off);
+    w.GT = (float*)(base + bw.gt_off);
+    w.phi = R.phi;
+    w.flag = (int*)(base + bw.flag_off);
+    w.bias = e->prep.bias;
+    w.M = R.M;
+    w.Mpad = bw.Mpad;
+    w.F = R.F;
+    if (R.grad_phi) {
+        w.gb = (double*)base;
+        w.g = (double*)base + kGradHead;
+        w.n_g = e->n_blk_slots;
+        w.ent = e->blkdev.ent;
+        w.n_ent = e->blkdev.n_ent;
+        w.bias_leaf = e->blkdev.bias_leaf;
+        w.bias_z = e->blkdev.bias_z;
+        w.n_nodes = e->n_nodes;
+        w.d_leaf = R.d_leaf;
+        w.d_z = R.d_z;
+    }
+    return w;
+}
+
+struct WorkBlocks {
+    int64_t prepare = 0, bias = 0, entries = 0;
+};
+
+static void number_work(ReqWork& w, WorkBlocks* n) {
+    w.begin = n->prepare;
+    w.bias_begin = n->bias;
+    w.ent_begin = n->entries;
+    n->prepare += prepare_blocks(w);
+    n->bias += chunks_of(w.n_nodes, kNodeChunk);
+    n->entries += chunks_of(w.n_ent, kEntryChunk);
+}
+
+static ReqDev request_dev(const ReqWork& w, const qts_ensemble* e) {
+    return {w.XT, w.G ? w.GT : nullptr, w.phi, w.M, w.Mpad, w.F, e->prep.has_cat ? 1 : 0, w.flag, e->d_status};
 }
 
 // Per-width launch choices that override the ensembles' own while tuning:
@@ -545,92 +707,108 @@ static cudaError_t launch_ordered(const LaunchHost& l, BatchArgs& a, unsigned lo
     }
 }
 
+constexpr size_t kBatchBranches = 8;  // parallel branches of persistent kernels in a graph
+
 static qts_status build_plan(int n, const qts_request* reqs, int n_quad, BatchPlan* plan,
                              cudaStream_t cap, const BatchOverride* ov = nullptr) {
     std::vector<SegHost> segs;
     std::vector<ReqDev> rd(n);
+    std::vector<ReqWork> rw(n);
+    WorkBlocks nb;
+    const size_t flag_bytes = 256 * ((sizeof(int) * (size_t)n + 255) / 256);
     for (int r = 0; r < n; ++r) {
         const qts_request& R = reqs[r];
-        qts_ensemble* e = R.ens;
-        const bool grad = R.grad_phi != nullptr;
-        const BatchWork bw = batch_work(e, R.M, R.F, grad);
-        char* wbase = (char*)e->d_work;
-        rd[r] = {(const float*)(wbase + bw.xt_off), grad ? (const float*)(wbase + bw.gt_off) : nullptr, R.phi,
-                 R.M, bw.Mpad, R.F, 0, (const int*)(wbase + bw.flag_off), e->d_status};
+        rw[r] = request_work(R);
+        number_work(rw[r], &nb);
         if (R.M > 0) request_segments(R, r, n_quad, ov, &segs);
     }
     const std::vector<LaunchHost> launches = order_segments(segs, (size_t)1 << 30);
-    const size_t seg_bytes = (sizeof(SegDev) * std::max<size_t>(segs.size(), 1) + 255) / 256 * 256;
-    const size_t req_bytes = (sizeof(ReqDev) * std::max(n, 1) + 255) / 256 * 256;
-    const size_t cnt_bytes = (sizeof(unsigned long long) * std::max<size_t>(launches.size(), 1) + 255) / 256 * 256;
-    cudaError_t ce = cudaMalloc(&plan->dev, seg_bytes + req_bytes + cnt_bytes);
+    auto pad = [](size_t v) { return (v + 255) / 256 * 256; };
+    const size_t seg_bytes = pad(sizeof(SegDev) * std::max<size_t>(segs.size(), 1));
+    const size_t req_bytes = pad(sizeof(ReqDev) * (size_t)n), work_bytes = pad(sizeof(ReqWork) * (size_t)n);
+    const size_t cnt_bytes = pad(sizeof(unsigned long long) * std::max<size_t>(launches.size(), 1));
+    cudaError_t ce = cudaMalloc(&plan->dev, seg_bytes + req_bytes + work_bytes + cnt_bytes + flag_bytes);
     if (ce != cudaSuccess) return cuda_fail(ce, "batch plan allocation");
-    SegDev* d_segs = (SegDev*)plan->dev;
-    ReqDev* d_reqs = (ReqDev*)((char*)plan->dev + seg_bytes);
-    unsigned long long* d_cnt = (unsigned long long*)((char*)plan->dev + seg_bytes + req_bytes);
+    char* base = (char*)plan->dev;
+    SegDev* d_segs = (SegDev*)base;
+    ReqDev* d_reqs = (ReqDev*)(base + seg_bytes);
+    ReqWork* d_work = (ReqWork*)(base + seg_bytes + req_bytes);
+    unsigned long long* d_cnt = (unsigned long long*)(base + seg_bytes + req_bytes + work_bytes);
+    int* d_flag = (int*)(base + seg_bytes + req_bytes + work_bytes + cnt_bytes);
+    for (int r = 0; r < n; ++r) {
+        rw[r].flag = d_flag + r;
+        rd[r] = request_dev(rw[r], reqs[r].ens);
+    }
     std::vector<SegDev> sd(segs.size());
     for (size_t i = 0; i < segs.size(); ++i) sd[i] = segs[i].d;
     if (!sd.empty()) ce = cudaMemcpy(d_segs, sd.data(), sizeof(SegDev) * sd.size(), cudaMemcpyHostToDevice);
     if (ce == cudaSuccess) ce = cudaMemcpy(d_reqs, rd.data(), sizeof(ReqDev) * n, cudaMemcpyHostToDevice);
+    if (ce == cudaSuccess) ce = cudaMemcpy(d_work, rw.data(), sizeof(ReqWork) * n, cudaMemcpyHostToDevice);
     if (ce != cudaSuccess) return cuda_fail(ce, "batch plan upload");
 
     ce = cudaEventCreate(&plan->ev0);
     if (ce == cudaSuccess) ce = cudaEventCreate(&plan->ev1);
     if (ce != cudaSuccess) return cuda_fail(ce, "batch plan events");
-    // capture: init, persistent kernel(s), epilogues
-    ce = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-    if (ce != cudaSuccess) return cuda_fail(ce, "graph capture begin");
+    // capture: preparation, persistent kernels, epilogue.  The persistent kernels
+    // (and the gradients' start values) are branches of the graph, so one class's
+    // last items run beside the next one's first.
+    std::vector<cudaStream_t> side(std::min<size_t>(launches.size(), kBatchBranches), nullptr);
+    std::vector<cudaEvent_t> done(side.size() + 1, nullptr);
+    for (auto& x : side)
+        if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
+    for (auto& x : done)
+        if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
+    auto drop = [&] {
+        for (auto& x : side)
+            if (x) cudaStreamDestroy(x);
+        for (auto& x : done)
+            if (x) cudaEventDestroy(x);
+    };
+    if (ce == cudaSuccess) ce = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    if (ce != cudaSuccess) {
+        drop();
+        return cuda_fail(ce, "graph capture begin");
+    }
     int kernels = 0;
     cudaError_t err = cudaSuccess;
-    for (int r = 0; r < n && err == cudaSuccess; ++r) {
-        const qts_request& R = reqs[r];
-        const bool grad = R.grad_phi != nullptr;
-        const BatchWork bw = batch_work(R.ens, R.M, R.F, grad);
-        char* wbase = (char*)R.ens->d_work;
-        if (R.phi && R.M > 0) {
-            err = launch_phi_init(R.phi, R.M, R.F, R.ens->prep.bias, cap);
-            ++kernels;
+    WorkArgs wa;
+    std::memset(&wa, 0, sizeof(wa));
+    wa.many = d_work;
+    wa.n = n;
+    auto work = [&](auto kernel, int64_t blocks, cudaStream_t st) {
+        if (blocks <= 0 || err != cudaSuccess) return;
+        if (blocks > 0x7fffffffLL) {
+            err = cudaErrorInvalidConfiguration;
+            return;
         }
-        if (grad && err == cudaSuccess) err = cudaMemsetAsync(wbase, 0, bw.grad_bytes, cap);
-        // the NaN flag starts set for ensembles with categorical elements, so
-        // their items take the NaN-aware (categorical-aware) variant
-        if (err == cudaSuccess)
-            err = cudaMemsetAsync(wbase + bw.flag_off, R.ens->prep.has_cat ? 1 : 0, 256, cap);
-        if (R.M > 0 && err == cudaSuccess) {
-            err = launch_transpose(R.X, R.M, R.F, R.F, (float*)(wbase + bw.xt_off), R.F + 1, bw.Mpad,
-                                   (int*)(wbase + bw.flag_off), cap);
-            ++kernels;
-            if (grad && err == cudaSuccess) {
-                err = launch_transpose(R.grad_phi, R.M, R.F + 1, R.F + 1, (float*)(wbase + bw.gt_off), R.F + 1,
-                                       bw.Mpad, nullptr, cap);
-                ++kernels;
-            }
-        }
-    }
-    if (err == cudaSuccess) err = cudaMemsetAsync(d_cnt, 0, cnt_bytes, cap);
+        kernel<<<(unsigned)blocks, 256, 0, st>>>(wa);
+        err = cudaGetLastError();
+        ++kernels;
+    };
+    err = cudaMemsetAsync(d_cnt, 0, cnt_bytes + flag_bytes, cap);
+    work(batch_prepare_kernel, nb.prepare, cap);
     if (err == cudaSuccess) err = cudaEventRecordWithFlags(plan->ev0, cap, cudaEventRecordExternal);
+    if (err == cudaSuccess) err = cudaEventRecord(done.back(), cap);
+    for (size_t b = 0; b < side.size() && err == cudaSuccess; ++b) err = cudaStreamWaitEvent(side[b], done.back(), 0);
     for (size_t c = 0; c < launches.size() && err == cudaSuccess; ++c) {
         BatchArgs a;
         a.segs = d_segs + launches[c].first;
         a.reqs = d_reqs;
-        err = launch_ordered(launches[c], a, d_cnt + c, cap);
+        err = launch_ordered(launches[c], a, d_cnt + c, side[c % side.size()]);
         ++kernels;
     }
-    if (err == cudaSuccess) err = cudaEventRecordWithFlags(plan->ev1, cap, cudaEventRecordExternal);
-    for (int r = 0; r < n && err == cudaSuccess; ++r) {
-        const qts_request& R = reqs[r];
-        if (!R.grad_phi) continue;
-        if (R.M > 0) {
-            double* gb = (double*)R.ens->d_work;
-            err = launch_bwd_epilogue_blocks(R.ens, R.grad_phi, R.M, R.F, gb + kGradHead, R.d_leaf, R.d_z, gb, cap);
-            kernels += 2 + (R.ens->blkdev.n_ent > 0);
-        } else {
-            err = cudaMemsetAsync(R.d_leaf, 0, sizeof(double) * R.ens->n_nodes, cap);
-            if (err == cudaSuccess) err = cudaMemsetAsync(R.d_z, 0, sizeof(double) * R.ens->n_nodes, cap);
-        }
+    work(batch_bias_kernel, nb.bias, cap);
+    for (size_t b = 0; b < side.size(); ++b) {
+        // join every branch, also after an error: the capture must end whole
+        cudaError_t j = cudaEventRecord(done[b], side[b]);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(cap, done[b], 0);
+        if (err == cudaSuccess) err = j;
     }
+    if (err == cudaSuccess) err = cudaEventRecordWithFlags(plan->ev1, cap, cudaEventRecordExternal);
+    work(batch_entries_kernel, nb.entries, cap);
     cudaGraph_t g = nullptr;
     ce = cudaStreamEndCapture(cap, &g);
+    drop();
     if (err != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
         return cuda_fail(err, "batched launch during capture");
@@ -859,8 +1037,6 @@ size_t adjoint_work_bytes(const qts_ensemble* e, int64_t M, int F) { return batc
 
 cudaError_t launch_adjoint_blocks(qts_ensemble* e, const float* X, const float* grad, int64_t M, int F, int n_quad,
                                   double* d_leaf, double* d_z, cudaStream_t st) {
-    const BatchWork bw = batch_work(e, M, F, true);
-    char* w = (char*)e->d_work;
     qts_request R;
     std::memset(&R, 0, sizeof(R));
     R.ens = e;
@@ -868,28 +1044,42 @@ cudaError_t launch_adjoint_blocks(qts_ensemble* e, const float* X, const float* 
     R.M = M;
     R.F = F;
     R.grad_phi = grad;
-    cudaError_t err = cudaMemsetAsync(w, 0, bw.grad_bytes, st);
-    if (err == cudaSuccess) err = cudaMemsetAsync(w + bw.flag_off, e->prep.has_cat ? 1 : 0, 256, st);
-    if (err == cudaSuccess)
-        err = launch_transpose(X, M, F, F, (float*)(w + bw.xt_off), F + 1, bw.Mpad, (int*)(w + bw.flag_off), st);
-    if (err == cudaSuccess)
-        err = launch_transpose(grad, M, F + 1, F + 1, (float*)(w + bw.gt_off), F + 1, bw.Mpad, nullptr, st);
+    R.d_leaf = d_leaf;
+    R.d_z = d_z;
+    WorkArgs wa;
+    wa.many = nullptr;
+    wa.n = 1;
+    wa.one = request_work(R);
+    WorkBlocks nb;
+    number_work(wa.one, &nb);
+    if (nb.prepare > 0x7fffffffLL || nb.bias > 0x7fffffffLL || nb.entries > 0x7fffffffLL)
+        return cudaErrorInvalidConfiguration;
     std::vector<SegHost> segs;
     request_segments(R, 0, n_quad, nullptr, &segs);
     const std::vector<LaunchHost> launches = order_segments(segs, kInlineSegs);
     if (launches.size() > kGradHead - 1) return cudaErrorInvalidConfiguration;
-    unsigned long long* counter = (unsigned long long*)w + 1;  // cleared with the sums
+    unsigned long long* counter = (unsigned long long*)wa.one.gb + 1;  // in the head before the sums
+    cudaError_t err = cudaMemsetAsync(wa.one.gb, 0, kGradHead * sizeof(double), st);
+    if (err == cudaSuccess) err = cudaMemsetAsync(wa.one.flag, 0, sizeof(int), st);
+    if (err != cudaSuccess) return err;
+    batch_prepare_kernel<<<(unsigned)nb.prepare, 256, 0, st>>>(wa);
+    err = cudaGetLastError();
     for (size_t c = 0; c < launches.size() && err == cudaSuccess; ++c) {
         BatchArgs a;
         a.segs = nullptr;
         a.reqs = nullptr;
         for (size_t i = 0; i < launches[c].count; ++i) a.seg[i] = segs[launches[c].first + i].d;
-        a.req = {(const float*)(w + bw.xt_off), (const float*)(w + bw.gt_off), nullptr, M, bw.Mpad, F, 0,
-                 (const int*)(w + bw.flag_off), e->d_status};
+        a.req = request_dev(wa.one, e);
         err = launch_ordered(launches[c], a, counter + c, st);
     }
-    double* gb = (double*)w;
-    if (err == cudaSuccess) err = launch_bwd_epilogue_blocks(e, grad, M, F, gb + kGradHead, d_leaf, d_z, gb, st);
+    if (err == cudaSuccess) {
+        batch_bias_kernel<<<(unsigned)nb.bias, 256, 0, st>>>(wa);
+        err = cudaGetLastError();
+    }
+    if (err == cudaSuccess && nb.entries > 0) {
+        batch_entries_kernel<<<(unsigned)nb.entries, 256, 0, st>>>(wa);
+        err = cudaGetLastError();
+    }
     return err;
 }
 

@@ -16,7 +16,7 @@
 // dL/dw_e = dL/dz_k * prod_{other edges e' merged into k} w_e'.
 //
 // FP32 runs on the block tables with the batched pass's kernels (qts_batch.cu);
-// this file holds the epilogues and the FP64 kernels, which run path by path:
+// this file holds the FP64 kernels, which run path by path:
 // lanes are samples, the per-path sums over a tile of 32 samples are reduced in
 // the warp and added to FP64 per-path / per-element accumulators.
 //
@@ -252,38 +252,6 @@ static cudaError_t launch_bwd_bucket(const qts_ensemble* e, const Bucket& b, con
 #undef QTS_CASE
         default: return cudaErrorInvalidValue;
     }
-}
-
-// Block tables: both gradients start at their share of E[f]'s, G times a constant
-// per node, ...
-__global__ void block_bias_kernel(int64_t n, const double* __restrict__ bias_leaf, const double* __restrict__ bias_z,
-                                  const double* __restrict__ gb, double* d_leaf, double* d_z) {
-    const double G = *gb;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        d_leaf[i] = G * bias_leaf[i];
-        d_z[i] = G * bias_z[i];
-    }
-}
-
-// ... then every block's sums are chained to its leaves and edges.
-__global__ void block_entries_kernel(int64_t n, const BlockEntry* __restrict__ ent, const double* __restrict__ g,
-                                     double* d_leaf, double* d_z) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const BlockEntry e = ent[i];
-        atomicAdd(((e.target & 1u) ? d_leaf : d_z) + (e.target >> 1), e.coef * g[e.slot]);
-    }
-}
-
-cudaError_t launch_bwd_epilogue_blocks(const qts_ensemble* e, const float* grad, int64_t M, int F, const double* g,
-                                       double* d_leaf, double* d_z, double* gb, cudaStream_t st) {
-    const BlockDev& T = e->blkdev;
-    bias_grad_kernel<<<1, 1024, 0, st>>>(grad, M, F, gb);
-    block_bias_kernel<<<(int)std::min<int64_t>((e->n_nodes + 255) / 256, 8 * 152), 256, 0, st>>>(
-        e->n_nodes, T.bias_leaf, T.bias_z, gb, d_leaf, d_z);
-    if (T.n_ent > 0)
-        block_entries_kernel<<<(int)std::min<int64_t>((T.n_ent + 255) / 256, 16 * 152), 256, 0, st>>>(
-            T.n_ent, T.ent, g, d_leaf, d_z);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_bwd_epilogue(const qts_ensemble* e, const float* grad, int64_t M, int F,

@@ -304,8 +304,6 @@ cudaError_t launch_int_bucket(const qts_ensemble* e, const Bucket& b, bool pairs
                               cudaStream_t st);
 cudaError_t launch_int_finalize(const double* acc_pair, const double* acc_phi, int64_t M, int F,
                                 double bias, float* out, cudaStream_t st);
-cudaError_t launch_bwd_epilogue_blocks(const qts_ensemble* e, const float* grad, int64_t M, int F, const double* g,
-                                       double* d_leaf, double* d_z, double* g_bias_scratch, cudaStream_t st);
 // FP32 adjoint of one request (workspace: adjoint_work_bytes, block tables with grad)
 size_t adjoint_work_bytes(const qts_ensemble* e, int64_t M, int F);
 cudaError_t launch_adjoint_blocks(qts_ensemble* e, const float* X, const float* grad, int64_t M, int F, int n_quad,
