@@ -13,7 +13,13 @@
 // FP64 accumulators in the workspace laid out [pair][sample] and
 // [feature][sample]; a finalize kernel writes the (F+1) x (F+1) matrices.
 //
-// qts-build-parts: 6 (part 0: host code; parts 1-5: the per-width kernels)
+// All widths of a register class and rule are one launch (a thread block finds
+// its segment by its index).  500 trees of depth 6 (31,449 leaves, F = 30), 2,000
+// samples: 1.78 ms with a launch per width of 512 paths per thread block, which left
+// most SMs idle on the narrow widths, 1.56 ms here.  Bound by the shared-memory
+// float atomics of the pair sums (compare-and-swap loops) at 12 warps per SM.
+//
+// qts-build-parts: 6 (part 0: host code; parts 1-5: the kernels)
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -32,11 +38,22 @@ __host__ __device__ __forceinline__ int64_t tri_index(int a, int b, int F) {
     return (int64_t)a * F - (int64_t)a * (a + 1) / 2 + (b - a - 1);
 }
 
-struct IntArgs {
+constexpr int kIntSegs = 24;
+constexpr int kIntWarps = 4;
+
+struct IntSeg {
     const Rec32* rec;
     int64_t n_paths;
-    int64_t paths_per_block;
-    int sub;
+    int64_t cta_begin;  // first thread block
+    int32_t per_cta;    // paths per thread block
+    int32_t D;
+};
+
+struct IntArgs {
+    IntSeg seg[kIntSegs];
+    int n_seg;
+    int sub;            // paths per staged sub-chunk
+    int stage;          // records per staging buffer
     int n_tiles;
     const float* X;
     int64_t M;
@@ -54,9 +71,12 @@ struct IntArgs {
 // the widest register pass a width takes (nodes per pass)
 __host__ __device__ constexpr int int_max_np(int D) { return D <= 6 ? 8 : (D <= 12 ? 4 : 2); }
 
-template <int D>
-cudaError_t launch_int_d(const IntArgs& a, int np, bool pair_smem, int warps, int64_t blocks, size_t smem,
-                         cudaStream_t st);
+// launch classes: widths up to 4, 6, 12, 16 and the padded ones above
+__host__ __device__ constexpr int int_class(int D) { return D <= 4 ? 0 : D <= 6 ? 1 : D <= 12 ? 2 : D <= 16 ? 3 : 4; }
+[[maybe_unused]] constexpr int kIntClasses = 5;
+
+template <int CLS>
+cudaError_t launch_int_c(const IntArgs& a, int np, bool pair_smem, int64_t blocks, size_t smem, cudaStream_t st);
 
 #if QTS_DEVICE_PARTS
 
@@ -169,7 +189,35 @@ __device__ __forceinline__ void int_path_f32(const Rec32* __restrict__ r, const 
 }
 
 template <int D, int NP, bool PAIR_SMEM>
-__global__ void __launch_bounds__(256) int_kernel(IntArgs a) {
+__device__ __forceinline__ bool int_segment(const IntArgs& a, const IntSeg& sg, int64_t p0, int64_t p1, bool has_nan,
+                                            int64_t s, const float* xs, float* ps, float* pt, Rec32* st0, Rec32* st1,
+                                            uint64_t* bars, uint32_t* s_phase, int* s_flag) {
+    const int lane = threadIdx.x & 31;
+    const int F = a.F;
+    if (a.group > 0) {
+        // few samples: lane (slot, sample) evaluates path slot of each group for
+        // its sample (tile column); the pair and phi tiles take atomics anyway
+        const int slot = lane / (int)a.M, col = lane - slot * (int)a.M;
+        walk_paths_grouped<Rec32, D>(sg.rec, p0, p1, a.group, slot, [&](int64_t, const Rec32* r, bool valid) {
+            if (!valid) return;
+            int_path_f32<D, NP, true, PAIR_SMEM>(r, xs, ps, pt, a.acc_pair, col, a.M, col, F, a.q);
+        });
+        __syncthreads();  // every warp's adds are in the tiles before the flush
+        return true;
+    }
+    return stream_paths<Rec32, D>(sg.rec, p0, p1, a.sub, st0, st1, bars, s_phase, s_flag, a.status,
+                                  [&](int64_t, const Rec32* r) {
+                                      if (has_nan)
+                                          int_path_f32<D, NP, true, PAIR_SMEM>(r, xs, ps, pt, a.acc_pair, s, a.M, lane,
+                                                                               F, a.q);
+                                      else
+                                          int_path_f32<D, NP, false, PAIR_SMEM>(r, xs, ps, pt, a.acc_pair, s, a.M,
+                                                                                lane, F, a.q);
+                                  });
+}
+
+template <int CLS, int NP, bool PAIR_SMEM>
+__global__ void __launch_bounds__(kIntWarps * 32) int_kernel(const __grid_constant__ IntArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int F = a.F;
     const size_t rows = F + 1;
@@ -180,17 +228,18 @@ __global__ void __launch_bounds__(256) int_kernel(IntArgs a) {
     if (PAIR_SMEM) off += (size_t)a.n_pairs * kTileLd * 4;
     off = (off + 15) & ~(size_t)15;
     Rec32* st0 = (Rec32*)(smem + off);
-    Rec32* st1 = st0 + (size_t)a.sub * (D + 1);
-    uint64_t* bars = (uint64_t*)(st1 + (size_t)a.sub * (D + 1));
+    Rec32* st1 = st0 + a.stage;
+    uint64_t* bars = (uint64_t*)(st1 + a.stage);
     __shared__ int s_flag;
     __shared__ uint32_t s_phase[2];
-
+    int si = 0;
+    while (si + 1 < a.n_seg && (int64_t)blockIdx.x >= a.seg[si + 1].cta_begin) ++si;
+    const IntSeg sg = a.seg[si];
+    const int64_t local = (int64_t)blockIdx.x - sg.cta_begin;
     const int lane = threadIdx.x & 31;
-    const int tile = (int)(blockIdx.x % (unsigned)a.n_tiles);
-    const int64_t chunk = blockIdx.x / (unsigned)a.n_tiles;
-    const int64_t s0 = (int64_t)tile * 32;
-    const int64_t p0 = chunk * a.paths_per_block;
-    const int64_t p1 = imin64(p0 + a.paths_per_block, a.n_paths);
+    const int64_t s0 = (local % a.n_tiles) * 32;
+    const int64_t p0 = (local / a.n_tiles) * sg.per_cta;
+    const int64_t p1 = imin64(p0 + sg.per_cta, sg.n_paths);
 
     if (threadIdx.x == 0) {
         mbar_init(&bars[0], 1);
@@ -202,28 +251,39 @@ __global__ void __launch_bounds__(256) int_kernel(IntArgs a) {
     if (PAIR_SMEM)
         for (int64_t idx = threadIdx.x; idx < a.n_pairs * kTileLd; idx += blockDim.x) pt[idx] = 0.f;
     const bool has_nan = load_tile_t(xs, a.X, s0, a.M, F, F, 1) || a.cat != 0;
-    const int64_t s = s0 + lane;
-
-    bool ok;
-    if (a.group > 0) {
-        // few samples: lane (slot, sample) evaluates path slot of each group for
-        // its sample (tile column); the pair and phi tiles take atomics anyway
-        const int slot = lane / (int)a.M, col = lane - slot * (int)a.M;
-        walk_paths_grouped<Rec32, D>(a.rec, p0, p1, a.group, slot, [&](int64_t, const Rec32* r, bool valid) {
-            if (!valid) return;
-            if (has_nan) int_path_f32<D, NP, true, PAIR_SMEM>(r, xs, ps, pt, a.acc_pair, col, a.M, col, F, a.q);
-            else int_path_f32<D, NP, false, PAIR_SMEM>(r, xs, ps, pt, a.acc_pair, col, a.M, col, F, a.q);
-        });
-        ok = true;
-        __syncthreads();  // every warp's adds are in the tiles before the flush
+    bool ok = false;
+#define QTS_CASE(DD)                                                                                              \
+    case DD:                                                                                                      \
+        ok = int_segment<DD, NP, PAIR_SMEM>(a, sg, p0, p1, has_nan, s0 + lane, xs, ps, pt, st0, st1, bars, s_phase, \
+                                            &s_flag);                                                             \
+        break;
+    if constexpr (CLS == 0) {
+        switch (sg.D) {
+            QTS_CASE(1) QTS_CASE(2) QTS_CASE(3) QTS_CASE(4)
+            default: break;
+        }
+    } else if constexpr (CLS == 1) {
+        switch (sg.D) {
+            QTS_CASE(5) QTS_CASE(6)
+            default: break;
+        }
+    } else if constexpr (CLS == 2) {
+        switch (sg.D) {
+            QTS_CASE(7) QTS_CASE(8) QTS_CASE(9) QTS_CASE(10) QTS_CASE(11) QTS_CASE(12)
+            default: break;
+        }
+    } else if constexpr (CLS == 3) {
+        switch (sg.D) {
+            QTS_CASE(13) QTS_CASE(14) QTS_CASE(15) QTS_CASE(16)
+            default: break;
+        }
     } else {
-        ok = stream_paths<Rec32, D>(
-            a.rec, p0, p1, a.sub, st0, st1, bars, s_phase, &s_flag, a.status,
-            [&](int64_t, const Rec32* r) {
-                if (has_nan) int_path_f32<D, NP, true, PAIR_SMEM>(r, xs, ps, pt, a.acc_pair, s, a.M, lane, F, a.q);
-                else int_path_f32<D, NP, false, PAIR_SMEM>(r, xs, ps, pt, a.acc_pair, s, a.M, lane, F, a.q);
-            });
+        switch (sg.D) {
+            QTS_CASE(20) QTS_CASE(24) QTS_CASE(28) QTS_CASE(32)
+            default: break;
+        }
     }
+#undef QTS_CASE
     if (!ok) return;
     // flush: consecutive threads take consecutive samples of one row, so the
     // FP64 adds into the [row][sample] accumulators are coalesced
@@ -242,49 +302,47 @@ __global__ void __launch_bounds__(256) int_kernel(IntArgs a) {
     }
 }
 
-template <int D, int NP, bool PS>
-static cudaError_t launch_int_t(const IntArgs& a, int warps, int64_t blocks, size_t smem, cudaStream_t st) {
-    auto k = int_kernel<D, NP, PS>;
+template <int CLS, int NP, bool PS>
+static cudaError_t launch_int_t(const IntArgs& a, int64_t blocks, size_t smem, cudaStream_t st) {
+    auto k = int_kernel<CLS, NP, PS>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k<<<(unsigned)blocks, warps * 32, smem, st>>>(a);
+    k<<<(unsigned)blocks, kIntWarps * 32, smem, st>>>(a);
     return cudaGetLastError();
 }
 
-// np: nodes per register pass, int_max_np(D), or 4 for widths up to 6 (a
-// rule of four points)
-template <int D>
-cudaError_t launch_int_d(const IntArgs& a, int np, bool pair_smem, int warps, int64_t blocks, size_t smem,
-                         cudaStream_t st) {
-    constexpr int NP = int_max_np(D);
+// np: nodes per register pass, int_max_np of the class's widths, or 4 for widths
+// up to 6 (a rule of four points)
+template <int CLS>
+cudaError_t launch_int_c(const IntArgs& a, int np, bool pair_smem, int64_t blocks, size_t smem, cudaStream_t st) {
+    constexpr int NP = CLS <= 1 ? 8 : CLS == 2 ? 4 : 2;
     if constexpr (NP == 8) {
         if (np < NP) {
-            if (pair_smem) return launch_int_t<D, NP / 2, true>(a, warps, blocks, smem, st);
-            return launch_int_t<D, NP / 2, false>(a, warps, blocks, smem, st);
+            if (pair_smem) return launch_int_t<CLS, NP / 2, true>(a, blocks, smem, st);
+            return launch_int_t<CLS, NP / 2, false>(a, blocks, smem, st);
         }
     }
-    if (pair_smem) return launch_int_t<D, NP, true>(a, warps, blocks, smem, st);
-    return launch_int_t<D, NP, false>(a, warps, blocks, smem, st);
+    if (pair_smem) return launch_int_t<CLS, NP, true>(a, blocks, smem, st);
+    return launch_int_t<CLS, NP, false>(a, blocks, smem, st);
 }
 
-#define QTS_INST(DD) \
-    template cudaError_t launch_int_d<DD>(const IntArgs&, int, bool, int, int64_t, size_t, cudaStream_t);
+#define QTS_INST(C) template cudaError_t launch_int_c<C>(const IntArgs&, int, bool, int64_t, size_t, cudaStream_t);
 #if QTS_IN_PART(1)
-QTS_INST(32)
+QTS_INST(0)
 #endif
 #if QTS_IN_PART(2)
-QTS_INST(28)
+QTS_INST(1)
 #endif
 #if QTS_IN_PART(3)
-QTS_INST(24) QTS_INST(1) QTS_INST(2) QTS_INST(3) QTS_INST(4) QTS_INST(5) QTS_INST(6) QTS_INST(7) QTS_INST(8)
+QTS_INST(2)
 #endif
 #if QTS_IN_PART(4)
-QTS_INST(20) QTS_INST(9) QTS_INST(10) QTS_INST(11) QTS_INST(12)
+QTS_INST(3)
 #endif
 #if QTS_IN_PART(5)
-QTS_INST(13) QTS_INST(14) QTS_INST(15) QTS_INST(16)
+QTS_INST(4)
 #endif
 #undef QTS_INST
 
@@ -296,14 +354,12 @@ QTS_INST(13) QTS_INST(14) QTS_INST(15) QTS_INST(16)
 
 #if QTS_HOST_PART
 
-size_t int_smem_bytes(int F, int sub, int D, bool pair_smem) {
+static size_t int_smem_bytes(int F, int stage, bool pair_smem) {
     const size_t rows = F + 1;
     size_t off = 2 * rows * kTileLd * 4;
     if (pair_smem) off += (size_t)F * (F - 1) / 2 * kTileLd * 4;
     off = (off + 15) & ~(size_t)15;
-    off += 2 * (size_t)sub * (D + 1) * sizeof(Rec32);
-    off = (off + 15) & ~(size_t)15;
-    return off + 16;
+    return off + 2 * (size_t)stage * sizeof(Rec32) + 16;
 }
 
 // out[s][i][j] (F+1 x F+1, fp32) from the FP64 accumulators; one thread per (s, i).
@@ -335,49 +391,75 @@ __global__ void int_finalize_kernel(const double* __restrict__ acc_pair, const d
 
 static constexpr size_t kSmemBudget = 200 * 1024;
 
-cudaError_t launch_int_bucket(const qts_ensemble* e, const Bucket& b, bool pairs, const float* X, int64_t M,
-                              int F, const QuadF& q, double* acc_pair, double* acc_phi, cudaStream_t st) {
-    if (M <= 0 || b.n_paths == 0) return cudaSuccess;
-    IntArgs a;
-    // pairs: the sibling-pair tables (the bucket is one of e->bprep's)
-    a.rec = (pairs ? (const Rec32*)e->bdev.rec : (const Rec32*)e->d_rec) + b.rec_off;
-    a.n_paths = b.n_paths;
-    a.sub = b.D <= 16 ? 16 : 8;
-    // wide inputs: stage fewer paths at a time until the block fits shared memory
-    while (a.sub > 1 && int_smem_bytes(F, a.sub, b.D, false) > kSmemMax) a.sub /= 2;
-    a.group = M <= kFewRows ? (int)(32 / M) : 0;
-    a.paths_per_block = std::max<int64_t>(a.sub, 512 / a.sub * a.sub);
-    if (a.group) a.paths_per_block = std::max<int64_t>(a.paths_per_block, 4LL * 4 * a.group);
-    a.n_tiles = (int)((M + 31) / 32);
-    a.X = X;
-    a.M = M;
-    a.F = F;
-    a.cat = (pairs ? e->bprep.has_cat : e->prep.has_cat) ? 1 : 0;
-    a.n_pairs = (int64_t)F * (F - 1) / 2;
-    a.acc_pair = acc_pair;
-    a.acc_phi = acc_phi;
-    a.status = e->d_status;
-    a.q = q;
-    bool pair_smem = int_smem_bytes(F, a.sub, b.D, true) <= kSmemBudget;
-    const size_t smem = int_smem_bytes(F, a.sub, b.D, pair_smem);
-    if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
-    const int64_t chunks = (b.n_paths + a.paths_per_block - 1) / a.paths_per_block;
-    const int64_t blocks = chunks * a.n_tiles;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    const int warps = 4;
-    // nodes per register pass: the width's widest, or half of it when that
-    // does not divide the rule's padded node count
-    const int np = q.n_pad % int_max_np(b.D) == 0 ? int_max_np(b.D) : int_max_np(b.D) / 2;
-    if (q.n_pad % np != 0) return cudaErrorInvalidValue;
-    switch (b.D) {
-#define QTS_CASE(DD) \
-    case DD: return launch_int_d<DD>(a, np, pair_smem, warps, blocks, smem, st);
-        QTS_CASE(1) QTS_CASE(2) QTS_CASE(3) QTS_CASE(4) QTS_CASE(5) QTS_CASE(6) QTS_CASE(7)
-        QTS_CASE(8) QTS_CASE(9) QTS_CASE(10) QTS_CASE(11) QTS_CASE(12) QTS_CASE(13) QTS_CASE(14)
-        QTS_CASE(15) QTS_CASE(16) QTS_CASE(20) QTS_CASE(24) QTS_CASE(28) QTS_CASE(32)
-#undef QTS_CASE
-        default: return cudaErrorInvalidValue;
+// Pairwise sums of every bucket of the sibling-pair tables (pairs) or the per-leaf
+// tables; nq: points per bucket width, or one rule of nq_all points.
+cudaError_t launch_int_buckets(const qts_ensemble* e, bool pairs, const float* X, int64_t M, int F, int n_quad,
+                               int nq_all, double* acc_pair, double* acc_phi, cudaStream_t st) {
+    if (M <= 0) return cudaSuccess;
+    const Prepared& P = pairs ? e->bprep : e->prep;
+    const Rec32* rec = pairs ? (const Rec32*)e->bdev.rec : (const Rec32*)e->d_rec;
+    const int64_t tiles = (M + 31) / 32;
+    const int group = M <= kFewRows ? (int)(32 / M) : 0;
+    // work per thread block: about eight rounds of the whole chip (three thread
+    // blocks per SM); at least what makes the pair tile's set-up and flush, F^2 / 2
+    // rows, small beside the paths'
+    double total = 0.0;
+    for (const Bucket& b : P.buckets) total += (double)b.n_paths * b.D * (b.D + 8);
+    const double least = std::min(512.0, 64.0 + (double)F * F / 8.0) * 60.0;
+    const double share = std::max(least, std::min(512.0 * 84.0, total * (double)tiles / (8.0 * 3 * num_sms())));
+    for (int cls = 0; cls < kIntClasses; ++cls) {
+        for (int nq = QTS_MAX_QUAD; nq >= 1; --nq) {  // one launch per rule of the class
+            IntArgs a;
+            a.n_seg = 0;
+            int64_t ctas = 0;
+            int max_d = 0;
+            // widest first: its thread blocks are the longest
+            for (auto it = P.buckets.rbegin(); it != P.buckets.rend(); ++it) {
+                const Bucket& b = *it;
+                if (b.n_paths == 0 || int_class(b.D) != cls) continue;
+                if ((nq_all > 0 ? nq_all : nodes_for(n_quad, b.D, 1)) != nq) continue;
+                max_d = std::max(max_d, b.D);
+                int64_t per = std::max<int64_t>(16, (int64_t)(share / (b.D * (b.D + 8))));
+                if (group) per = std::max<int64_t>(per, 4LL * kIntWarps * group);
+                per = std::min<int64_t>((per + 15) / 16 * 16, 1 << 20);
+                a.seg[a.n_seg++] = {rec + b.rec_off, b.n_paths, ctas, (int32_t)per, b.D};
+                ctas += (b.n_paths + per - 1) / per * tiles;
+            }
+            if (a.n_seg == 0) continue;
+            if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+            // the rule, padded to 4 nodes up to width 12 (a pass of 4 or 8 nodes) and to
+            // 2 above
+            if (!make_quad(nq, &a.q, nullptr, cls <= 2 ? 4 : 2)) return cudaErrorInvalidValue;
+            a.sub = max_d <= 16 ? 16 : 8;
+            // wide inputs: stage fewer paths at a time until the block fits shared memory
+            while (a.sub > 1 && int_smem_bytes(F, a.sub * (max_d + 1), false) > kSmemMax) a.sub /= 2;
+            a.stage = a.sub * (max_d + 1);
+            a.n_tiles = (int)tiles;
+            a.X = X;
+            a.M = M;
+            a.F = F;
+            a.cat = P.has_cat ? 1 : 0;
+            a.n_pairs = (int64_t)F * (F - 1) / 2;
+            a.group = group;
+            a.acc_pair = acc_pair;
+            a.acc_phi = acc_phi;
+            a.status = e->d_status;
+            const bool pair_smem = int_smem_bytes(F, a.stage, true) <= kSmemBudget;
+            const size_t smem = int_smem_bytes(F, a.stage, pair_smem);
+            if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
+            // nodes per register pass: the class's widest, or half of it when that
+            // does not divide the rule's padded node count
+            const int np = a.q.n_pad % int_max_np(max_d) == 0 ? int_max_np(max_d) : int_max_np(max_d) / 2;
+            if (a.q.n_pad % np != 0) return cudaErrorInvalidValue;
+            const cudaError_t r = cls == 0   ? launch_int_c<0>(a, np, pair_smem, ctas, smem, st)
+                                  : cls == 1 ? launch_int_c<1>(a, np, pair_smem, ctas, smem, st)
+                                  : cls == 2 ? launch_int_c<2>(a, np, pair_smem, ctas, smem, st)
+                                  : cls == 3 ? launch_int_c<3>(a, np, pair_smem, ctas, smem, st)
+                                             : launch_int_c<4>(a, np, pair_smem, ctas, smem, st);
+            if (r != cudaSuccess) return r;
+        }
     }
+    return cudaSuccess;
 }
 
 cudaError_t launch_int_finalize(const double* acc_pair, const double* acc_phi, int64_t M, int F,
@@ -415,17 +497,11 @@ extern "C" qts_status qts_shap_interactions(qts_ensemble* e, const float* X, int
     double* acc_phi = acc_pair + n_pairs * M;
     cudaError_t ce = cudaMemsetAsync(e->d_work, 0, bytes, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "workspace clear");
-    for (const Bucket& b : e->bprep.buckets) {
-        // the bucket's rule, padded to 4 nodes up to width 12 (a pass of 4 or 8
-        // nodes) and to 2 above.  QTS_NQ_EXACT: the pair terms need
-        // ceil((D - 1) / 2) points, but the diagonal holds first-order values,
-        // so the kernel takes the first-order count ceil(D / 2) (Thm 2)
-        QuadF qf;
-        if (!make_quad(nodes_for(n_quad, b.D, 1), &qf, nullptr, b.D <= 12 ? 4 : 2))
-            return fail(QTS_ERR_ARG, "quadrature rule");
-        ce = launch_int_bucket(e, b, true, X, M, F, qf, acc_pair, acc_phi, s);
-        if (ce != cudaSuccess) return cuda_fail(ce, "interaction kernel launch");
-    }
+    // QTS_NQ_EXACT: the pair terms need ceil((D - 1) / 2) points, but the diagonal
+    // holds first-order values, so a bucket takes the first-order count ceil(D / 2)
+    // (Thm 2)
+    ce = launch_int_buckets(e, true, X, M, F, n_quad, 0, acc_pair, acc_phi, s);
+    if (ce != cudaSuccess) return cuda_fail(ce, "interaction kernel launch");
     ce = launch_int_finalize(acc_pair, acc_phi, M, F, e->bprep.bias, phi_ij, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction finalize launch");
     return QTS_OK;
@@ -528,9 +604,8 @@ extern "C" qts_status qts_shap_interactions_noalloc(qts_ensemble* e, const float
     cudaStream_t s = (cudaStream_t)stream;
     // QTS_NQ_EXACT: exact for the ensemble's widest path; first-order count,
     // because the diagonal holds first-order values (Thm 2)
-    QuadF qf;
-    if (!make_quad(nodes_for(n_quad, e->prep.max_unique, 1), &qf, nullptr))
-        return fail(QTS_ERR_ARG, "quadrature rule");
+    const int nq = nodes_for(n_quad, std::max(1, e->prep.max_unique), 1);
+    if (nq < 1 || nq > QTS_MAX_QUAD) return fail(QTS_ERR_ARG, "quadrature rule");
     void* scratch = nullptr;
     st = noalloc_scratch(&scratch);
     if (st != QTS_OK) return st;
@@ -539,10 +614,8 @@ extern "C" qts_status qts_shap_interactions_noalloc(qts_ensemble* e, const float
     // the array keeps the previous call's sums: clear the part this call uses
     cudaError_t ce = cudaMemsetAsync(scratch, 0, sizeof(double) * (size_t)need, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "scratch clear");
-    for (const Bucket& b : e->prep.buckets) {
-        ce = launch_int_bucket(e, b, false, X, M, F, qf, acc_pair, acc_phi, s);
-        if (ce != cudaSuccess) return cuda_fail(ce, "interaction kernel launch");
-    }
+    ce = launch_int_buckets(e, false, X, M, F, n_quad, nq, acc_pair, acc_phi, s);
+    if (ce != cudaSuccess) return cuda_fail(ce, "interaction kernel launch");
     ce = launch_int_finalize(acc_pair, acc_phi, M, F, e->prep.bias, phi_ij, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction finalize launch");
     return QTS_OK;

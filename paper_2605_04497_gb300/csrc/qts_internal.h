@@ -298,10 +298,6 @@ cudaError_t launch_fwd_few(const qts_ensemble* e, const float* X, int64_t M, int
                            cudaStream_t st);
 cudaError_t launch_fwd64(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* phi,
                          cudaStream_t st);
-// pairs: b is a bucket of the sibling-pair tables (e->bprep), else of e->prep
-cudaError_t launch_int_bucket(const qts_ensemble* e, const Bucket& b, bool pairs, const float* X, int64_t M,
-                              int F, const QuadF& q, double* acc_pair, double* acc_phi,
-                              cudaStream_t st);
 cudaError_t launch_int_finalize(const double* acc_pair, const double* acc_phi, int64_t M, int F,
                                 double bias, float* out, cudaStream_t st);
 // FP32 adjoint of one request (workspace: adjoint_work_bytes, block tables with grad)
