@@ -5,12 +5,12 @@
 // blocks of one bucket at a time, which all have the same shape, so its lanes
 // stay together.  Each lane reads its own block's records from global memory
 // (the loads of a block are independent of each other), and phi goes to one
-// shared tile with atomics.  All buckets of a register class are one launch.
+// shared tile with atomics.  All buckets of a class of widths are one launch.
 //
 // Bound by latency: 300 trees of depth 8 (71,759 leaves, F = 50), one row: 113 us
-// as one launch per path width on the path tables, 38 us here (of which the kernel is a third).
+// as one launch per path width on the path tables, 38 us with three classes of widths, 35 us here (the host's part is most of it).
 //
-// qts-build-parts: 6 (part 0: host code; parts 1-5: one register class each)
+// qts-build-parts: 4 (part 0: host code; parts 1-3: one class of widths each)
 #include <algorithm>
 
 #include "qts_blocks.cuh"
@@ -40,8 +40,8 @@ struct FewArgs {
     double* phi;
 };
 
-__host__ __device__ constexpr int few_class(int D) { return D <= 5 ? 0 : D <= 8 ? 1 : D <= 12 ? 2 : D <= 16 ? 3 : 4; }
-[[maybe_unused]] constexpr int kFewClasses = 5;
+__host__ __device__ constexpr int few_class(int D) { return D <= 8 ? 0 : D <= 16 ? 1 : 2; }
+[[maybe_unused]] constexpr int kFewClasses = 3;
 
 template <int CLS>
 cudaError_t launch_few(const FewArgs& a, int64_t ctas, size_t smem, cudaStream_t st);
@@ -97,22 +97,12 @@ __global__ void __launch_bounds__(kFewWarps * 32) few_kernel(const __grid_consta
     case DD: few_segment<DD>(a, sg, p0, p1, xs, ps); break;
     if constexpr (CLS == 0) {
         switch (sg.D) {
-            QTS_CASE(0) QTS_CASE(1) QTS_CASE(2) QTS_CASE(3) QTS_CASE(4) QTS_CASE(5)
+            QTS_CASE(0) QTS_CASE(1) QTS_CASE(2) QTS_CASE(3) QTS_CASE(4) QTS_CASE(5) QTS_CASE(6) QTS_CASE(7) QTS_CASE(8)
             default: break;
         }
     } else if constexpr (CLS == 1) {
         switch (sg.D) {
-            QTS_CASE(6) QTS_CASE(7) QTS_CASE(8)
-            default: break;
-        }
-    } else if constexpr (CLS == 2) {
-        switch (sg.D) {
-            QTS_CASE(9) QTS_CASE(10) QTS_CASE(11) QTS_CASE(12)
-            default: break;
-        }
-    } else if constexpr (CLS == 3) {
-        switch (sg.D) {
-            QTS_CASE(13) QTS_CASE(14) QTS_CASE(15) QTS_CASE(16)
+            QTS_CASE(9) QTS_CASE(10) QTS_CASE(11) QTS_CASE(12) QTS_CASE(13) QTS_CASE(14) QTS_CASE(15) QTS_CASE(16)
             default: break;
         }
     } else {
@@ -151,12 +141,6 @@ QTS_INST(1)
 #if QTS_IN_PART(3)
 QTS_INST(2)
 #endif
-#if QTS_IN_PART(4)
-QTS_INST(3)
-#endif
-#if QTS_IN_PART(5)
-QTS_INST(4)
-#endif
 #undef QTS_INST
 
 #endif  // QTS_DEVICE_PARTS
@@ -187,9 +171,7 @@ cudaError_t launch_fwd_few(const qts_ensemble* e, const float* X, int64_t M, int
                 if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
                 const cudaError_t r = cls == 0   ? launch_few<0>(a, ctas, smem, st)
                                       : cls == 1 ? launch_few<1>(a, ctas, smem, st)
-                                      : cls == 2 ? launch_few<2>(a, ctas, smem, st)
-                                      : cls == 3 ? launch_few<3>(a, ctas, smem, st)
-                                                 : launch_few<4>(a, ctas, smem, st);
+                                                 : launch_few<2>(a, ctas, smem, st);
                 a.n_seg = 0;
                 ctas = 0;
                 return r;
