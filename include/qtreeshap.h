@@ -138,8 +138,8 @@ qts_status qts_load_ensemble_cat(int32_t n_trees, const int64_t *tree_node_offse
 /*
  * qts_update_params - replace edge weights and leaf values (same topology) and
  * rebuild the path tables (Sec. 2).  z, leaf_value: host, one entry per node.
- * Synchronous.  The sibling-pair tables of the FP32 calls are dropped and built
- * again on the next call that needs them.  Errors as qts_load_ensemble.
+ * Synchronous.  The block tables of the first-order, adjoint, batched and pairwise
+ * calls are dropped and built again on the next call that needs them.  Errors as qts_load_ensemble.
  */
 qts_status qts_update_params(qts_ensemble *ens, const float *z, const float *leaf_value);
 
@@ -149,19 +149,18 @@ qts_status qts_update_params(qts_ensemble *ens, const float *z, const float *lea
  *   X       device, M x F fp32 row-major
  *   M       samples (>= 0; 0 is a no-op), F must equal the ensemble's n_features
  *   n_quad  Gauss-Legendre points, 1..QTS_MAX_QUAD (8 is the fast path), or
- *           QTS_NQ_EXACT: ceil(w / 2) points for the paths of width w
+ *           QTS_NQ_EXACT: the fewest points that Thm 2 makes exact, per bucket
  *   phi     device, M x (F+1) fp64, overwritten; phi[s][F] = E[f] = sum_v R_empty^v
  *           (the bias, so that sum_f phi[s][f] = f(x_s))
  * Per-path arithmetic is FP32 (FP64 with QTS_FLAG_FP64); contributions are
- * accumulated in FP32 over at most a few thousand paths, then in FP64 across
- * path chunks and trees.  With M <= 16 lanes are (path, sample) pairs instead
- * of one sample per lane.
- * FP32 ensembles run on a second set of path tables in which each pair of
- * sibling leaves of a numerical split is one path (see qts_get_batch_info);
- * it is built by the first FP32 forward, adjoint or batched call (host
- * preparation, cudaMalloc and synchronous copies, about 60% more device memory
- * than the per-leaf tables), so that first call must not be inside a stream
- * capture; later calls only enqueue on `stream`.
+ * accumulated in FP32 (FP64) within a thread block, then in FP64 across thread
+ * blocks.  With M <= 16 lanes are (block, sample) pairs instead of one sample per
+ * lane.
+ * Runs on a second set of tables in which a small subtree's leaves (up to
+ * eight) are evaluated together against the merged elements they share; it is
+ * built by the first call that needs it (host preparation, cudaMalloc and
+ * synchronous copies), so that first call must not be inside a stream capture;
+ * later calls only enqueue on `stream`.
  */
 qts_status qts_shap_values(qts_ensemble *ens, const float *X, int64_t M, int32_t F,
                            int32_t n_quad, double *phi, qts_stream_t stream);
@@ -201,12 +200,11 @@ qts_status qts_shap_values_alg1(qts_ensemble *ens, const float *X, int64_t M, in
  *           [s][F][F] = E[f], other entries of row/column F are 0.
  * Cross-tree accumulation is FP64 in the ensemble's workspace (device memory
  * of M * (F(F+1)/2) doubles, grown on demand with cudaMalloc).  Runs on the
- * sibling-pair tables of qts_shap_values (each pair's element is one more
- * linear factor of every pair term; built by the first call that needs them,
- * so that call must not be inside a stream capture).  n_quad as
- * qts_shap_values; QTS_NQ_EXACT takes ceil(D / 2) points per bucket of width
- * D (the pair terms need ceil((D - 1) / 2), the diagonal's first-order values
- * ceil(D / 2)).
+ * block tables of qts_shap_values (built by the first call that needs them, so
+ * that call must not be inside a stream capture).  n_quad as qts_shap_values;
+ * QTS_NQ_EXACT takes the first-order count ceil(w / 2) of a bucket's widest path
+ * w (the pair terms need ceil((w - 1) / 2), the diagonal's first-order values
+ * ceil(w / 2)).
  */
 qts_status qts_shap_interactions(qts_ensemble *ens, const float *X, int64_t M, int32_t F,
                                  int32_t n_quad, float *phi_ij, qts_stream_t stream);
@@ -263,7 +261,7 @@ qts_status qts_shap_interactions_order(qts_ensemble *ens, const float *X, int64_
  * ensembles) race and give wrong results: serialise all calls on a device
  * across the process, not per ensemble.  Arguments and output layout as
  * qts_shap_interactions; it runs on the per-leaf path tables (building the
- * sibling-pair tables would allocate), so its sums match
+ * block tables would allocate), so its sums match
  * qts_shap_interactions' to rounding, not bit for bit.
  */
 qts_status qts_shap_interactions_noalloc(qts_ensemble *ens, const float *X, int64_t M, int32_t F,
@@ -279,8 +277,10 @@ qts_status qts_shap_interactions_noalloc(qts_ensemble *ens, const float *X, int6
  * shap_as_weighted_banzhafs with the same n_quad rule, recomputing per-path
  * products instead of storing them.
  *   grad_phi device, M x (F+1) fp32 (column F weights the bias E[f]).
- * FP32 ensembles run on the sibling-pair tables (built on first use, as for
- * qts_shap_values); a pair's dL/dval is split over its two leaves exactly.
+ * FP32 ensembles run on the block tables (built on first use, as for
+ * qts_shap_values) with the batched pass's kernels; the workspace holds transposed
+ * copies of X and grad_phi (a captured call that would have to grow it takes that
+ * memory from the captured graph instead).
  */
 qts_status qts_shap_backward(qts_ensemble *ens, const float *X, int64_t M, int32_t F,
                              int32_t n_quad, const float *grad_phi, double *d_leaf, double *d_z,
@@ -300,16 +300,15 @@ typedef struct qts_request {
 
 /*
  * qts_batched_fwd_bwd - forward (and, where grad_phi is given, backward) of many
- * heterogeneous requests in ONE persistent kernel launch: a device work list of
- * (request, path bucket, path chunk, sample tile) items sorted by cost is
- * consumed through an atomic counter, and one pass over each (sample, path)
- * produces both phi and the adjoint (the forward product terms are a subset of
- * the adjoint's).  The whole call (initialisation, persistent kernel, adjoint
- * epilogue) is captured once into a CUDA graph keyed by the request set and
+ * heterogeneous requests in one persistent kernel per register class: a device
+ * work list of (request, block bucket, run of blocks, sample tile) items sorted by
+ * cost is consumed through an atomic counter, and one pass over each (sample,
+ * block) produces both phi and the adjoint (the forward product terms are a subset
+ * of the adjoint's).  The whole call (one preparation kernel, the persistent
+ * kernels as parallel branches, the adjoint epilogue) is captured once into a CUDA graph keyed by the request set and
  * replayed on later calls with the same requests.  Each ensemble may appear in
  * at most one request of a call.  FP32 ensembles only.  n_quad as
- * qts_shap_values; with QTS_NQ_EXACT every bucket takes ceil(D / 2) points for
- * its width D and the graph holds one persistent launch per (register class,
+ * qts_shap_values; the graph holds one persistent launch per (register class,
  * accumulator-tile size, rule).
  */
 qts_status qts_batched_fwd_bwd(int32_t n_requests, const qts_request *reqs, int32_t n_quad,
@@ -318,16 +317,12 @@ qts_status qts_batched_fwd_bwd(int32_t n_requests, const qts_request *reqs, int3
 /*
  * qts_batched_autotune - pick the batched launch's per-width parameters for a
  * set of requests by timing its persistent kernel on the requests' own data (the
- * autotuner of the batched form; the paper has no batching).  For every bucket
- * width that carries at least 1% of the batch's work it times, with that
- * width's work items alone in the launch, the paths per work item (one, two,
- * four and eight times the default, at most 4,096) and, where the fused pass
- * packs two samples per lane,
- * the sample mapping (each warp its own 64 samples, or the block's warps sharing
- * 64 samples and splitting the paths), and keeps the fastest.  Then, for the
- * register classes of widths 1-6 and 7-10 (four and three blocks per SM), it
- * times the class's launch with all blocks that fit and with one fewer, which
- * leaves more of the SM's shared memory to L1, and keeps the faster.  The
+ * autotuner of the batched form; the paper has no batching).  For every block
+ * width (shared elements) that carries at least 1% of the batch's work it times,
+ * with that width's work items alone in the launch, 64, 256, 1,024 and 2,048 blocks
+ * per work item and, where the pass holds two samples per lane, the sample mapping
+ * (each warp its own 64 samples, or the thread block's warps sharing 64 samples and
+ * splitting the blocks), and keeps the fastest.  The
  * choices are stored in each request's ensemble and used by later batched
  * calls that include it (their cached graphs are rebuilt).
  *   reqs, n, n_quad  as qts_batched_fwd_bwd; the requests' outputs are
@@ -335,21 +330,20 @@ qts_status qts_batched_fwd_bwd(int32_t n_requests, const qts_request *reqs, int3
  *   max_samples      time on the first min(M, max_samples) samples of each
  *                    request (0: all)
  *   chosen           host, 3 * (QTS_MAX_UNIQUE_FEATURES_PER_PATH + 1) int32 or
- *                    NULL: for width D, [3D] paths per item, [3D + 1] mapping
- *                    (2 or 3, 0 where not packed), [3D + 2] blocks per SM of
- *                    its class (0: all that fit); 0 for untuned widths
+ *                    NULL: for width D, [3D] blocks per item, [3D + 1] mapping
+ *                    (2 or 3, 0 where one sample per lane), [3D + 2] 0 (all
+ *                    thread blocks that fit an SM); 0 for untuned widths
  * Synchronous on `stream`.  Errors as qts_batched_fwd_bwd.
  */
 qts_status qts_batched_autotune(int32_t n_requests, const qts_request *reqs, int32_t n_quad,
                                 int64_t max_samples, int32_t *chosen, qts_stream_t stream);
 
 /*
- * qts_get_batch_info - size of the path tables the batched pass uses for this
- * ensemble (built on first use, as by a batched call).  These tables hold each
- * pair of sibling leaves of a numerical split as one path: the pair's combined
+ * qts_get_batch_info - size of the ensemble's path tables with each pair of
+ * sibling leaves of a numerical split counted as one path: the pair's combined
  * leaf polynomial val_A a_A(p) + val_B a_B(p) is linear in p, so it is one more
- * element of the shared path (exact algebra of Eq. shap_as_weighted_banzhafs;
- * the paper evaluates the two paths separately).
+ * element of the shared path.  (The kernels go further and evaluate whole small
+ * subtrees, see qts_shap_values.)  Host preparation on the first call.
  *   n_paths       paths, pairs counted once
  *   sum_unique    sum over paths of their unique features (the work unit)
  *   n_pair_paths  paths that stand for two leaves
@@ -361,6 +355,15 @@ qts_status qts_batched_autotune(int32_t n_requests, const qts_request *reqs, int
 qts_status qts_get_batch_info(qts_ensemble *ens, int64_t *n_paths, int64_t *sum_unique, int64_t *n_pair_paths,
                               int32_t *n_buckets, int32_t *bucket_width, int64_t *bucket_paths);
 
+/*
+ * qts_get_block_info - size of the block tables that the first-order, adjoint,
+ * batched and pairwise calls run on (built on first use): blocks, shared elements
+ * (with padding), inner nodes (two edges to subtrees each) and pair nodes (two
+ * leaves each) of all blocks.  Any output pointer may be NULL.
+ */
+qts_status qts_get_block_info(qts_ensemble *ens, int64_t *n_blocks, int64_t *elements, int64_t *inner_nodes,
+                              int64_t *pair_nodes);
+
 /* Number of kernels in the graph of the calling thread's last batched call. */
 int32_t qts_batched_kernel_count(void);
 
@@ -369,8 +372,8 @@ int32_t qts_batched_kernel_count(void);
 qts_status qts_batched_last_kernel_ms(float *ms);
 
 /*
- * qts_autotune - time candidate launch configurations (warps per block, paths
- * per chunk, node-group width) for this ensemble and sample count on `stream`,
+ * qts_autotune - time candidate launch configurations (work per thread block of
+ * the forward) for this ensemble and sample count on `stream`,
  * keep the fastest in the ensemble, and, if cache_path is not NULL, merge the
  * result into that JSON file keyed by (bucket width, F range, M range).
  * X: device M x F.  Synchronous.  Scratch output is allocated internally.
@@ -401,8 +404,8 @@ qts_status qts_get_info(const qts_ensemble *ens, qts_info *out);
  * preparation (Sec. 2 merging and bucketing): same arguments and checks, no
  * device memory is touched; fills `out` (device_bytes = the bytes an upload
  * would take).  Usable without a GPU.  With QTS_DESCRIBE_PAIRS in flags it
- * describes the tables of the batched pass instead (sibling leaves of a
- * numerical split as one path; see qts_get_batch_info).
+ * describes the tables with sibling leaves of a numerical split as one path
+ * instead (see qts_get_batch_info).
  */
 #define QTS_DESCRIBE_PAIRS 2u
 qts_status qts_describe_ensemble(int32_t n_trees, const int64_t *tree_node_offsets,

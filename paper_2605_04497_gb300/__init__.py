@@ -29,7 +29,7 @@ STATUS_NAMES = {0: "QTS_OK", 1: "QTS_ERR_ARG", 2: "QTS_ERR_CUDA", 3: "QTS_ERR_OO
 EXPORTS = ("qts_load_ensemble", "qts_load_ensemble_cat", "qts_update_params", "qts_shap_values", "qts_shap_values_alg1",
            "qts_shap_interactions",
            "qts_shap_interactions_noalloc", "qts_shap_interactions3", "qts_shap_interactions_order",
-           "qts_shap_backward", "qts_batched_fwd_bwd", "qts_batched_autotune", "qts_get_batch_info", "qts_autotune", "qts_sync_status",
+           "qts_shap_backward", "qts_batched_fwd_bwd", "qts_batched_autotune", "qts_get_batch_info", "qts_get_block_info", "qts_autotune", "qts_sync_status",
            "qts_get_info", "qts_describe_ensemble", "qts_describe_paths", "qts_describe_alg1_program", "qts_selftest_wait_timeout", "qts_batched_kernel_count", "qts_batched_last_kernel_ms", "qts_gauss_legendre", "qts_exact_nodes", "qts_fp32_pipe_peak", "qts_last_error",
            "qts_free")
 
@@ -84,6 +84,7 @@ def lib():
         L.qts_batched_fwd_bwd.argtypes = [i32, vp, i32, vp]
         L.qts_batched_autotune.argtypes = [i32, vp, i32, i64, vp, vp]
         L.qts_get_batch_info.argtypes = [vp, vp, vp, vp, vp, vp, vp]
+        L.qts_get_block_info.argtypes = [vp, vp, vp, vp, vp]
         L.qts_autotune.argtypes = [vp, vp, i64, i32, ctypes.c_char_p, vp]
         L.qts_sync_status.argtypes = [vp, vp]
         L.qts_selftest_wait_timeout.argtypes = [vp, vp]
@@ -157,8 +158,8 @@ def _info_dict(i: QtsInfo) -> dict:
 
 
 def describe(ens, fp64: bool = False, pairs: bool = False) -> dict:
-    """Host-only path preparation summary (no GPU needed); pairs: the tables of
-    the batched pass (sibling leaves merged)."""
+    """Host-only path preparation summary (no GPU needed); pairs: the tables
+    with sibling leaves merged."""
     arr = lambda a, dt: np.ascontiguousarray(a, dtype=dt)
     a = [arr(ens.node_offsets, np.int64), arr(ens.left, np.int32), arr(ens.right, np.int32),
          arr(ens.feature, np.int32), arr(ens.threshold, np.float32), arr(ens.default_left, np.uint8),
@@ -259,7 +260,7 @@ class Ensemble:
         return _info_dict(i)
 
     def batch_info(self) -> dict:
-        """Sizes of the tables the batched pass uses (sibling leaf pairs merged)."""
+        """Sizes of the path tables with sibling leaf pairs merged."""
         n, su, npair = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_int64()
         nb = ctypes.c_int32()
         bw = (ctypes.c_int32 * 32)()
@@ -268,6 +269,13 @@ class Ensemble:
                                         ctypes.byref(nb), bw, bp))
         return dict(n_paths=n.value, sum_unique=su.value, n_pair_paths=npair.value,
                     buckets=[(int(bw[i]), int(bp[i])) for i in range(nb.value)])
+
+    def block_info(self) -> dict:
+        """Sizes of the block tables the first-order, adjoint, batched and pairwise
+        calls run on: blocks, shared elements, inner and pair nodes of all blocks."""
+        v = [ctypes.c_int64() for _ in range(4)]
+        _check(lib().qts_get_block_info(self.handle, *[ctypes.byref(x) for x in v]))
+        return dict(zip(("n_blocks", "elements", "inner_nodes", "pair_nodes"), (x.value for x in v)))
 
     def sync_status(self, stream=None):
         _check(lib().qts_sync_status(self.handle, _stream(stream)))
@@ -440,8 +448,7 @@ def batched_fwd_bwd(reqs, n_quad: int = 8, stream=None):
 
 def batched_autotune(reqs, n_quad: int = 8, max_samples: int = 1024, stream=None) -> dict:
     """Tune the batched launch for these requests (see qts_batched_autotune);
-    returns {width: (paths per item, sample mapping, blocks per SM or 0)} for
-    the tuned widths."""
+    returns {width: (blocks per item, sample mapping, 0)} for the tuned widths."""
     n = 65  # QTS_MAX_UNIQUE_FEATURES_PER_PATH + 1
     chosen = np.zeros(3 * n, dtype=np.int32)
     _check(lib().qts_batched_autotune(len(reqs), ctypes.cast(reqs, ctypes.c_void_p), n_quad, max_samples,

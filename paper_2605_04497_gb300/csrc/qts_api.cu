@@ -69,19 +69,8 @@ void release_device(qts_ensemble* e) {
     e->d_empty_leaf = nullptr;
     e->device_bytes = 0;
     release_dfs(e);
-    release_batch_tables(e);
+    e->pair_ready = false;
     release_blocks(e);
-}
-
-void release_batch_tables(qts_ensemble* e) {
-    DevTables& T = e->bdev;
-    for (void* p : {T.rec, (void*)T.path_leaf, (void*)T.path_zprod, (void*)T.path_val, (void*)T.slot_zexcl,
-                    (void*)T.slot_edge_begin, (void*)T.edge_node, (void*)T.edge_coef, (void*)T.empty_leaf,
-                    (void*)T.pair_leaf2, (void*)T.pair_zprod2, (void*)T.pair_z, (void*)T.pair_gslot})
-        cudaFree(p);
-    T = DevTables();
-    e->bprep = Prepared();
-    e->bready = false;
 }
 
 template <typename T>
@@ -130,11 +119,11 @@ qts_status upload(qts_ensemble* e) {
     return QTS_OK;
 }
 
-// Pair tables of the batched pass: prepared from the host copy of the model
-// with sibling leaves merged, uploaded, host copies dropped.
-qts_status ensure_batch_tables(qts_ensemble* e) {
-    if (e->bready) return QTS_OK;
-    Prepared& P = e->bprep;
+// Sizes of the path tables with sibling leaves merged (qts_get_batch_info): prepared
+// from the host copy of the model, nothing is kept but the counts.
+qts_status ensure_pair_sizes(qts_ensemble* e) {
+    if (e->pair_ready) return QTS_OK;
+    Prepared P;
     std::string err;
     const bool cat = !e->is_cat.empty();
     qts_status st = prepare(e->n_trees, e->off.data(), e->left.data(), e->right.data(), e->feature.data(),
@@ -142,32 +131,11 @@ qts_status ensure_batch_tables(qts_ensemble* e) {
                             cat ? e->is_cat.data() : nullptr, cat ? e->cat_left.data() : nullptr,
                             e->n_features, false, &P, &err, true);
     if (st != QTS_OK) return fail(st, err);
-    DevTables& T = e->bdev;
-    int64_t tot = 0;
-    st = up((Rec32**)&T.rec, P.rec32, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.path_leaf, P.path_leaf, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.path_zprod, P.path_zprod, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.path_val, P.path_val, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.slot_zexcl, P.slot_zexcl, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.slot_edge_begin, P.slot_edge_begin, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.edge_node, P.edge_node, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.edge_coef, P.edge_coef, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.empty_leaf, P.empty_leaf, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.pair_leaf2, P.pair_leaf2, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.pair_zprod2, P.pair_zprod2, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.pair_z, P.pair_z, &tot, "upload pair tables");
-    if (st == QTS_OK) st = up(&T.pair_gslot, P.pair_gslot, &tot, "upload pair tables");
-    if (st != QTS_OK) {
-        release_batch_tables(e);
-        return st;
-    }
-    T.bytes = tot;
-    for (auto* v : {&P.path_zprod, &P.path_val, &P.slot_zexcl, &P.edge_coef, &P.pair_zprod2, &P.pair_z})
-        std::vector<double>().swap(*v);
-    for (auto* v : {&P.path_leaf, &P.slot_edge_begin, &P.edge_node, &P.pair_leaf2, &P.pair_gslot})
-        std::vector<int64_t>().swap(*v);
-    std::vector<Rec32>().swap(P.rec32);
-    e->bready = true;
+    e->pair_sizes.buckets = P.buckets;
+    e->pair_sizes.n_paths = P.n_paths;
+    e->pair_sizes.sum_unique = P.sum_unique;
+    e->pair_sizes.n_pair_paths = P.n_pair_paths;
+    e->pair_ready = true;
     return QTS_OK;
 }
 

@@ -309,9 +309,25 @@ extern "C" qts_status qts_shap_backward(qts_ensemble* e, const float* X, int64_t
         // FP32: the block tables and the batched pass's kernels
         st = ensure_blocks(e, true);
         if (st != QTS_OK) return st;
-        st = ensure_workspace(e, adjoint_work_bytes(e, M, F));
-        if (st != QTS_OK) return st;
-        ce = launch_adjoint_blocks(e, X, grad_phi, M, F, n_quad, d_leaf, d_z, s);
+        // The workspace holds the samples' transposed copies, so it grows with M.
+        // A stream capture must not grow it: there a call that needs more takes
+        // memory of the captured graph's own.
+        const size_t need = adjoint_work_bytes(e, M, F);
+        void* own = nullptr;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (need > e->work_bytes && cudaStreamIsCapturing(s, &cap) == cudaSuccess &&
+            cap == cudaStreamCaptureStatusActive) {
+            ce = cudaMallocAsync(&own, need, s);
+            if (ce != cudaSuccess) return cuda_fail(ce, "adjoint workspace");
+        } else {
+            st = ensure_workspace(e, need);
+            if (st != QTS_OK) return st;
+        }
+        ce = launch_adjoint_blocks(e, own ? own : e->d_work, X, grad_phi, M, F, n_quad, d_leaf, d_z, s);
+        if (own) {
+            const cudaError_t fe = cudaFreeAsync(own, s);
+            if (ce == cudaSuccess) ce = fe;
+        }
         return ce == cudaSuccess ? QTS_OK : cuda_fail(ce, "adjoint kernel launch");
     }
     const Prepared& P = e->prep;

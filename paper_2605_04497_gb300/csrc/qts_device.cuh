@@ -233,7 +233,7 @@ __device__ __forceinline__ void walk_paths_grouped(const Rec* __restrict__ rec, 
 
 // Transposed tile of 32 rows of a row-major matrix: tile[c * kTileLd + s] =
 // A[(s0 + s) * ld + c] for c < ncols (0 beyond M), plus `extra` zero rows.
-// Returns (block-wide) whether any loaded value is NaN.
+// Returns (block-wide) whether any loaded value is NaN or +inf.
 __device__ __forceinline__ bool load_tile_t(float* tile, const float* __restrict__ A, int64_t s0,
                                             int64_t M, int ncols, int64_t ld, int extra) {
     int nan_seen = 0;
@@ -241,7 +241,7 @@ __device__ __forceinline__ bool load_tile_t(float* tile, const float* __restrict
         const int s = idx / ncols, c = idx - s * ncols;
         const float v = (s0 + s < M) ? A[(s0 + s) * ld + c] : 0.f;
         tile[c * kTileLd + s] = v;
-        nan_seen |= (v != v);
+        nan_seen |= !(v < INFINITY);
     }
     for (int idx = threadIdx.x; idx < extra * kTileLd; idx += blockDim.x) tile[ncols * kTileLd + idx] = 0.f;
     return __syncthreads_or(nan_seen) != 0;
@@ -256,40 +256,13 @@ __device__ __forceinline__ bool load_tiles_t(float* tile, const float* __restric
         const int s = idx / ncols, c = idx - s * ncols;
         const float v = (s0 + s < M) ? A[(s0 + s) * ld + c] : 0.f;
         tile[(s >> 5) * tile_stride + c * kTileLd + (s & 31)] = v;
-        nan_seen |= (v != v);
+        nan_seen |= !(v < INFINITY);
     }
     for (int idx = threadIdx.x; idx < ntiles * extra * kTileLd; idx += blockDim.x) {
         const int w = idx / (extra * kTileLd), r = idx - w * extra * kTileLd;
         tile[w * tile_stride + ncols * kTileLd + r] = 0.f;
     }
     return __syncthreads_or(nan_seen) != 0;
-}
-
-// ------------------------------------------------------- sibling pairs --
-//
-// Pair tables (FP32 forward, adjoint, batched pass, pairwise interactions)
-// hold sibling leaves A, B of a numerical split as one path with val = 1 whose
-// last element e (kPairElem) stands for both: for a sample x it gives
-// d = val_k - alpha for the leaf k the sample reaches (x in the element's
-// interval, then left of theta), -alpha if neither.  h is the path header
-// {1, val_A - alpha, val_B - alpha, bits of theta}.
-__device__ __forceinline__ void pair_sides(float x, const Rec32& e, const Rec32& h, bool* oa, bool* ob) {
-    bool in, left;
-    if (x != x) {
-        in = (e.bits & kNanOk) != 0;
-        left = (e.bits & kDefLeft) != 0;
-    } else {
-        in = x >= e.lo && x < e.hi;
-        left = x < __uint_as_float(h.bits);
-    }
-    *oa = in && left;
-    *ob = in && !left;
-}
-
-__device__ __forceinline__ float pair_d(float x, const Rec32& e, const Rec32& h) {
-    bool oa, ob;
-    pair_sides(x, e, h, &oa, &ob);
-    return oa ? h.lo : (ob ? h.hi : -e.z);
 }
 
 }  // namespace qts

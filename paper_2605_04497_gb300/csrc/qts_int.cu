@@ -1,5 +1,8 @@
 // Pairwise Shapley interaction values (Thm 1 with S = {i, j}; Alg. 1 with
-// s = 2), in the pred_interactions layout.
+// s = 2), in the pred_interactions layout: the entry points, the finalize kernel,
+// and the path kernels of the allocation-free call.  qts_shap_interactions runs on
+// the block tables (qts_int_blocks.cu), which are built and allocated on first use;
+// the allocation-free call must not do that and keeps the per-leaf path tables.
 //
 // For a path with merged elements sorted by feature and a sample,
 //     SII_ij += val d_i d_j sum_m w_m prod_{k != i,j} a_k(t_m),   d = o - z,
@@ -14,10 +17,9 @@
 // [feature][sample]; a finalize kernel writes the (F+1) x (F+1) matrices.
 //
 // All widths of a register class and rule are one launch (a thread block finds
-// its segment by its index).  500 trees of depth 6 (31,449 leaves, F = 30), 2,000
-// samples: 1.78 ms with a launch per width of 512 paths per thread block, which left
-// most SMs idle on the narrow widths, 1.56 ms here.  Bound by the shared-memory
-// float atomics of the pair sums (compare-and-swap loops) at 12 warps per SM.
+// its segment by its index, and its paths follow from the call's work: one
+// launch per width of 512 paths per thread block left most SMs idle on narrow
+// widths; 500 trees of depth 6, 2,000 samples: 1.79 -> 1.56 ms).
 //
 // qts-build-parts: 6 (part 0: host code; parts 1-5: the kernels)
 #include <cuda.h>
@@ -88,10 +90,6 @@ __device__ __forceinline__ void int_path_f32(const Rec32* __restrict__ r, const 
                                              int64_t M, int lane, int F, const QuadF& q) {
     constexpr int K = NP / 2;
     const float val = r[0].z;
-    // a sibling pair (pair tables only): its element sits last, after the
-    // padding and out of feature order, with d = val_k - alpha per sample and
-    // val = 1 (the pair polynomial is one more linear factor of every term)
-    const bool pair = (r[D].bits & kPairElem) != 0;
     float dd[D], c1[D];
     int nreal = D;  // sorted elements before the padding (padding sorts last)
 #pragma unroll
@@ -101,11 +99,9 @@ __device__ __forceinline__ void int_path_f32(const Rec32* __restrict__ r, const 
         const float x = xs[f * kTileLd + lane];
         const bool o = satisfies<HAS_NAN>(x, e.lo, e.hi, e.bits);
         dd[j] = (o ? 1.f : 0.f) - e.z;
-        if (j == D - 1 && pair) dd[j] = pair_d(x, e, r[0]);
         c1[j] = 0.f;
         if (f >= F && j < nreal) nreal = j;
     }
-    if (pair && nreal > D - 1) nreal = D - 1;
     const int npass = q.n_pad / NP;
     for (int pass = 0; pass < npass; ++pass) {
         float2 T[K], A[D][K], P[D][K], S[D][K];
@@ -138,10 +134,10 @@ __device__ __forceinline__ void int_path_f32(const Rec32* __restrict__ r, const 
             for (int k = 1; k < K; ++k) a1 = fma2(P[j][k], S[j][k], a1);
             c1[j] += a1.x + a1.y;
         }
-        // pairs i < j among the sorted elements, then (i, pair element)
+        // pairs i < j
 #pragma unroll
         for (int i = 0; i < D - 1; ++i) {
-            if (i + (pair ? 0 : 1) >= nreal) break;
+            if (i + 1 >= nreal) break;
             const int fi = feat_of(r[1 + i].bits);
             const int64_t rowbase = tri_index(fi, fi + 1, F) - (fi + 1);  // + fj gives the index
             float2 R[K];
@@ -165,26 +161,11 @@ __device__ __forceinline__ void int_path_f32(const Rec32* __restrict__ r, const 
                     if (s < M && v != 0.f) atomicAdd(&acc_pair[idx * M + s], (double)v);
                 }
             }
-            if (pair) {
-                // R spans the elements between i and the pair element (padding
-                // factors are 1), and the pair element's suffix is 1
-                float2 acc = R[0];
-#pragma unroll
-                for (int k = 1; k < K; ++k) acc = add2(R[k], acc);
-                const float v = (acc.x + acc.y) * (dd[i] * dd[D - 1]);
-                const int fp = feat_of(r[D].bits);
-                const int64_t idx = fi < fp ? tri_index(fi, fp, F) : tri_index(fp, fi, F);
-                if constexpr (PAIR_SMEM) {
-                    atomicAdd(&pt[idx * kTileLd + lane], v);
-                } else {
-                    if (s < M && v != 0.f) atomicAdd(&acc_pair[idx * M + s], (double)v);
-                }
-            }
         }
     }
 #pragma unroll
     for (int j = 0; j < D; ++j)
-        if (j < nreal || (pair && j == D - 1))
+        if (j < nreal)
             atomicAdd(&ps[feat_of(r[1 + j].bits) * kTileLd + lane], dd[j] * c1[j]);
 }
 
@@ -391,13 +372,12 @@ __global__ void int_finalize_kernel(const double* __restrict__ acc_pair, const d
 
 static constexpr size_t kSmemBudget = 200 * 1024;
 
-// Pairwise sums of every bucket of the sibling-pair tables (pairs) or the per-leaf
-// tables; nq: points per bucket width, or one rule of nq_all points.
-cudaError_t launch_int_buckets(const qts_ensemble* e, bool pairs, const float* X, int64_t M, int F, int n_quad,
-                               int nq_all, double* acc_pair, double* acc_phi, cudaStream_t st) {
+// Pairwise sums of every bucket of the per-leaf tables with a rule of nq points.
+static cudaError_t launch_int_buckets(const qts_ensemble* e, const float* X, int64_t M, int F, int nq,
+                                      double* acc_pair, double* acc_phi, cudaStream_t st) {
     if (M <= 0) return cudaSuccess;
-    const Prepared& P = pairs ? e->bprep : e->prep;
-    const Rec32* rec = pairs ? (const Rec32*)e->bdev.rec : (const Rec32*)e->d_rec;
+    const Prepared& P = e->prep;
+    const Rec32* rec = (const Rec32*)e->d_rec;
     const int64_t tiles = (M + 31) / 32;
     const int group = M <= kFewRows ? (int)(32 / M) : 0;
     // work per thread block: about eight rounds of the whole chip (three thread
@@ -408,56 +388,53 @@ cudaError_t launch_int_buckets(const qts_ensemble* e, bool pairs, const float* X
     const double least = std::min(512.0, 64.0 + (double)F * F / 8.0) * 60.0;
     const double share = std::max(least, std::min(512.0 * 84.0, total * (double)tiles / (8.0 * 3 * num_sms())));
     for (int cls = 0; cls < kIntClasses; ++cls) {
-        for (int nq = QTS_MAX_QUAD; nq >= 1; --nq) {  // one launch per rule of the class
-            IntArgs a;
-            a.n_seg = 0;
-            int64_t ctas = 0;
-            int max_d = 0;
-            // widest first: its thread blocks are the longest
-            for (auto it = P.buckets.rbegin(); it != P.buckets.rend(); ++it) {
-                const Bucket& b = *it;
-                if (b.n_paths == 0 || int_class(b.D) != cls) continue;
-                if ((nq_all > 0 ? nq_all : nodes_for(n_quad, b.D, 1)) != nq) continue;
-                max_d = std::max(max_d, b.D);
-                int64_t per = std::max<int64_t>(16, (int64_t)(share / (b.D * (b.D + 8))));
-                if (group) per = std::max<int64_t>(per, 4LL * kIntWarps * group);
-                per = std::min<int64_t>((per + 15) / 16 * 16, 1 << 20);
-                a.seg[a.n_seg++] = {rec + b.rec_off, b.n_paths, ctas, (int32_t)per, b.D};
-                ctas += (b.n_paths + per - 1) / per * tiles;
-            }
-            if (a.n_seg == 0) continue;
-            if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-            // the rule, padded to 4 nodes up to width 12 (a pass of 4 or 8 nodes) and to
-            // 2 above
-            if (!make_quad(nq, &a.q, nullptr, cls <= 2 ? 4 : 2)) return cudaErrorInvalidValue;
-            a.sub = max_d <= 16 ? 16 : 8;
-            // wide inputs: stage fewer paths at a time until the block fits shared memory
-            while (a.sub > 1 && int_smem_bytes(F, a.sub * (max_d + 1), false) > kSmemMax) a.sub /= 2;
-            a.stage = a.sub * (max_d + 1);
-            a.n_tiles = (int)tiles;
-            a.X = X;
-            a.M = M;
-            a.F = F;
-            a.cat = P.has_cat ? 1 : 0;
-            a.n_pairs = (int64_t)F * (F - 1) / 2;
-            a.group = group;
-            a.acc_pair = acc_pair;
-            a.acc_phi = acc_phi;
-            a.status = e->d_status;
-            const bool pair_smem = int_smem_bytes(F, a.stage, true) <= kSmemBudget;
-            const size_t smem = int_smem_bytes(F, a.stage, pair_smem);
-            if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
-            // nodes per register pass: the class's widest, or half of it when that
-            // does not divide the rule's padded node count
-            const int np = a.q.n_pad % int_max_np(max_d) == 0 ? int_max_np(max_d) : int_max_np(max_d) / 2;
-            if (a.q.n_pad % np != 0) return cudaErrorInvalidValue;
-            const cudaError_t r = cls == 0   ? launch_int_c<0>(a, np, pair_smem, ctas, smem, st)
-                                  : cls == 1 ? launch_int_c<1>(a, np, pair_smem, ctas, smem, st)
-                                  : cls == 2 ? launch_int_c<2>(a, np, pair_smem, ctas, smem, st)
-                                  : cls == 3 ? launch_int_c<3>(a, np, pair_smem, ctas, smem, st)
-                                             : launch_int_c<4>(a, np, pair_smem, ctas, smem, st);
-            if (r != cudaSuccess) return r;
+        IntArgs a;
+        a.n_seg = 0;
+        int64_t ctas = 0;
+        int max_d = 0;
+        // widest first: its thread blocks are the longest
+        for (auto it = P.buckets.rbegin(); it != P.buckets.rend(); ++it) {
+            const Bucket& b = *it;
+            if (b.n_paths == 0 || int_class(b.D) != cls) continue;
+            max_d = std::max(max_d, b.D);
+            int64_t per = std::max<int64_t>(16, (int64_t)(share / (b.D * (b.D + 8))));
+            if (group) per = std::max<int64_t>(per, 4LL * kIntWarps * group);
+            per = std::min<int64_t>((per + 15) / 16 * 16, 1 << 20);
+            a.seg[a.n_seg++] = {rec + b.rec_off, b.n_paths, ctas, (int32_t)per, b.D};
+            ctas += (b.n_paths + per - 1) / per * tiles;
         }
+        if (a.n_seg == 0) continue;
+        if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        // the rule, padded to 4 nodes up to width 12 (a pass of 4 or 8 nodes) and to
+        // 2 above
+        if (!make_quad(nq, &a.q, nullptr, cls <= 2 ? 4 : 2)) return cudaErrorInvalidValue;
+        a.sub = max_d <= 16 ? 16 : 8;
+        // wide inputs: stage fewer paths at a time until the block fits shared memory
+        while (a.sub > 1 && int_smem_bytes(F, a.sub * (max_d + 1), false) > kSmemMax) a.sub /= 2;
+        a.stage = a.sub * (max_d + 1);
+        a.n_tiles = (int)tiles;
+        a.X = X;
+        a.M = M;
+        a.F = F;
+        a.cat = P.has_cat ? 1 : 0;
+        a.n_pairs = (int64_t)F * (F - 1) / 2;
+        a.group = group;
+        a.acc_pair = acc_pair;
+        a.acc_phi = acc_phi;
+        a.status = e->d_status;
+        const bool pair_smem = int_smem_bytes(F, a.stage, true) <= kSmemBudget;
+        const size_t smem = int_smem_bytes(F, a.stage, pair_smem);
+        if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
+        // nodes per register pass: the class's widest, or half of it when that
+        // does not divide the rule's padded node count
+        const int np = a.q.n_pad % int_max_np(max_d) == 0 ? int_max_np(max_d) : int_max_np(max_d) / 2;
+        if (a.q.n_pad % np != 0) return cudaErrorInvalidValue;
+        const cudaError_t r = cls == 0   ? launch_int_c<0>(a, np, pair_smem, ctas, smem, st)
+                              : cls == 1 ? launch_int_c<1>(a, np, pair_smem, ctas, smem, st)
+                              : cls == 2 ? launch_int_c<2>(a, np, pair_smem, ctas, smem, st)
+                              : cls == 3 ? launch_int_c<3>(a, np, pair_smem, ctas, smem, st)
+                                         : launch_int_c<4>(a, np, pair_smem, ctas, smem, st);
+        if (r != cudaSuccess) return r;
     }
     return cudaSuccess;
 }
@@ -486,8 +463,8 @@ extern "C" qts_status qts_shap_interactions(qts_ensemble* e, const float* X, int
         return fail(QTS_ERR_UNSUPPORTED, "interactions support paths of at most 32 unique features");
     cudaStream_t s = (cudaStream_t)stream;
     if (n_quad != QTS_NQ_EXACT && (n_quad < 1 || n_quad > QTS_MAX_QUAD)) return fail(QTS_ERR_ARG, "quadrature rule");
-    // the sibling-pair tables (built on the first call that needs them)
-    st = ensure_batch_tables(e);
+    // the block tables (built on the first call that needs them)
+    st = ensure_blocks(e, false);
     if (st != QTS_OK) return st;
     const int64_t n_pairs = (int64_t)F * (F - 1) / 2;
     const size_t bytes = sizeof(double) * (size_t)((n_pairs + F) * M);
@@ -497,12 +474,9 @@ extern "C" qts_status qts_shap_interactions(qts_ensemble* e, const float* X, int
     double* acc_phi = acc_pair + n_pairs * M;
     cudaError_t ce = cudaMemsetAsync(e->d_work, 0, bytes, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "workspace clear");
-    // QTS_NQ_EXACT: the pair terms need ceil((D - 1) / 2) points, but the diagonal
-    // holds first-order values, so a bucket takes the first-order count ceil(D / 2)
-    // (Thm 2)
-    ce = launch_int_buckets(e, true, X, M, F, n_quad, 0, acc_pair, acc_phi, s);
+    ce = launch_int_blocks(e, X, M, F, n_quad, acc_pair, acc_phi, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction kernel launch");
-    ce = launch_int_finalize(acc_pair, acc_phi, M, F, e->bprep.bias, phi_ij, s);
+    ce = launch_int_finalize(acc_pair, acc_phi, M, F, e->prep.bias, phi_ij, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction finalize launch");
     return QTS_OK;
 }
@@ -614,7 +588,7 @@ extern "C" qts_status qts_shap_interactions_noalloc(qts_ensemble* e, const float
     // the array keeps the previous call's sums: clear the part this call uses
     cudaError_t ce = cudaMemsetAsync(scratch, 0, sizeof(double) * (size_t)need, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "scratch clear");
-    ce = launch_int_buckets(e, false, X, M, F, n_quad, nq, acc_pair, acc_phi, s);
+    ce = launch_int_buckets(e, X, M, F, nq, acc_pair, acc_phi, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction kernel launch");
     ce = launch_int_finalize(acc_pair, acc_phi, M, F, e->prep.bias, phi_ij, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction finalize launch");

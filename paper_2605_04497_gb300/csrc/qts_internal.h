@@ -116,24 +116,6 @@ qts_status prepare(int32_t n_trees, const int64_t* off, const int32_t* left, con
 // Gauss-Legendre nodes on [0,1] (Golub-Welsch via Jacobi eigen-decomposition).
 bool gauss_legendre(int n, double* t, double* w);
 
-// Device copies of one set of path tables and the adjoint's metadata.
-struct DevTables {
-    void* rec = nullptr;               // Rec32 records
-    int64_t* path_leaf = nullptr;
-    double* path_zprod = nullptr;
-    double* path_val = nullptr;
-    double* slot_zexcl = nullptr;
-    int64_t* slot_edge_begin = nullptr;
-    int64_t* edge_node = nullptr;
-    double* edge_coef = nullptr;
-    int64_t* empty_leaf = nullptr;
-    int64_t* pair_leaf2 = nullptr;     // pair tables only
-    double* pair_zprod2 = nullptr;
-    double* pair_z = nullptr;
-    int64_t* pair_gslot = nullptr;
-    int64_t bytes = 0;
-};
-
 // Block tables of the FP32 first-order and adjoint passes (layout: qts_blocks.h).
 struct BlockBucket {  // all blocks of one width and height
     int D = 0, h = 0;
@@ -221,11 +203,9 @@ struct qts_ensemble {
     int64_t* d_dfs_off = nullptr;     // per tree, n_trees + 1
     int dfs_levels = 0;               // internal-node depth + 1
     int64_t dfs_records = 0;
-    // pair tables of the batched pass (sibling leaves merged), built on the
-    // first batched call that includes this ensemble
-    qts::Prepared bprep;
-    qts::DevTables bdev;
-    bool bready = false;
+    // sizes of the path tables with sibling leaves merged (qts_get_batch_info)
+    qts::Prepared pair_sizes;
+    bool pair_ready = false;
     // block tables of the FP32 first-order and adjoint passes, built on the
     // first call that needs them (the adjoint's part on the first such call)
     std::vector<qts::BlockBucket> blk;
@@ -247,8 +227,7 @@ qts_status ensure_workspace(qts_ensemble* e, size_t bytes);
 qts_status upload(qts_ensemble* e);
 void release_device(qts_ensemble* e);
 void release_dfs(qts_ensemble* e);      // drop the depth-first program (rebuilt on demand)
-qts_status ensure_batch_tables(qts_ensemble* e);  // build the pair tables of the batched pass
-void release_batch_tables(qts_ensemble* e);
+qts_status ensure_pair_sizes(qts_ensemble* e);
 // build the block tables, with grad those of the adjoint too
 void build_blocks(const qts_ensemble* e, bool grad, BlockHost* out);
 qts_status ensure_blocks(qts_ensemble* e, bool grad);
@@ -298,11 +277,14 @@ cudaError_t launch_fwd_few(const qts_ensemble* e, const float* X, int64_t M, int
                            cudaStream_t st);
 cudaError_t launch_fwd64(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* phi,
                          cudaStream_t st);
+cudaError_t launch_int_blocks(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* acc_pair,
+                              double* acc_phi, cudaStream_t st);
 cudaError_t launch_int_finalize(const double* acc_pair, const double* acc_phi, int64_t M, int F,
                                 double bias, float* out, cudaStream_t st);
-// FP32 adjoint of one request (workspace: adjoint_work_bytes, block tables with grad)
+// FP32 adjoint of one request (work: adjoint_work_bytes of device memory; block
+// tables with grad)
 size_t adjoint_work_bytes(const qts_ensemble* e, int64_t M, int F);
-cudaError_t launch_adjoint_blocks(qts_ensemble* e, const float* X, const float* grad, int64_t M, int F, int n_quad,
-                                  double* d_leaf, double* d_z, cudaStream_t st);
+cudaError_t launch_adjoint_blocks(qts_ensemble* e, void* work, const float* X, const float* grad, int64_t M, int F,
+                                  int n_quad, double* d_leaf, double* d_z, cudaStream_t st);
 
 }  // namespace qts
