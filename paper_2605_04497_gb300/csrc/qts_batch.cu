@@ -103,7 +103,7 @@ __host__ __device__ constexpr int batch_class(int D, int h) {
     if (D > 32) return D;
     if (D > 16) return 32;
     const int regs = 12 * D + (h == 0 ? 0 : h == 1 ? 10 : h == 2 ? 36 : 88) + 35;
-    return regs <= 128 ? 8 : regs <= 168 ? 12 : 16;
+    return regs <= 90 ? 8 : regs <= 168 ? 12 : 16;
 }
 constexpr int batch_blocks(int cls) { return cls == 8 ? 4 : cls == 12 ? 3 : cls == 16 ? 2 : 1; }
 

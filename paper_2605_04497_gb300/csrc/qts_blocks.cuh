@@ -10,16 +10,20 @@ namespace qts {
 __device__ __forceinline__ float4 rec4(const Rec32* r) { return *reinterpret_cast<const float4*>(r); }
 
 // Whether a sample takes a node's left edge, its right edge.  Only a block's root
-// (ROOT) can have an interval left by splits above it.
+// (ROOT) can have an interval left by splits above it; below it hi = +inf still
+// excludes x = +inf, as the path tables' half-open intervals do (HAS_NAN: some
+// value of the tile is NaN or +inf, so the others need no test).
 template <bool ROOT, bool HAS_NAN>
 __device__ __forceinline__ void node_sides(float x, const float4& b, bool* l, bool* r) {
-    const uint32_t bits = __float_as_uint(b.w);
-    bool in = !ROOT || (x >= b.y && x < b.z), left = x < b.x;
+    bool in = true, left = x < b.x;
+    if (ROOT) in = x >= b.y && x < b.z;
+    else if (HAS_NAN) in = x < b.z;
     if (HAS_NAN && x != x) {
+        const uint32_t bits = __float_as_uint(b.w);
         in = !ROOT || (bits & kNanOk) != 0;
         left = (bits & kDefLeft) != 0;
     }
-    *l = in && left;
+    *l = ROOT ? in && left : left;  // below the root, theta <= hi: left implies x < hi
     *r = in && !left;
 }
 

@@ -279,7 +279,7 @@ cudaError_t launch_fwd64(const qts_ensemble* e, const float* X, int64_t M, int F
     for (const BlockBucket& b : e->blk) total += (double)b.n * blk_cost(b.D, b.h);
     total *= (double)tiles;
     for (int cls = 0; cls < k64Classes; ++cls) {
-        for (int nq = QTS_MAX_QUAD; nq >= 1; --nq) {  // one launch per rule of the class
+        for (int nq = n_quad == QTS_NQ_EXACT ? QTS_MAX_QUAD : n_quad; nq >= (n_quad == QTS_NQ_EXACT ? 1 : n_quad); --nq) {  // one launch per rule of the class
             Args64 a;
             a.n_seg = 0;
             a.n_tiles = (int)tiles;

@@ -17,7 +17,7 @@
 // SM and a chain of dependent products), shape flags tested per node instead of
 // complete subtrees (13.0 ms), four nodes per pass at widths up to 5 (9.3 ms).
 //
-// qts-build-parts: 11 (part 0: host code; parts 1-10: the kernels)
+// qts-build-parts: 9 (part 0: host code; parts 1-8: the kernels)
 #include <algorithm>
 
 #include "qts_blocks.cuh"
@@ -51,12 +51,15 @@ struct FbArgs {
     int* status;
 };
 
-// Register classes by width; each runs NP quadrature nodes per pass.
+// Register classes by width; each runs NP quadrature nodes per pass: eight while the
+// prefix products fit 128 registers, then four, and two from width 9 (depth 20, 8
+// trees, 5,000 samples: 18.3 ms with four nodes at 166-243 registers, 17.7 with two
+// at 128, where four thread blocks per SM make up for the second decoding).
 __host__ __device__ constexpr int fb_class(int D) { return D <= 5 ? 0 : D <= 8 ? 1 : D <= 12 ? 2 : D <= 16 ? 3 : 4; }
 [[maybe_unused]] constexpr int kFbClasses = 5;
 // nodes per pass of a class for a rule of n_pad points (padded to pairs)
 static inline int fb_np(int cls, int n_pad) {
-    int np = cls == 0 ? 8 : cls <= 3 ? 4 : 2;
+    int np = cls == 0 ? 8 : cls == 1 ? 4 : 2;
     while (np > 2 && n_pad % np != 0) np /= 2;
     return np;
 }
@@ -99,7 +102,7 @@ __device__ __forceinline__ bool fb_segment(const FbArgs& a, const FbSeg& sg, int
 }
 
 template <int CLS, int NP>
-__global__ void __launch_bounds__(kFbWarps * 32, CLS <= 1 ? 4 : CLS == 2 ? 3 : 2)
+__global__ void __launch_bounds__(kFbWarps * 32, CLS <= 3 ? 4 : 2)
     fwd_blocks_kernel(const __grid_constant__ FbArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int F = a.F;
@@ -196,18 +199,12 @@ QTS_INST(1, 4)
 QTS_INST(1, 2)
 #endif
 #if QTS_IN_PART(6)
-QTS_INST(2, 4)
-#endif
-#if QTS_IN_PART(7)
 QTS_INST(2, 2)
 #endif
-#if QTS_IN_PART(8)
-QTS_INST(3, 4)
-#endif
-#if QTS_IN_PART(9)
+#if QTS_IN_PART(7)
 QTS_INST(3, 2)
 #endif
-#if QTS_IN_PART(10)
+#if QTS_IN_PART(8)
 QTS_INST(4, 2)
 #endif
 #undef QTS_INST
@@ -250,7 +247,7 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
     total *= (double)tiles;
     for (int cls = 0; cls < kFbClasses; ++cls) {
         // one launch per rule of the class (QTS_NQ_EXACT takes one per bucket)
-        for (int nq = QTS_MAX_QUAD; nq >= 1; --nq) {
+        for (int nq = n_quad == QTS_NQ_EXACT ? QTS_MAX_QUAD : n_quad; nq >= (n_quad == QTS_NQ_EXACT ? 1 : n_quad); --nq) {
             FbArgs a;
             a.n_seg = 0;
             int64_t ctas = 0;
@@ -291,8 +288,8 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
                 cudaError_t r = cudaErrorInvalidValue;
 #define QTS_GO(C, N) \
     if (cls == C && np == N) r = launch_fb<C, N>(a, ctas, smem, st);
-                QTS_GO(0, 8) QTS_GO(0, 4) QTS_GO(0, 2) QTS_GO(1, 4) QTS_GO(1, 2) QTS_GO(2, 4) QTS_GO(2, 2)
-                QTS_GO(3, 4) QTS_GO(3, 2) QTS_GO(4, 2)
+                QTS_GO(0, 8) QTS_GO(0, 4) QTS_GO(0, 2) QTS_GO(1, 4) QTS_GO(1, 2) QTS_GO(2, 2)
+                QTS_GO(3, 2) QTS_GO(4, 2)
 #undef QTS_GO
                 a.n_seg = 0;
                 ctas = 0;

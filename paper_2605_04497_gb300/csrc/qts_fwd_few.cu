@@ -157,7 +157,7 @@ cudaError_t launch_fwd_few(const qts_ensemble* e, const float* X, int64_t M, int
     const int group = (int)(32 / M);
     const size_t smem = 2 * (size_t)(F + 1) * kTileLd * 4;
     for (int cls = 0; cls < kFewClasses; ++cls) {
-        for (int nq = QTS_MAX_QUAD; nq >= 1; --nq) {  // one launch per rule of the class
+        for (int nq = n_quad == QTS_NQ_EXACT ? QTS_MAX_QUAD : n_quad; nq >= (n_quad == QTS_NQ_EXACT ? 1 : n_quad); --nq) {  // one launch per rule of the class
             FewArgs a;
             a.n_seg = 0;
             a.F = F;
