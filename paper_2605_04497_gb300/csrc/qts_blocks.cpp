@@ -59,6 +59,10 @@ struct Walker {
     std::vector<int8_t> root;
     std::vector<double> best;
     std::vector<int32_t> order;
+    std::vector<int32_t> count;  // per feature: edges of the walk's path that split on it
+    int n_uniq = 0;              // features with count > 0
+    std::vector<int> own;        // scratch of chain()
+    std::vector<double> after;
     int64_t base = 0;
 
     // scratch of the block under construction
@@ -121,12 +125,25 @@ struct Walker {
     // chain the z-gradient in `slot` (times scale) of the path's element on f to
     // its edges: dz/dw = product of the element's other edge weights
     void chain(int32_t f, int slot, double scale) {
-        for (size_t a = 0; a < path.size(); ++a) {
-            if (path[a].feat != f) continue;
-            double c = scale;
-            for (size_t b = 0; b < path.size(); ++b)
-                if (b != a && path[b].feat == f) c *= path[b].w;
-            add(path[a].child, false, slot, c);
+        own.clear();
+        for (size_t k = 0; k < path.size(); ++k)
+            if (path[k].feat == f) own.push_back((int)k);
+        if (own.size() <= 8) {
+            for (int a : own) {
+                double c = scale;
+                for (int b : own)
+                    if (b != a) c *= path[b].w;
+                add(path[a].child, false, slot, c);
+            }
+            return;
+        }
+        // long chains (degenerate trees): products before and after each edge
+        after.assign(own.size() + 1, 1.0);
+        for (size_t k = own.size(); k-- > 0;) after[k] = after[k + 1] * path[own[k]].w;
+        double before = scale;
+        for (size_t k = 0; k < own.size(); ++k) {
+            add(path[own[k]].child, false, slot, before * after[k + 1]);
+            before *= path[own[k]].w;
         }
     }
 
@@ -274,11 +291,17 @@ struct Walker {
         std::vector<Item> stack;
         stack.push_back({0, 0, {}});
         path.clear();
+        count.assign((size_t)e->n_features, 0);
+        n_uniq = 0;
         while (!stack.empty()) {
             const Item it = stack.back();
             stack.pop_back();
-            path.resize((size_t)std::max(0, it.depth - 1));
-            if (it.depth > 0) path.push_back(it.in);
+            for (; (int)path.size() > std::max(0, it.depth - 1); path.pop_back())
+                if (--count[path.back().feat] == 0) --n_uniq;
+            if (it.depth > 0) {
+                path.push_back(it.in);
+                if (count[it.in.feat]++ == 0) ++n_uniq;
+            }
             on(it.v);
             if (is_leaf(it.v)) continue;
             for (int side = 1; side >= 0; --side) {
@@ -299,16 +322,8 @@ struct Walker {
         order.clear();
         walk([&](int32_t v) {
             order.push_back(v);
-            int u = 0;
-            bool r = false;
-            for (size_t k = 0; k < path.size(); ++k) {
-                bool first = true;
-                for (size_t q = 0; q < k && first; ++q) first = path[q].feat != path[k].feat;
-                u += first;
-                r = r || (!is_leaf(v) && path[k].feat == e->feature[base + v]);
-            }
-            uniq[v] = (int16_t)u;
-            rep[v] = r;
+            uniq[v] = (int16_t)n_uniq;
+            rep[v] = !is_leaf(v) && count[e->feature[base + v]] > 0;
         });
         // children come after their parents in `order`
         for (size_t i = order.size(); i-- > 0;) {
