@@ -11,12 +11,12 @@
 //
 // Bound by instruction issue and FP32 (8 to 16 warps per SM).  Measured, path
 // tables before and block tables now: eight requests of 17-100 trees, depth 4-13,
-// 40-2,000 samples 8.61 -> 4.60 ms (4.16 with the classes' kernels as parallel
-// branches); sixteen of at most 200 samples 3.28 -> 0.38 ms (0.17 with one launch for
+// 40-2,000 samples 8.61 -> 4.60 ms (4.10 with the classes' kernels as parallel
+// branches); sixteen of at most 200 samples 3.28 -> 0.38 ms (0.15 with one launch for
 // all requests' preparation and epilogue; by
 // default the warps of a thread block now share 64 samples and split the blocks:
 // with 64 samples per warp a request of fewer than 193 left warps idle); adjoint
-// alone, 200 trees of depth 8, 4,001 samples 3.30 -> 2.00 ms.
+// alone, 200 trees of depth 8, 4,001 samples 3.30 -> 1.93 ms.
 //
 // qts-build-parts: 12 (part 0: host code; parts 1-3: the pass of two samples per
 // lane, parts 4-11: the others, one register class each)
@@ -575,14 +575,14 @@ struct SegHost {
 
 constexpr int kBatchSub = 16;  // blocks per staged sub-chunk
 
-// Blocks per item of the default launch, from the work of the whole launch: a
+// Blocks per item of the default launch, from the work of the whole launch: two
 // dozen items per resident thread block evens out the tail and serves small
 // requests; at least 32 blocks keep the tile set-up and the phi flush (about
 // 64 F atomics) small beside the sweeps, and 2,048 are plenty.
 static void default_items(std::vector<SegHost>& segs) {
     double total = 0.0;
     for (const SegHost& s : segs) total += s.unit * (double)s.d.n * s.d.n_tiles;
-    const double share = total / (12.0 * 2.5 * num_sms());
+    const double share = total / (24.0 * 2.5 * num_sms());
     for (SegHost& s : segs) {
         if (s.d.per_item > 0) continue;
         const double per = std::min(2048.0, std::max(32.0, share / s.unit));

@@ -11,8 +11,9 @@
 //
 // Bound by instruction issue and FP32: at 1,000 trees of depth 8 (239,216 leaves,
 // 10,000 samples, F = 50) the path tables needed 14.98 ms at about 150 warp
-// instructions per leaf and 32 samples; the blocks take 8.85 ms (at most two
-// levels of splits per block: 11.0, one: about 15).  Tried on the way and
+// instructions per leaf and 32 samples; the blocks take 8.34 ms (8.85 before
+// staging 16 and more at a time; then at most two levels of splits per block: 11.0,
+// one: about 15).  Tried on the way and
 // slower: two samples per lane with a loop over the nodes (18-31 ms: 8 warps per
 // SM and a chain of dependent products), shape flags tested per node instead of
 // complete subtrees (13.0 ms), four nodes per pass at widths up to 5 (9.3 ms).
@@ -54,7 +55,7 @@ struct FbArgs {
 // Register classes by width; each runs NP quadrature nodes per pass: eight while the
 // prefix products fit 128 registers, then four, and two from width 9 (depth 20, 8
 // trees, 5,000 samples: 18.3 ms with four nodes at 166-243 registers, 17.7 with two
-// at 128, where four thread blocks per SM make up for the second decoding).
+// at 128 and 16.7 with longer staging, where four thread blocks per SM make up for the second decoding).
 __host__ __device__ constexpr int fb_class(int D) { return D <= 5 ? 0 : D <= 8 ? 1 : D <= 12 ? 2 : D <= 16 ? 3 : 4; }
 [[maybe_unused]] constexpr int kFbClasses = 5;
 // nodes per pass of a class for a rule of n_pad points (padded to pairs)
@@ -260,18 +261,18 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
             const int np = fb_np(cls, a.q.n_pad);
             std::sort(pick.begin(), pick.end(),
                       [](const BlockBucket* x, const BlockBucket* y) { return blk_cost(x->D, x->h) > blk_cost(y->D, y->h); });
-            // tiles of phi: one per warp while that leaves at least two thread
-            // blocks per SM, or the shared tile with atomics would not do better
-            a.sub = 8;
             int max_stride = 0;
             for (const BlockBucket* b : pick) max_stride = std::max(max_stride, blk_stride(b->D, b->h));
+            // tiles of phi: one per warp while that leaves two thread blocks per SM,
+            // then a shared one with atomics.  Blocks staged at a time: the most
+            // that keeps four thread blocks per SM (a staged sub-chunk ends on a
+            // barrier: 8 instead of 16 cost 5% on 1,000 trees of depth 8), and for
+            // wide inputs what fits at all
+            a.nphi = fb_smem(F, kFbWarps, 8 * max_stride) <= 110 * 1024 ? kFbWarps : 1;
+            a.sub = 32;
+            while (a.sub > 8 && fb_smem(F, a.nphi, a.sub * max_stride) > 56 * 1024) a.sub /= 2;
+            while (a.sub > 1 && fb_smem(F, a.nphi, a.sub * max_stride) > kSmemMax) a.sub /= 2;
             stage = a.sub * max_stride;
-            a.nphi = kFbWarps;
-            if (fb_smem(F, a.nphi, stage) > 110 * 1024) a.nphi = 1;
-            while (a.sub > 1 && fb_smem(F, a.nphi, stage) > kSmemMax) {
-                a.sub /= 2;
-                stage = a.sub * max_stride;
-            }
             const size_t smem = fb_smem(F, a.nphi, stage);
             if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
             a.stage = stage;

@@ -46,7 +46,8 @@ constexpr uint32_t kNanOk = 0x80000000u;
 constexpr uint32_t kCat = 0x40000000u;
 constexpr uint32_t kOtherOk = 0x20000000u;
 constexpr uint32_t kFeatMask = 0x00FFFFFFu;
-// Sibling-pair element (pair tables of the batched pass; always the path's last
+// Sibling-pair element (path tables with sibling leaves merged, which
+// QTS_DESCRIBE_PAIRS describes and qts_get_batch_info counts; always the path's last
 // record).  Leaves A (left) and B (right) of a numerical split at threshold
 // theta share every other element; this one has z = alpha = val_A z_A +
 // val_B z_B and [lo, hi) = the interval of the splits on the feature above the
@@ -97,7 +98,7 @@ struct Prepared {
     int max_unique = 0;
     double bias = 0.0;  // E[f]
     bool has_cat = false;  // some element is categorical: kernels take their NaN-aware variant
-    // pair tables (sibling leaves of a numerical split as one path, kPairElem)
+    // sibling leaves of a numerical split as one path (kPairElem)
     bool pairs = false;
     int64_t n_pair_paths = 0;
     std::vector<int64_t> pair_leaf2;   // per path: leaf B of a pair, -1 otherwise (path_leaf is A)
