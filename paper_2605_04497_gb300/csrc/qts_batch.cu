@@ -46,8 +46,8 @@ struct SegDev {
 
 constexpr int kBatchWarps = 4;
 
-// Per request: x and grad_phi transposed to [feature][Mpad] (row F of XT is
-// zero for padding elements; columns >= M are zero), so a warp reads one
+// Per request: x and grad_phi transposed to [feature][Mpad] (row F of both is
+// zero for padding elements and neutral nodes; columns >= M are zero), so a warp reads one
 // feature of its 32 samples as one coalesced 128-byte line.
 struct ReqDev {
     const float* XT;
@@ -380,7 +380,10 @@ __global__ void __launch_bounds__(256) batch_prepare_kernel(const __grid_constan
     k -= tiles;
     if (w.G) {
         if (k < tiles) {
-            transpose_tile(w.G, w.M, w.F + 1, w.F + 1, w.GT, w.F + 1, w.Mpad, nullptr, k / rows * 32,
+            // Row F stays zero: neutral nodes and padding name feature F, and the
+            // weight of E[f] (column F of grad_phi) is no gradient of theirs.  In a
+            // neutral node it cancels only to FP32 rounding between a leaf's two sums.
+            transpose_tile(w.G, w.M, w.F, w.F + 1, w.GT, w.F + 1, w.Mpad, nullptr, k / rows * 32,
                            (int)(k % rows) * 32);
             return;
         }

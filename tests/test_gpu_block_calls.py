@@ -1,0 +1,65 @@
+"""Calls around the block tables: what a call may rely on besides its inputs
+(captures, workspaces, saved tuning files) and inputs at the edge of what the
+kernels' FP32 sums hold, against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from helpers import rel_err_rows
+
+pytestmark = pytest.mark.gpu
+
+TOL32 = 1e-5  # FP32 tables: the bound every FP32 test of this suite uses
+
+
+@pytest.fixture(scope="module")
+def qts():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2605_04497_gb300 import build as b
+
+    b.build()
+    import paper_2605_04497_gb300 as q
+
+    return q
+
+
+def _rel(a, b):
+    return np.abs(a - b).max() / max(np.abs(b).max(), 1e-300)
+
+
+def _request(qts, E, X, G=None):
+    """One batched request on new outputs; without G forward only."""
+    import torch
+
+    new = lambda *s: torch.empty(s, dtype=torch.float64, device="cuda")
+    it = dict(ens=E, X=X, phi=new(len(X), E.n_features + 1))
+    if G is not None:
+        it.update(grad_phi=G, d_leaf=new(E.n_nodes), d_z=new(E.n_nodes))
+    return it
+
+
+@pytest.mark.parametrize("F", [9, 130])  # two samples per lane, one sample per lane
+def test_bias_weights_stay_out_of_the_leaf_gradients(qts, F):
+    """grad_phi's last column weighs E[f]; where its sum cancels, whatever its
+    size, it leaves the leaf gradients' digits alone, at leaves of every height."""
+    import torch
+
+    ens = synth.grow(9500, 6, 6, F, 2000, 0.5, min_rows=3)
+    M = 64
+    X = synth.normal(9500, synth.STREAM_X, (M, F))
+    G = synth.normal(9500, synth.STREAM_GRAD, (M, F + 1))
+    G[:, F] = np.where(np.arange(M) % 2, 1e4, -1e4)  # their sum is exactly zero
+    dl_ref, dz_ref = oracle.grad_exact(ens, X, G)
+    E = qts.Ensemble.from_arrays(ens)
+    Xd, Gd = torch.from_numpy(X).cuda(), torch.from_numpy(G).cuda()
+    dl, dz = qts.shap_backward(E, Xd, Gd)
+    it = _request(qts, E, Xd, Gd)
+    qts.batched_fwd_bwd(qts.make_requests([it]))
+    E.sync_status()
+    for a, b in ((dl, dl_ref), (dz, dz_ref), (it["d_leaf"], dl_ref), (it["d_z"], dz_ref)):
+        assert _rel(a.cpu().numpy(), b) <= TOL32
+    E.close()
