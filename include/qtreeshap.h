@@ -29,6 +29,11 @@
  *     qts_last_error() describes it (thread-local string).
  *   - Calls that use the same ensemble must not overlap on the GPU (they share
  *     the ensemble's workspace); enqueue them on one stream.
+ *   - A call may be captured into a CUDA graph (exceptions are named at the
+ *     entry points).  The graph then holds the ensemble's tables and workspace:
+ *     replay it only until qts_update_params or qts_free; other calls, also larger
+ *     ones, may come between its replays.  A workspace that a capture used
+ *     and a later call outgrew stays allocated until qts_free.
  *   - X is M x F row-major fp32 with F equal to the ensemble's n_features.
  *     x[f] < threshold goes left, x[f] >= threshold right, NaN goes the node's
  *     default direction (categorical splits: see qts_load_ensemble_cat).

@@ -184,20 +184,36 @@ void release_blocks(qts_ensemble* e) {
     e->blk_ready = e->blk_grad_ready = false;
 }
 
-qts_status ensure_workspace(qts_ensemble* e, size_t bytes) {
-    if (bytes <= e->work_bytes) return QTS_OK;
-    if (e->d_work) {
-        batch_forget(e);
-        cudaError_t err = cudaDeviceSynchronize();
-        if (err != cudaSuccess) return cuda_fail(err, "workspace resize sync");
-        cudaFree(e->d_work);
-        e->d_work = nullptr;
-        e->work_bytes = 0;
+bool is_capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) {
+        cudaGetLastError();  // the legacy stream, while another stream is being captured
+        return false;
     }
-    size_t want = std::max(bytes, (size_t)1 << 20);
-    cudaError_t err = cudaMalloc(&e->d_work, want);
-    if (err != cudaSuccess) return cuda_fail(err, "workspace allocation");
-    e->work_bytes = want;
+    return s == cudaStreamCaptureStatusActive;
+}
+
+// A captured call leaves the workspace's address in the caller's graph, which may be
+// replayed after any later call: such a workspace is never freed before the
+// ensemble, a call that outgrows it gets a new one beside it.
+qts_status ensure_workspace(qts_ensemble* e, size_t bytes, cudaStream_t st) {
+    if (bytes > e->work_bytes) {
+        if (e->d_work) {
+            batch_forget(e);
+            cudaError_t err = cudaDeviceSynchronize();
+            if (err != cudaSuccess) return cuda_fail(err, "workspace resize sync");
+            if (e->work_captured) e->retired.push_back(e->d_work);
+            else cudaFree(e->d_work);
+            e->d_work = nullptr;
+            e->work_bytes = 0;
+            e->work_captured = false;
+        }
+        size_t want = std::max(bytes, (size_t)1 << 20);
+        cudaError_t err = cudaMalloc(&e->d_work, want);
+        if (err != cudaSuccess) return cuda_fail(err, "workspace allocation");
+        e->work_bytes = want;
+    }
+    if (!e->work_captured && is_capturing(st)) e->work_captured = true;
     return QTS_OK;
 }
 
@@ -498,6 +514,7 @@ void qts_free(qts_ensemble* e) {
     release_device(e);
     cudaFree(e->d_status);
     cudaFree(e->d_work);
+    for (void* p : e->retired) cudaFree(p);
     delete e;
 }
 

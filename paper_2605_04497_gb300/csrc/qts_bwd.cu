@@ -314,13 +314,11 @@ extern "C" qts_status qts_shap_backward(qts_ensemble* e, const float* X, int64_t
         // memory of the captured graph's own.
         const size_t need = adjoint_work_bytes(e, M, F);
         void* own = nullptr;
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (need > e->work_bytes && cudaStreamIsCapturing(s, &cap) == cudaSuccess &&
-            cap == cudaStreamCaptureStatusActive) {
+        if (need > e->work_bytes && is_capturing(s)) {
             ce = cudaMallocAsync(&own, need, s);
             if (ce != cudaSuccess) return cuda_fail(ce, "adjoint workspace");
         } else {
-            st = ensure_workspace(e, need);
+            st = ensure_workspace(e, need, s);
             if (st != QTS_OK) return st;
         }
         ce = launch_adjoint_blocks(e, own ? own : e->d_work, X, grad_phi, M, F, n_quad, d_leaf, d_z, s);
@@ -332,7 +330,7 @@ extern "C" qts_status qts_shap_backward(qts_ensemble* e, const float* X, int64_t
     }
     const Prepared& P = e->prep;
     const size_t bytes = sizeof(double) * (size_t)(4 + P.n_paths + P.n_slots);
-    st = ensure_workspace(e, bytes);
+    st = ensure_workspace(e, bytes, s);
     if (st != QTS_OK) return st;
     double* gb = (double*)e->d_work;
     double* g_val = gb + 4;

@@ -468,7 +468,7 @@ extern "C" qts_status qts_shap_interactions(qts_ensemble* e, const float* X, int
     if (st != QTS_OK) return st;
     const int64_t n_pairs = (int64_t)F * (F - 1) / 2;
     const size_t bytes = sizeof(double) * (size_t)((n_pairs + F) * M);
-    st = ensure_workspace(e, bytes);
+    st = ensure_workspace(e, bytes, s);
     if (st != QTS_OK) return st;
     double* acc_pair = (double*)e->d_work;
     double* acc_phi = acc_pair + n_pairs * M;

@@ -268,7 +268,7 @@ extern "C" qts_status qts_shap_interactions3(qts_ensemble* e, const float* X, in
     const int64_t n_tri = choose3(F);
     if (n_tri == 0) return QTS_OK;
     const size_t bytes = sizeof(double) * (size_t)(n_tri * M);
-    st = ensure_workspace(e, bytes);
+    st = ensure_workspace(e, bytes, s);
     if (st != QTS_OK) return st;
     double* acc = (double*)e->d_work;
     cudaError_t ce = cudaMemsetAsync(acc, 0, bytes, s);

@@ -196,6 +196,8 @@ struct qts_ensemble {
     // grow-only workspace (interaction accumulators, adjoint per-path sums)
     void* d_work = nullptr;
     size_t work_bytes = 0;
+    bool work_captured = false;       // a captured call holds d_work's address
+    std::vector<void*> retired;       // outgrown workspaces that captured graphs may still use
     // depth-first (Algorithm 1) program: preorder records of the internal
     // nodes, built on the first call that needs it
     void* d_dfs = nullptr;
@@ -222,7 +224,9 @@ namespace qts {
 void set_error(const std::string& msg);
 qts_status fail(qts_status st, const std::string& msg);
 qts_status cuda_fail(cudaError_t e, const char* what);
-qts_status ensure_workspace(qts_ensemble* e, size_t bytes);
+// At least `bytes` of workspace for a call on `st`.
+qts_status ensure_workspace(qts_ensemble* e, size_t bytes, cudaStream_t st);
+bool is_capturing(cudaStream_t st);
 qts_status upload(qts_ensemble* e);
 void release_device(qts_ensemble* e);
 void release_dfs(qts_ensemble* e);      // drop the depth-first program (rebuilt on demand)

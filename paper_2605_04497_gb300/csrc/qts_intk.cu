@@ -343,7 +343,7 @@ extern "C" qts_status qts_shap_interactions_order(qts_ensemble* e, const float* 
     if (!make_quad(nodes_for(n_quad, e->prep.max_unique, order), &qf, nullptr))
         return fail(QTS_ERR_ARG, "quadrature rule");
     const size_t bytes = sizeof(double) * (size_t)(n_sub * M);
-    st = ensure_workspace(e, bytes);
+    st = ensure_workspace(e, bytes, s);
     if (st != QTS_OK) return st;
     double* acc = (double*)e->d_work;
     cudaError_t ce = cudaMemsetAsync(acc, 0, bytes, s);

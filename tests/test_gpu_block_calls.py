@@ -63,3 +63,50 @@ def test_bias_weights_stay_out_of_the_leaf_gradients(qts, F):
     for a, b in ((dl, dl_ref), (dz, dz_ref), (it["d_leaf"], dl_ref), (it["d_z"], dz_ref)):
         assert _rel(a.cpu().numpy(), b) <= TOL32
     E.close()
+
+
+@pytest.mark.parametrize("kind", ["adjoint", "pairs"])
+def test_captured_call_survives_a_larger_one(qts, kind):
+    """A graph that holds the workspace is replayed after an adjoint call of more
+    samples, which needs a larger one: the captured one must not have been freed."""
+    import torch
+
+    F, M, M2 = 10, 400000, 2000000
+    ens = synth.grow(9600, 2, 4, F, 2000, 0.5, min_rows=3)
+    E = qts.Ensemble.from_arrays(ens)
+    X = torch.from_numpy(synth.normal(9600, synth.STREAM_X, (M2, F))).cuda()
+    G = torch.from_numpy(synth.normal(9600, synth.STREAM_GRAD, (M2, F + 1))).cuda()
+    new = lambda: torch.zeros(E.n_nodes, dtype=torch.float64, device="cuda")
+    outs, out2 = (new(), new()), (new(), new())
+    rows = M if kind == "adjoint" else 100000
+    Xs, Gs = X[:rows].contiguous(), G[:rows].contiguous()
+    if kind == "pairs":
+        outs = (torch.zeros((rows, F + 1, F + 1), dtype=torch.float32, device="cuda"),)
+
+    def call():
+        if kind == "adjoint":
+            qts.shap_backward(E, Xs, Gs, d_leaf=outs[0], d_z=outs[1])
+        else:
+            qts.shap_interactions(E, Xs, out=outs[0])
+
+    call()
+    torch.cuda.synchronize()
+    ref = [o.cpu().numpy() for o in outs]
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        call()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    qts.shap_backward(E, X, G, d_leaf=out2[0], d_z=out2[1])
+    torch.cuda.synchronize()
+    # transposed copies of the M2 samples; the captured workspace is not given back
+    grown = 2 * 4 * (F + 1) * M2
+    assert free - torch.cuda.mem_get_info()[0] >= 0.95 * grown
+    for o in outs:
+        o.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    for o, r in zip(outs, ref):
+        assert _rel(o.cpu().numpy(), r) <= (1e-9 if kind == "adjoint" else 1e-6)
+    E.sync_status()
+    E.close()
