@@ -163,9 +163,9 @@ qts_status qts_update_params(qts_ensemble *ens, const float *z, const float *lea
  * lane.
  * Runs on a second set of tables in which a small subtree's leaves (up to
  * eight) are evaluated together against the merged elements they share; it is
- * built by the first call that needs it (host preparation, cudaMalloc and
- * synchronous copies), so that first call must not be inside a stream capture;
- * later calls only enqueue on `stream`.
+ * built by the first call that needs it (host preparation, cudaMalloc and copies
+ * that the call waits for, on a stream of its own, so that it may itself be under
+ * capture); later calls only enqueue on `stream`.
  */
 qts_status qts_shap_values(qts_ensemble *ens, const float *X, int64_t M, int32_t F,
                            int32_t n_quad, double *phi, qts_stream_t stream);
@@ -205,8 +205,9 @@ qts_status qts_shap_values_alg1(qts_ensemble *ens, const float *X, int64_t M, in
  *           [s][F][F] = E[f], other entries of row/column F are 0.
  * Cross-tree accumulation is FP64 in the ensemble's workspace (device memory
  * of M * (F(F+1)/2) doubles, grown on demand with cudaMalloc).  Runs on the
- * block tables of qts_shap_values (built by the first call that needs them, so
- * that call must not be inside a stream capture).  n_quad as qts_shap_values;
+ * block tables of qts_shap_values (built by the first call that needs them); under
+ * capture the workspace must have been grown before, by a call of the same size.
+ * n_quad as qts_shap_values;
  * QTS_NQ_EXACT takes the first-order count ceil(w / 2) of a bucket's widest path
  * w (the pair terms need ceil((w - 1) / 2), the diagonal's first-order values
  * ceil(w / 2)).

@@ -139,9 +139,48 @@ qts_status ensure_pair_sizes(qts_ensemble* e) {
     return QTS_OK;
 }
 
+static void free_blocks(BlockDev& T) {
+    for (void* p : {(void*)T.rec, (void*)T.dbl, (void*)T.ent, (void*)T.bias_leaf, (void*)T.bias_z}) cudaFree(p);
+    T = BlockDev();
+}
+
+// Allocations and copies of tables that a call builds on first use.  The call may be
+// under stream capture, on this thread or another, where cudaMalloc is refused
+// unless the thread's capture mode is relaxed and a copy on the legacy stream
+// would break the capture; so the copies go through a stream of their own, and the
+// tables are there when the call returns, whatever becomes of the graph.
+struct TableUpload {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaStream_t st = nullptr;
+    cudaError_t err;
+    TableUpload() {
+        err = cudaThreadExchangeStreamCaptureMode(&mode);
+        if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    }
+    ~TableUpload() {
+        if (st) cudaStreamDestroy(st);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    TableUpload(const TableUpload&) = delete;
+    TableUpload& operator=(const TableUpload&) = delete;
+    template <typename T>
+    void add(T** dst, const std::vector<T>& src) {
+        const size_t bytes = std::max<size_t>(src.size(), 1) * sizeof(T);
+        if (err == cudaSuccess) err = cudaMalloc((void**)dst, bytes);
+        if (err == cudaSuccess && !src.empty())
+            err = cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, st);
+    }
+    cudaError_t finish() {
+        if (err == cudaSuccess) err = cudaStreamSynchronize(st);
+        return err;
+    }
+};
+
 // Block tables: built from the host copy of the model; `grad` adds the adjoint's
-// part (the records are the same either way, so they are kept).
+// part.  The records are the same either way: once they are there nothing that a
+// forward on another thread or a captured graph uses changes, also on failure.
 qts_status ensure_blocks(qts_ensemble* e, bool grad) {
+    std::lock_guard<std::mutex> lk(e->blk_mu);
     if (e->blk_ready && (!grad || e->blk_grad_ready)) return QTS_OK;
     if (grad && e->n_nodes >= ((int64_t)1 << 31)) return fail(QTS_ERR_UNSUPPORTED, "gradients of 2^31 nodes or more");
     BlockHost H;
@@ -151,34 +190,43 @@ qts_status ensure_blocks(qts_ensemble* e, bool grad) {
         return fail(QTS_ERR_OOM, "host allocation of the block tables");
     }
     if (grad && H.n_slots >= ((int64_t)1 << 32)) return fail(QTS_ERR_UNSUPPORTED, "too many adjoint sums");
-    int64_t tot = 0;
-    qts_status st = QTS_OK;
+    BlockDev T;
+    TableUpload up;
     if (!e->blk_ready) {
-        st = up(&e->blkdev.rec, H.rec, &tot, "upload block tables");
-        if (st == QTS_OK && !H.dbl.empty()) st = up(&e->blkdev.dbl, H.dbl, &tot, "upload block tables");
+        up.add(&T.rec, H.rec);
+        if (!H.dbl.empty()) up.add(&T.dbl, H.dbl);
     }
     if (grad) {
-        if (st == QTS_OK) st = up(&e->blkdev.ent, H.ent, &tot, "upload block tables");
+        up.add(&T.ent, H.ent);
+        up.add(&T.bias_leaf, H.bias_leaf);
+        up.add(&T.bias_z, H.bias_z);
+    }
+    const cudaError_t err = up.finish();
+    if (err != cudaSuccess) {
+        if (err == cudaErrorMemoryAllocation) cudaGetLastError();
+        free_blocks(T);
+        return cuda_fail(err, "upload block tables");
+    }
+    if (!e->blk_ready) {
+        e->blkdev.rec = T.rec;
+        e->blkdev.dbl = T.dbl;
+        e->blk = std::move(H.buckets);
+        e->n_blocks = H.n_blocks;
+        e->n_blk_slots = H.n_slots;
+        e->blk_ready = true;
+    }
+    if (grad) {
+        e->blkdev.ent = T.ent;
         e->blkdev.n_ent = (int64_t)H.ent.size();
-        if (st == QTS_OK) st = up(&e->blkdev.bias_leaf, H.bias_leaf, &tot, "upload block tables");
-        if (st == QTS_OK) st = up(&e->blkdev.bias_z, H.bias_z, &tot, "upload block tables");
+        e->blkdev.bias_leaf = T.bias_leaf;
+        e->blkdev.bias_z = T.bias_z;
+        e->blk_grad_ready = true;
     }
-    if (st != QTS_OK) {
-        release_blocks(e);
-        return st;
-    }
-    e->blk = std::move(H.buckets);
-    e->n_blocks = H.n_blocks;
-    e->n_blk_slots = H.n_slots;
-    e->blk_ready = true;
-    e->blk_grad_ready = e->blk_grad_ready || grad;
     return QTS_OK;
 }
 
 void release_blocks(qts_ensemble* e) {
-    BlockDev& T = e->blkdev;
-    for (void* p : {(void*)T.rec, (void*)T.dbl, (void*)T.ent, (void*)T.bias_leaf, (void*)T.bias_z}) cudaFree(p);
-    T = BlockDev();
+    free_blocks(e->blkdev);
     e->blk.clear();
     e->n_blocks = e->n_blk_slots = 0;
     e->blk_ready = e->blk_grad_ready = false;

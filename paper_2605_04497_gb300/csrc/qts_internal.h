@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -213,6 +214,7 @@ struct qts_ensemble {
     qts::BlockDev blkdev;
     int64_t n_blocks = 0, n_blk_slots = 0;
     bool blk_ready = false, blk_grad_ready = false;
+    std::mutex blk_mu;                // one thread builds them
     // per-width launch tuning (index = bucket width)
     qts::Tune tune[qts::kMaxD + 1];
     bool tuned = false;

@@ -110,3 +110,37 @@ def test_captured_call_survives_a_larger_one(qts, kind):
         assert _rel(o.cpu().numpy(), r) <= (1e-9 if kind == "adjoint" else 1e-6)
     E.sync_status()
     E.close()
+
+
+@pytest.mark.parametrize("kind", ["fp64", "fp32", "few", "adjoint", "adjoint-after-forward"])
+def test_first_call_under_capture(qts, kind):
+    """The tables that a call builds on first use may be built under capture (the
+    FP64 forward, and the adjoint's part after a forward)."""
+    import torch
+
+    F, M = 7, 5 if kind == "few" else 40
+    ens = synth.grow(9700, 4, 5, F, 2000, 0.5, min_rows=3)
+    Xh = synth.normal(9700, synth.STREAM_X, (M, F))
+    Gh = synth.normal(9700, synth.STREAM_GRAD, (M, F + 1))
+    X, G = torch.from_numpy(Xh).cuda(), torch.from_numpy(Gh).cuda()
+    E = qts.Ensemble.from_arrays(ens, fp64=kind == "fp64")
+    if kind == "adjoint-after-forward":
+        qts.shap_values(E, X)
+    phi = torch.zeros((M, F + 1), dtype=torch.float64, device="cuda")
+    dl = torch.zeros(E.n_nodes, dtype=torch.float64, device="cuda")
+    dz = torch.zeros_like(dl)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        if kind.startswith("adjoint"):
+            qts.shap_backward(E, X, G, d_leaf=dl, d_z=dz)
+        else:
+            qts.shap_values(E, X, out=phi)
+    g.replay()
+    E.sync_status()
+    if kind.startswith("adjoint"):
+        for a, b in zip((dl, dz), oracle.grad_exact(ens, Xh, Gh)):
+            assert _rel(a.cpu().numpy(), b) <= TOL32
+    else:
+        assert rel_err_rows(phi.cpu().numpy(), oracle.shap_exact(ens, Xh)).max() <= TOL32
+    E.close()
