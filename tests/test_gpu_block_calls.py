@@ -144,3 +144,30 @@ def test_first_call_under_capture(qts, kind):
     else:
         assert rel_err_rows(phi.cpu().numpy(), oracle.shap_exact(ens, Xh)).max() <= TOL32
     E.close()
+
+
+@pytest.mark.parametrize("M", [1, 8192, 8193, 20000])  # a thread block sums 8,192 samples' weights
+def test_weights_of_the_expected_value(qts, M):
+    """The gradient through E[f] alone: the sum of grad_phi's last column over all
+    samples, times a constant per node.  FP32 weights, FP64 sums."""
+    import torch
+
+    ens = synth.grow(9800, 3, 3, 4, 2000, 0.5, min_rows=3)
+    E = qts.Ensemble.from_arrays(ens)
+    X = torch.from_numpy(synth.normal(9800, synth.STREAM_X, (M, 4))).cuda()
+    g = synth.normal(9800, synth.STREAM_GRAD, (M,)) + np.float32(0.5)
+    G = torch.zeros((M, 5), device="cuda")
+    G[:, 4] = torch.from_numpy(g).cuda()
+    one = np.zeros((1, 5), np.float32)
+    one[0, 4] = 1.0
+    total = g.astype(np.float64).sum()
+    ref = [total * r for r in oracle.grad_exact(ens, np.zeros((1, 4), np.float32), one)]
+    dl, dz = qts.shap_backward(E, X, G)
+    it = _request(qts, E, X, G)
+    for _ in range(2):  # the sum starts at zero in a replay too
+        qts.batched_fwd_bwd(qts.make_requests([it]))
+    E.sync_status()
+    # other gradients are zero, so only the FP64 sum's order differs
+    for a, b in zip((dl, dz, it["d_leaf"], it["d_z"]), ref + ref):
+        assert _rel(a.cpu().numpy(), b) <= 1e-12
+    E.close()
