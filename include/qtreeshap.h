@@ -285,8 +285,9 @@ qts_status qts_shap_interactions_noalloc(qts_ensemble *ens, const float *X, int6
  *   grad_phi device, M x (F+1) fp32 (column F weights the bias E[f]).
  * FP32 ensembles run on the block tables (built on first use, as for
  * qts_shap_values) with the batched pass's kernels; the workspace holds transposed
- * copies of X and grad_phi (a captured call that would have to grow it takes that
- * memory from the captured graph instead).
+ * copies of X and grad_phi, 256 MiB of samples at a time (less where the device
+ * has no more; a captured call that would have to grow it takes that memory from
+ * the captured graph instead).
  */
 qts_status qts_shap_backward(qts_ensemble *ens, const float *X, int64_t M, int32_t F,
                              int32_t n_quad, const float *grad_phi, double *d_leaf, double *d_z,

@@ -258,7 +258,11 @@ qts_status ensure_workspace(qts_ensemble* e, size_t bytes, cudaStream_t st) {
         }
         size_t want = std::max(bytes, (size_t)1 << 20);
         cudaError_t err = cudaMalloc(&e->d_work, want);
-        if (err != cudaSuccess) return cuda_fail(err, "workspace allocation");
+        if (err != cudaSuccess) {
+            e->d_work = nullptr;
+            cudaGetLastError();  // not the next launch's error
+            return cuda_fail(err, "workspace allocation");
+        }
         e->work_bytes = want;
     }
     if (!e->work_captured && is_capturing(st)) e->work_captured = true;

@@ -1045,53 +1045,75 @@ extern "C" qts_status qts_get_batch_info(qts_ensemble* e, int64_t* n_paths, int6
 }
 
 // Adjoint of one request by the batched kernels, without a graph (qts_shap_backward).
+// The samples go through in slabs, one after the other, so that their transposed
+// copies stay small beside X and grad_phi, whatever M is.  A slab of 256 MiB (658,000
+// samples at F = 50, 40,000 at F = 832) is many times what fills the chip.
 namespace qts {
 
-size_t adjoint_work_bytes(const qts_ensemble* e, int64_t M, int F) { return batch_work(e, M, F, true).total; }
+constexpr size_t kSlabBytes = (size_t)256 << 20;
 
-cudaError_t launch_adjoint_blocks(qts_ensemble* e, void* work, const float* X, const float* grad, int64_t M, int F,
-                                  int n_quad, double* d_leaf, double* d_z, cudaStream_t st) {
+int64_t adjoint_slab(int64_t M, int F) {
+    constexpr int64_t unit = 64 * kBatchWarps;
+    const int64_t s = (int64_t)(kSlabBytes / (2 * sizeof(float) * (size_t)(F + 1))) / unit * unit;
+    return std::min(M, std::max(s, unit));
+}
+
+int64_t smaller_slab(int64_t slab) {
+    constexpr int64_t unit = 64 * kBatchWarps;
+    return slab <= unit ? 0 : std::max(unit, slab / 4 / unit * unit);
+}
+
+size_t adjoint_work_bytes(const qts_ensemble* e, int64_t slab, int F) { return batch_work(e, slab, F, true).total; }
+
+cudaError_t launch_adjoint_blocks(qts_ensemble* e, void* work, int64_t slab, const float* X, const float* grad,
+                                  int64_t M, int F, int n_quad, double* d_leaf, double* d_z, cudaStream_t st) {
     qts_request R;
     std::memset(&R, 0, sizeof(R));
     R.ens = e;
-    R.X = X;
-    R.M = M;
     R.F = F;
-    R.grad_phi = grad;
     R.d_leaf = d_leaf;
     R.d_z = d_z;
+    cudaError_t err = cudaSuccess;
     WorkArgs wa;
     wa.many = nullptr;
     wa.n = 1;
-    wa.one = request_work(R, (char*)work);
-    WorkBlocks nb;
-    number_work(wa.one, &nb);
-    if (nb.prepare > 0x7fffffffLL || nb.bias > 0x7fffffffLL || nb.entries > 0x7fffffffLL)
-        return cudaErrorInvalidConfiguration;
-    std::vector<SegHost> segs;
-    request_segments(R, (char*)work, 0, n_quad, nullptr, &segs);
-    const std::vector<LaunchHost> launches = order_segments(segs, kInlineSegs);
-    if (launches.size() > kGradHead - 1) return cudaErrorInvalidConfiguration;
-    unsigned long long* counter = (unsigned long long*)wa.one.gb + 1;  // in the head before the sums
-    cudaError_t err = cudaMemsetAsync(wa.one.gb, 0, kGradHead * sizeof(double), st);
-    if (err == cudaSuccess) err = cudaMemsetAsync(wa.one.flag, 0, sizeof(int), st);
-    if (err != cudaSuccess) return err;
-    batch_prepare_kernel<<<(unsigned)nb.prepare, 256, 0, st>>>(wa);
-    err = cudaGetLastError();
-    for (size_t c = 0; c < launches.size() && err == cudaSuccess; ++c) {
-        BatchArgs a;
-        a.segs = nullptr;
-        a.reqs = nullptr;
-        for (size_t i = 0; i < launches[c].count; ++i) a.seg[i] = segs[launches[c].first + i].d;
-        a.req = request_dev(wa.one, e);
-        err = launch_ordered(launches[c], a, counter + c, st);
+    for (int64_t s0 = 0; s0 < M && err == cudaSuccess; s0 += slab) {
+        R.X = X + s0 * F;
+        R.grad_phi = grad + s0 * (F + 1);
+        R.M = std::min(slab, M - s0);
+        wa.one = request_work(R, (char*)work);
+        if (s0 > 0) wa.one.n_g = 0;  // the sums go on from the slab before
+        WorkBlocks nb;
+        number_work(wa.one, &nb);
+        if (nb.prepare > 0x7fffffffLL || nb.bias > 0x7fffffffLL || nb.entries > 0x7fffffffLL)
+            return cudaErrorInvalidConfiguration;
+        std::vector<SegHost> segs;
+        request_segments(R, (char*)work, 0, n_quad, nullptr, &segs);
+        const std::vector<LaunchHost> launches = order_segments(segs, kInlineSegs);
+        if (launches.size() > kGradHead - 1) return cudaErrorInvalidConfiguration;
+        // the head before the sums: G (of all slabs), then a counter per launch
+        unsigned long long* counter = (unsigned long long*)wa.one.gb + 1;
+        if (s0 == 0) err = cudaMemsetAsync(wa.one.gb, 0, kGradHead * sizeof(double), st);
+        else err = cudaMemsetAsync(counter, 0, (kGradHead - 1) * sizeof(double), st);
+        if (err == cudaSuccess) err = cudaMemsetAsync(wa.one.flag, 0, sizeof(int), st);
+        if (err != cudaSuccess) return err;
+        batch_prepare_kernel<<<(unsigned)nb.prepare, 256, 0, st>>>(wa);
+        err = cudaGetLastError();
+        for (size_t c = 0; c < launches.size() && err == cudaSuccess; ++c) {
+            BatchArgs a;
+            a.segs = nullptr;
+            a.reqs = nullptr;
+            for (size_t i = 0; i < launches[c].count; ++i) a.seg[i] = segs[launches[c].first + i].d;
+            a.req = request_dev(wa.one, e);
+            err = launch_ordered(launches[c], a, counter + c, st);
+        }
     }
     if (err == cudaSuccess) {
-        batch_bias_kernel<<<(unsigned)nb.bias, 256, 0, st>>>(wa);
+        batch_bias_kernel<<<(unsigned)chunks_of(wa.one.n_nodes, kNodeChunk), 256, 0, st>>>(wa);
         err = cudaGetLastError();
     }
-    if (err == cudaSuccess && nb.entries > 0) {
-        batch_entries_kernel<<<(unsigned)nb.entries, 256, 0, st>>>(wa);
+    if (err == cudaSuccess && wa.one.n_ent > 0) {
+        batch_entries_kernel<<<(unsigned)chunks_of(wa.one.n_ent, kEntryChunk), 256, 0, st>>>(wa);
         err = cudaGetLastError();
     }
     return err;

@@ -309,19 +309,25 @@ extern "C" qts_status qts_shap_backward(qts_ensemble* e, const float* X, int64_t
         // FP32: the block tables and the batched pass's kernels
         st = ensure_blocks(e, true);
         if (st != QTS_OK) return st;
-        // The workspace holds the samples' transposed copies, so it grows with M.
-        // A stream capture must not grow it: there a call that needs more takes
-        // memory of the captured graph's own.
-        const size_t need = adjoint_work_bytes(e, M, F);
+        // The workspace holds a slab of the samples' transposed copies.  A stream
+        // capture must not grow it: there a call that needs more takes memory of
+        // the captured graph's own.
+        int64_t slab = adjoint_slab(M, F);
+        const size_t need = adjoint_work_bytes(e, slab, F);
         void* own = nullptr;
         if (need > e->work_bytes && is_capturing(s)) {
             ce = cudaMallocAsync(&own, need, s);
             if (ce != cudaSuccess) return cuda_fail(ce, "adjoint workspace");
         } else {
             st = ensure_workspace(e, need, s);
+            // a device that is nearly full: smaller slabs
+            for (int64_t k = smaller_slab(slab); st == QTS_ERR_OOM && k > 0; k = smaller_slab(k)) {
+                slab = k;
+                st = ensure_workspace(e, adjoint_work_bytes(e, slab, F), s);
+            }
             if (st != QTS_OK) return st;
         }
-        ce = launch_adjoint_blocks(e, own ? own : e->d_work, X, grad_phi, M, F, n_quad, d_leaf, d_z, s);
+        ce = launch_adjoint_blocks(e, own ? own : e->d_work, slab, X, grad_phi, M, F, n_quad, d_leaf, d_z, s);
         if (own) {
             const cudaError_t fe = cudaFreeAsync(own, s);
             if (ce == cudaSuccess) ce = fe;

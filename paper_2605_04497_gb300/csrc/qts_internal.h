@@ -286,10 +286,13 @@ cudaError_t launch_int_blocks(const qts_ensemble* e, const float* X, int64_t M, 
                               double* acc_phi, cudaStream_t st);
 cudaError_t launch_int_finalize(const double* acc_pair, const double* acc_phi, int64_t M, int F,
                                 double bias, float* out, cudaStream_t st);
-// FP32 adjoint of one request (work: adjoint_work_bytes of device memory; block
-// tables with grad)
-size_t adjoint_work_bytes(const qts_ensemble* e, int64_t M, int F);
-cudaError_t launch_adjoint_blocks(qts_ensemble* e, void* work, const float* X, const float* grad, int64_t M, int F,
-                                  int n_quad, double* d_leaf, double* d_z, cudaStream_t st);
+// FP32 adjoint of one request, `slab` samples at a time (work: adjoint_work_bytes of
+// device memory; block tables with grad).  The slab to take, and the next smaller
+// one where its workspace cannot be had (0: none).
+int64_t adjoint_slab(int64_t M, int F);
+int64_t smaller_slab(int64_t slab);
+size_t adjoint_work_bytes(const qts_ensemble* e, int64_t slab, int F);
+cudaError_t launch_adjoint_blocks(qts_ensemble* e, void* work, int64_t slab, const float* X, const float* grad,
+                                  int64_t M, int F, int n_quad, double* d_leaf, double* d_z, cudaStream_t st);
 
 }  // namespace qts

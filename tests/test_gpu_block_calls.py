@@ -171,3 +171,30 @@ def test_weights_of_the_expected_value(qts, M):
     for a, b in zip((dl, dz, it["d_leaf"], it["d_z"]), ref + ref):
         assert _rel(a.cpu().numpy(), b) <= 1e-12
     E.close()
+
+
+def test_adjoint_in_slabs_of_samples(qts):
+    """More samples than the transposed copies hold at a time (41,728 at F = 800):
+    the workspace stays bounded, and the gradients are the sum over two halves."""
+    import torch
+
+    F, M, cut = 800, 90001, 16384
+    ens = synth.grow(9900, 2, 4, F, 2000, 0.5, min_rows=3)
+    E = qts.Ensemble.from_arrays(ens)
+    gen = torch.Generator("cuda").manual_seed(9900)
+    X = torch.randn((M, F), device="cuda", generator=gen)
+    G = torch.randn((M, F + 1), device="cuda", generator=gen)
+    new = lambda: torch.empty(E.n_nodes, dtype=torch.float64, device="cuda")
+    dl, dz = new(), new()
+    a = qts.shap_backward(E, X[:cut], G[:cut])
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    qts.shap_backward(E, X, G, d_leaf=dl, d_z=dz)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] <= 280 << 20  # all samples at once: 577 MB
+    b = qts.shap_backward(E, X[cut:].contiguous(), G[cut:].contiguous())
+    E.sync_status()
+    # the cut and the slabs lie on whole tiles of samples, so only the order of FP64 sums differs
+    for got, p, q in ((dl, a[0], b[0]), (dz, a[1], b[1])):
+        assert _rel(got.cpu().numpy(), (p + q).cpu().numpy()) <= 1e-11
+    E.close()
