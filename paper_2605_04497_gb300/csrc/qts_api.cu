@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 
@@ -184,11 +185,7 @@ qts_status ensure_blocks(qts_ensemble* e, bool grad) {
     if (e->blk_ready && (!grad || e->blk_grad_ready)) return QTS_OK;
     if (grad && e->n_nodes >= ((int64_t)1 << 31)) return fail(QTS_ERR_UNSUPPORTED, "gradients of 2^31 nodes or more");
     BlockHost H;
-    try {
-        build_blocks(e, grad, &H);
-    } catch (const std::bad_alloc&) {
-        return fail(QTS_ERR_OOM, "host allocation of the block tables");
-    }
+    build_blocks(e, grad, &H);
     if (grad && H.n_slots >= ((int64_t)1 << 32)) return fail(QTS_ERR_UNSUPPORTED, "too many adjoint sums");
     BlockDev T;
     TableUpload up;
@@ -322,7 +319,7 @@ static qts_status load_impl(int32_t n_trees, const int64_t* off, const int32_t* 
                             const int32_t* right, const int32_t* feature, const float* threshold,
                             const uint8_t* default_left, const float* z, const float* leaf_value,
                             const uint8_t* is_cat, const uint64_t* cat_left, int32_t n_features,
-                            uint32_t flags, qts_ensemble** out) {
+                            uint32_t flags, qts_ensemble** out) try {
     if (!out) return fail(QTS_ERR_ARG, "out is NULL");
     *out = nullptr;
     if (n_trees < 1 || !off || !left || !right || !feature || !threshold || !z || !leaf_value)
@@ -334,8 +331,14 @@ static qts_status load_impl(int32_t n_trees, const int64_t* off, const int32_t* 
     for (int t = 0; t < n_trees; ++t)
         if (off[t + 1] <= off[t]) return fail(QTS_ERR_ARG, "tree_node_offsets must be increasing");
     if (off[0] != 0) return fail(QTS_ERR_ARG, "tree_node_offsets[0] must be 0");
-    auto* e = new (std::nothrow) qts_ensemble();
-    if (!e) return fail(QTS_ERR_OOM, "host allocation");
+    struct Drop {  // an error on the way, thrown or returned, leaves nothing behind
+        void operator()(qts_ensemble* p) const {
+            release_device(p);
+            cudaFree(p->d_status);
+            delete p;
+        }
+    };
+    std::unique_ptr<qts_ensemble, Drop> e(new qts_ensemble());
     const int64_t N = off[n_trees];
     e->n_trees = n_trees;
     e->n_features = n_features;
@@ -361,26 +364,16 @@ static qts_status load_impl(int32_t n_trees, const int64_t* off, const int32_t* 
                             e->leaf.data(), is_cat ? e->is_cat.data() : nullptr,
                             is_cat ? e->cat_left.data() : nullptr, n_features,
                             (flags & QTS_FLAG_FP64) != 0, &e->prep, &err);
-    if (st != QTS_OK) {
-        delete e;
-        return fail(st, err);
-    }
+    if (st != QTS_OK) return fail(st, err);
     cudaError_t ce = cudaMalloc(&e->d_status, sizeof(int));
     if (ce == cudaSuccess) ce = cudaMemset(e->d_status, 0, sizeof(int));
-    if (ce != cudaSuccess) {
-        delete e;
-        return cuda_fail(ce, "status word");
-    }
-    st = upload(e);
-    if (st != QTS_OK) {
-        cudaFree(e->d_status);
-        delete e;
-        return st;
-    }
+    if (ce != cudaSuccess) return cuda_fail(ce, "status word");
+    st = upload(e.get());
+    if (st != QTS_OK) return st;
     for (int D = 0; D <= kMaxD; ++D) e->tune[D] = default_tune(std::max(D, 1));
-    *out = e;
+    *out = e.release();
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 qts_status qts_load_ensemble(int32_t n_trees, const int64_t* off, const int32_t* left,
                              const int32_t* right, const int32_t* feature, const float* threshold,
@@ -399,34 +392,29 @@ qts_status qts_load_ensemble_cat(int32_t n_trees, const int64_t* off, const int3
                      is_categorical, category_left_mask, n_features, flags, out);
 }
 
-qts_status qts_update_params(qts_ensemble* e, const float* z, const float* leaf_value) {
+qts_status qts_update_params(qts_ensemble* e, const float* z, const float* leaf_value) try {
     if (!e || !z || !leaf_value) return fail(QTS_ERR_ARG, "NULL argument");
-    std::vector<float> z0 = e->z, l0 = e->leaf;
-    e->z.assign(z, z + e->n_nodes);
-    e->leaf.assign(leaf_value, leaf_value + e->n_nodes);
     Prepared P;
     std::string err;
     const bool cat = !e->is_cat.empty();
     qts_status st = prepare(e->n_trees, e->off.data(), e->left.data(), e->right.data(),
-                            e->feature.data(), e->thr.data(), e->defl.data(), e->z.data(),
-                            e->leaf.data(), cat ? e->is_cat.data() : nullptr,
+                            e->feature.data(), e->thr.data(), e->defl.data(), z, leaf_value,
+                            cat ? e->is_cat.data() : nullptr,
                             cat ? e->cat_left.data() : nullptr, e->n_features,
                             (e->flags & QTS_FLAG_FP64) != 0, &P, &err);
-    if (st != QTS_OK) {
-        e->z = z0;
-        e->leaf = l0;
-        return fail(st, err);
-    }
+    if (st != QTS_OK) return fail(st, err);
     cudaError_t ce = cudaDeviceSynchronize();
     if (ce != cudaSuccess) return cuda_fail(ce, "update sync");
     batch_forget(e);
     release_device(e);
+    e->z.assign(z, z + e->n_nodes);  // no new memory: the sizes are the same
+    e->leaf.assign(leaf_value, leaf_value + e->n_nodes);
     e->prep = std::move(P);
     return upload(e);
-}
+} QTS_ENTRY_END
 
 qts_status qts_shap_values(qts_ensemble* e, const float* X, int64_t M, int32_t F, int32_t n_quad,
-                           double* phi, qts_stream_t stream) {
+                           double* phi, qts_stream_t stream) try {
     qts_status st = check_call(e, X, M, F, n_quad);
     if (st != QTS_OK) return st;
     if (M == 0) return QTS_OK;
@@ -441,7 +429,7 @@ qts_status qts_shap_values(qts_ensemble* e, const float* X, int64_t M, int32_t F
     else if (M <= kFewRows) ce = launch_fwd_few(e, X, M, F, n_quad, phi, s);
     else ce = launch_fwd_blocks(e, X, M, F, n_quad, phi, s);
     return ce == cudaSuccess ? QTS_OK : cuda_fail(ce, "forward kernel launch");
-}
+} QTS_ENTRY_END
 
 qts_status qts_selftest_wait_timeout(qts_ensemble* e, qts_stream_t stream) {
     if (!e) return fail(QTS_ERR_ARG, "ensemble handle is NULL");
@@ -489,7 +477,7 @@ qts_status qts_get_info(const qts_ensemble* e, qts_info* out) {
 qts_status qts_describe_ensemble(int32_t n_trees, const int64_t* off, const int32_t* left,
                                  const int32_t* right, const int32_t* feature, const float* threshold,
                                  const uint8_t* default_left, const float* z, const float* leaf_value,
-                                 int32_t n_features, uint32_t flags, qts_info* out) {
+                                 int32_t n_features, uint32_t flags, qts_info* out) try {
     if (!out || n_trees < 1 || !off || !left || !right || !feature || !threshold || !z || !leaf_value)
         return fail(QTS_ERR_ARG, "NULL argument or n_trees < 1");
     if (n_features < 1 || n_features > QTS_MAX_FEATURES)
@@ -525,13 +513,13 @@ qts_status qts_describe_ensemble(int32_t n_trees, const int64_t* off, const int3
                                   P.slot_edge_begin.size() * 8 + P.edge_node.size() * 16);
     out->flags = flags;
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 qts_status qts_describe_paths(int32_t n_trees, const int64_t* off, const int32_t* left, const int32_t* right,
                               const int32_t* feature, const float* threshold, const uint8_t* default_left,
                               const float* z, const float* leaf_value, const uint8_t* is_categorical,
                               const uint64_t* category_left_mask, int32_t n_features, int64_t* n_records,
-                              int64_t* n_paths, uint32_t* records, int64_t* path_leaf, int32_t* path_width) {
+                              int64_t* n_paths, uint32_t* records, int64_t* path_leaf, int32_t* path_width) try {
     if (!n_records || !n_paths || n_trees < 1 || !off || !left || !right || !feature || !threshold || !z ||
         !leaf_value)
         return fail(QTS_ERR_ARG, "NULL argument or n_trees < 1");
@@ -557,7 +545,7 @@ qts_status qts_describe_paths(int32_t n_trees, const int64_t* off, const int32_t
     for (const Bucket& b : P.buckets)
         for (int64_t p = 0; p < b.n_paths; ++p) path_width[b.path_base + p] = b.D;
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 void qts_free(qts_ensemble* e) {
     if (!e) return;

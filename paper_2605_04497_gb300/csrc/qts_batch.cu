@@ -873,7 +873,7 @@ static qts_status check_batch(int32_t n, const qts_request* reqs, int32_t n_quad
 }  // namespace qts
 
 extern "C" qts_status qts_batched_fwd_bwd(int32_t n, const qts_request* reqs, int32_t n_quad,
-                                          qts_stream_t stream) {
+                                          qts_stream_t stream) try {
     {
         const qts_status st = check_batch(n, reqs, n_quad, (cudaStream_t)stream);
         if (st != QTS_OK) return st;
@@ -931,7 +931,7 @@ extern "C" qts_status qts_batched_fwd_bwd(int32_t n, const qts_request* reqs, in
     cudaError_t ce = cudaGraphLaunch(exec, (cudaStream_t)stream);
     if (ce != cudaSuccess) return cuda_fail(ce, "graph launch");
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 namespace qts {
 
@@ -954,7 +954,7 @@ static qts_status time_plan(int n, const qts_request* reqs, int n_quad, const Ba
 }  // namespace qts
 
 extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, int32_t n_quad, int64_t max_samples,
-                                           int32_t* chosen, qts_stream_t stream) {
+                                           int32_t* chosen, qts_stream_t stream) try {
     qts_status st = check_batch(n, reqs, n_quad, (cudaStream_t)stream);
     if (st != QTS_OK) return st;
     if (max_samples < 0) return fail(QTS_ERR_ARG, "max_samples must be >= 0");
@@ -1023,11 +1023,11 @@ extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, i
             chosen[3 * D + 2] = 0;
         }
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 extern "C" qts_status qts_get_batch_info(qts_ensemble* e, int64_t* n_paths, int64_t* sum_unique,
                                          int64_t* n_pair_paths, int32_t* n_buckets, int32_t* bucket_width,
-                                         int64_t* bucket_paths) {
+                                         int64_t* bucket_paths) try {
     if (!e) return fail(QTS_ERR_ARG, "ensemble handle is NULL");
     if (e->flags & QTS_FLAG_FP64) return fail(QTS_ERR_UNSUPPORTED, "batched calls use FP32 tables");
     const qts_status st = ensure_pair_sizes(e);
@@ -1042,7 +1042,7 @@ extern "C" qts_status qts_get_batch_info(qts_ensemble* e, int64_t* n_paths, int6
         if (bucket_paths) bucket_paths[i] = e->pair_sizes.buckets[i].n_paths;
     }
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 // Adjoint of one request by the batched kernels, without a graph (qts_shap_backward).
 // The samples go through in slabs, one after the other, so that their transposed
@@ -1122,7 +1122,7 @@ cudaError_t launch_adjoint_blocks(qts_ensemble* e, void* work, int64_t slab, con
 }  // namespace qts
 
 extern "C" qts_status qts_get_block_info(qts_ensemble* e, int64_t* n_blocks, int64_t* elements, int64_t* inner_nodes,
-                                         int64_t* pair_nodes) {
+                                         int64_t* pair_nodes) try {
     if (!e) return fail(QTS_ERR_ARG, "ensemble handle is NULL");
     const qts_status st = ensure_blocks(e, false);
     if (st != QTS_OK) return st;
@@ -1138,7 +1138,7 @@ extern "C" qts_status qts_get_block_info(qts_ensemble* e, int64_t* n_blocks, int
     if (inner_nodes) *inner_nodes = v[2];
     if (pair_nodes) *pair_nodes = v[3];
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 extern "C" int32_t qts_batched_kernel_count(void) { return g_last_batch_kernels; }
 

@@ -4,10 +4,11 @@
 #include "qts_blocks.h"
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <thread>
+
+#include "qts_threads.h"
 
 namespace qts {
 
@@ -395,13 +396,7 @@ void build_blocks(const qts_ensemble* e, bool grad, BlockHost* out) {
         while (t < e->n_trees && e->off[t] < nodes * k / nth) ++t;
         cut[k] = std::max(cut[k - 1], t);
     }
-    auto run = [&](int n, auto&& fn) {
-        std::vector<std::thread> th;
-        for (int k = 1; k < n; ++k) th.emplace_back(fn, k);
-        fn(0);
-        for (auto& x : th) x.join();
-    };
-    run(nth, [&](int k) {
+    run_threads(nth, [&](int k) {
         w[k].e = e;
         w[k].grad = grad;
         w[k].fp64 = (e->flags & QTS_FLAG_FP64) != 0;
@@ -440,7 +435,7 @@ void build_blocks(const qts_ensemble* e, bool grad, BlockHost* out) {
     if (grad) {
         out->ent.resize((size_t)n_ent);
     }
-    run(nth, [&](int k) {
+    run_threads(nth, [&](int k) {
         for (int key = 0; key < kKeys; ++key) {
             const Part& p = w[k].part[key];
             const Place& a = at[(size_t)k * kKeys + key];
@@ -464,7 +459,7 @@ void build_blocks(const qts_ensemble* e, bool grad, BlockHost* out) {
     // dE/dw_c the reach of c's parent times the expectation below c
     out->bias_leaf.assign((size_t)nodes, 0.0);
     out->bias_z.assign((size_t)nodes, 0.0);
-    run(nth, [&](int k) {
+    run_threads(nth, [&](int k) {
         std::vector<int32_t> order;
         std::vector<double> reach, below;
         for (int t = cut[k]; t < cut[k + 1]; ++t) {

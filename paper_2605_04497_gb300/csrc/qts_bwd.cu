@@ -292,7 +292,7 @@ using namespace qts;
 
 extern "C" qts_status qts_shap_backward(qts_ensemble* e, const float* X, int64_t M, int32_t F,
                                         int32_t n_quad, const float* grad_phi, double* d_leaf,
-                                        double* d_z, qts_stream_t stream) {
+                                        double* d_z, qts_stream_t stream) try {
     qts_status st = check_call(e, X, M, F, n_quad);
     if (st != QTS_OK) return st;
     if (!d_leaf || !d_z) return fail(QTS_ERR_ARG, "d_leaf and d_z must be non-NULL");
@@ -353,6 +353,6 @@ extern "C" qts_status qts_shap_backward(qts_ensemble* e, const float* X, int64_t
     ce = launch_bwd_epilogue(e, grad_phi, M, F, g_val, g_slot, d_leaf, d_z, gb, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "adjoint epilogue");
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 #endif  // QTS_HOST_PART

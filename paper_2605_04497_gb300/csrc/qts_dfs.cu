@@ -527,7 +527,7 @@ void release_dfs(qts_ensemble* e) {
 using namespace qts;
 
 extern "C" qts_status qts_shap_values_alg1(qts_ensemble* e, const float* X, int64_t M, int32_t F,
-                                           int32_t n_quad, double* phi, qts_stream_t stream) {
+                                           int32_t n_quad, double* phi, qts_stream_t stream) try {
     qts_status st = check_call(e, X, M, F, n_quad);
     if (st != QTS_OK) return st;
     if (e->flags & QTS_FLAG_FP64)
@@ -594,14 +594,14 @@ extern "C" qts_status qts_shap_values_alg1(qts_ensemble* e, const float* X, int6
     ce = cudaGetLastError();
     if (ce != cudaSuccess) return cuda_fail(ce, "depth-first kernel launch");
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 extern "C" qts_status qts_describe_alg1_program(int32_t n_trees, const int64_t* off, const int32_t* left,
                                                 const int32_t* right, const int32_t* feature,
                                                 const float* threshold, const uint8_t* default_left,
                                                 const float* z, const float* leaf_value, int32_t n_features,
                                                 int64_t* n_records, uint32_t* records, int64_t* tree_off,
-                                                int32_t* levels) {
+                                                int32_t* levels) try {
     if (!n_records || n_trees < 1 || !off || !left || !right || !feature || !threshold || !z || !leaf_value)
         return fail(QTS_ERR_ARG, "NULL argument or n_trees < 1");
     if (n_features < 1 || n_features > QTS_MAX_FEATURES)
@@ -630,4 +630,4 @@ extern "C" qts_status qts_describe_alg1_program(int32_t n_trees, const int64_t* 
     std::memcpy(tree_off, toff.data(), toff.size() * sizeof(int64_t));
     *levels = lv;
     return QTS_OK;
-}
+} QTS_ENTRY_END

@@ -452,7 +452,7 @@ cudaError_t launch_int_finalize(const double* acc_pair, const double* acc_phi, i
 using namespace qts;
 
 extern "C" qts_status qts_shap_interactions(qts_ensemble* e, const float* X, int64_t M, int32_t F,
-                                            int32_t n_quad, float* phi_ij, qts_stream_t stream) {
+                                            int32_t n_quad, float* phi_ij, qts_stream_t stream) try {
     qts_status st = check_call(e, X, M, F, n_quad);
     if (st != QTS_OK) return st;
     if (M == 0) return QTS_OK;
@@ -479,7 +479,7 @@ extern "C" qts_status qts_shap_interactions(qts_ensemble* e, const float* X, int
     ce = launch_int_finalize(acc_pair, acc_phi, M, F, e->prep.bias, phi_ij, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction finalize launch");
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 // ------------------------------------------------- allocation-free variant --
 //
@@ -559,7 +559,7 @@ static qts_status noalloc_scratch(void** out) {
 }  // namespace qts
 
 extern "C" qts_status qts_shap_interactions_noalloc(qts_ensemble* e, const float* X, int64_t M, int32_t F,
-                                                    int32_t n_quad, float* phi_ij, qts_stream_t stream) {
+                                                    int32_t n_quad, float* phi_ij, qts_stream_t stream) try {
     qts_status st = check_call(e, X, M, F, n_quad);
     if (st != QTS_OK) return st;
     if (M == 0) return QTS_OK;
@@ -593,6 +593,6 @@ extern "C" qts_status qts_shap_interactions_noalloc(qts_ensemble* e, const float
     ce = launch_int_finalize(acc_pair, acc_phi, M, F, e->prep.bias, phi_ij, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction finalize launch");
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 #endif  // QTS_HOST_PART

@@ -246,7 +246,7 @@ static cudaError_t launch_int3_bucket(const qts_ensemble* e, const Bucket& b, co
 using namespace qts;
 
 extern "C" qts_status qts_shap_interactions3(qts_ensemble* e, const float* X, int64_t M, int32_t F,
-                                             int32_t n_quad, float* sii3, qts_stream_t stream) {
+                                             int32_t n_quad, float* sii3, qts_stream_t stream) try {
     qts_status st = check_call(e, X, M, F, n_quad);
     if (st != QTS_OK) return st;
     if (M == 0) return QTS_OK;
@@ -283,6 +283,6 @@ extern "C" qts_status qts_shap_interactions3(qts_ensemble* e, const float* X, in
     ce = cudaGetLastError();
     if (ce != cudaSuccess) return cuda_fail(ce, "third-order finalize launch");
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 #endif  // QTS_HOST_PART

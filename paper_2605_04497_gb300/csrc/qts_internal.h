@@ -4,7 +4,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <exception>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -222,6 +224,12 @@ struct qts_ensemble {
 };
 
 namespace qts {
+
+// Closes the body of a C entry, written as a function try block: host memory that runs
+// out is a status, no exception leaves the library.
+#define QTS_ENTRY_END                                                                            \
+    catch (const std::bad_alloc&) { return ::qts::fail(QTS_ERR_OOM, "host memory"); }            \
+    catch (const std::exception& x) { return ::qts::fail(QTS_ERR_CUDA, x.what()); }
 
 void set_error(const std::string& msg);
 qts_status fail(qts_status st, const std::string& msg);

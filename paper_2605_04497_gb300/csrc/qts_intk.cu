@@ -323,7 +323,7 @@ using namespace qts;
 
 extern "C" qts_status qts_shap_interactions_order(qts_ensemble* e, const float* X, int64_t M, int32_t F,
                                                   int32_t order, int32_t n_quad, float* out,
-                                                  qts_stream_t stream) {
+                                                  qts_stream_t stream) try {
     qts_status st = check_call(e, X, M, F, n_quad);
     if (st != QTS_OK) return st;
     if (order < 2 || order > kIntkMaxOrder)
@@ -358,6 +358,6 @@ extern "C" qts_status qts_shap_interactions_order(qts_ensemble* e, const float* 
     ce = cudaGetLastError();
     if (ce != cudaSuccess) return cuda_fail(ce, "order-s interaction finalize launch");
     return QTS_OK;
-}
+} QTS_ENTRY_END
 
 #endif  // QTS_HOST_PART

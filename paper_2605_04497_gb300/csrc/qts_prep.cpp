@@ -7,6 +7,7 @@
 #include <thread>
 
 #include "qts_internal.h"
+#include "qts_threads.h"
 
 namespace qts {
 
@@ -476,11 +477,10 @@ qts_status prepare(int32_t n_trees, const int64_t* off, const int32_t* left, con
             while (ti < n_trees && off[ti] < target) ++ti;
             cut[k] = std::max(cut[k - 1], ti);
         }
-        std::vector<std::thread> th;
-        for (int k = 0; k < nth; ++k)
-            th.emplace_back(extract_trees, cut[k], cut[k + 1], off, left, right, feature, thr, defl,
-                            z, leaf, is_cat, cat_left, pairs, &outs[k]);
-        for (auto& x : th) x.join();
+        run_threads(nth, [&](int k) {
+            extract_trees(cut[k], cut[k + 1], off, left, right, feature, thr, defl, z, leaf, is_cat, cat_left, pairs,
+                          &outs[k]);
+        });
     }
     for (auto& o : outs)
         if (o.st != QTS_OK) { *err = o.err; return o.st; }

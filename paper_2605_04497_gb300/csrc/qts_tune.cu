@@ -92,7 +92,7 @@ static float time_ms(F&& fn, cudaStream_t st, int reps) {
 using namespace qts;
 
 extern "C" qts_status qts_autotune(qts_ensemble* e, const float* X, int64_t M, int32_t F,
-                                   const char* cache_path, qts_stream_t stream) {
+                                   const char* cache_path, qts_stream_t stream) try {
     qts_status st = check_call(e, X, M, F, 8);
     if (st != QTS_OK) return st;
     if (M == 0) return QTS_OK;
@@ -137,4 +137,4 @@ extern "C" qts_status qts_autotune(qts_ensemble* e, const float* X, int64_t M, i
     batch_forget(e);
     if (cache_path) write_cache(cache_path, cache);
     return QTS_OK;
-}
+} QTS_ENTRY_END
