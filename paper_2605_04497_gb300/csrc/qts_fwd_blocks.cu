@@ -239,6 +239,13 @@ cudaError_t launch_phi_init(double* phi, int64_t M, int F, double bias, cudaStre
     return cudaGetLastError();
 }
 
+// Work per thread block (units of blk_cost) below which zeroing, loading and flushing the
+// tiles, rows of 32 samples for each feature, weighs too much beside the blocks.  With the
+// factor 200, 100 trees of depth 8 on 2,000 samples: F = 100 345 -> 305 us, 200 561 -> 433,
+// 400 1,118 -> 694, 784 3,527 -> 1,531 (100: 345, 516, 804, 1,783; 400: 256, 444, 658,
+// 1,423, but 33 samples of 20 trees of depth 14 180 -> 205).
+static double fb_least(int F) { return 200.0 * (F + 40); }
+
 cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* phi,
                               cudaStream_t st) {
     if (M <= 0) return cudaSuccess;
@@ -296,10 +303,14 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
                 ctas = 0;
                 return r;
             };
-            // work per thread block: about eight rounds of the whole chip, at
-            // most what keeps the tile set-up and flush small beside it
-            const double share = e->tune[0].bpaths > 0 ? kBlkUnit * e->tune[0].bpaths
-                                                       : std::min(400e3, std::max(4e3, total / (8.0 * num_sms() * 4)));
+            // work per thread block: about eight rounds of the whole chip, and what
+            // keeps the tiles' set-up and flush small beside it as far as that leaves
+            // two rounds of the thread blocks that fit
+            const int resident = std::min(cls <= 3 ? 4 : 2, std::max(1, (int)(kSmemMax / (smem + 1024))));
+            const double wide = std::min(fb_least(F), total / (2.0 * num_sms() * resident));
+            const double share = e->tune[0].bpaths > 0
+                                     ? kBlkUnit * e->tune[0].bpaths
+                                     : std::min(400e3, std::max({4e3, wide, total / (8.0 * num_sms() * 4)}));
             for (const BlockBucket* b : pick) {
                 if (a.n_seg == kFbSegs) {
                     const cudaError_t r = flush();
