@@ -25,7 +25,6 @@
 
 namespace qts {
 
-constexpr int kFbSegs = 40;
 constexpr int kFbWarps = 4;
 
 struct FbSeg {
@@ -260,16 +259,25 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
             a.n_seg = 0;
             int64_t ctas = 0;
             int stage = 0;
-            std::vector<const BlockBucket*> pick;
+            const BlockBucket* pick[kFbSegs];
+            int n_pick = 0;
             for (const BlockBucket& b : e->blk)
-                if (fb_class(b.D) == cls && nodes_for(n_quad, b.dmax, 1) == nq) pick.push_back(&b);
-            if (pick.empty()) continue;
+                if (fb_class(b.D) == cls && nodes_for(n_quad, b.dmax, 1) == nq) {
+                    if (n_pick == kFbSegs) return cudaErrorInvalidValue;
+                    pick[n_pick++] = &b;
+                }
+            if (n_pick == 0) continue;
             if (!make_quad(nq, &a.q, nullptr, 2)) return cudaErrorInvalidValue;
             const int np = fb_np(cls, a.q.n_pad);
-            std::sort(pick.begin(), pick.end(),
+            if (fwd_own_wins(pick, n_pick, M, F)) {
+                const cudaError_t r = launch_fwd_own(e, X, M, F, cls, nq, np, pick, n_pick, phi, st);
+                if (r != cudaSuccess) return r;
+                continue;
+            }
+            std::sort(pick, pick + n_pick,
                       [](const BlockBucket* x, const BlockBucket* y) { return blk_cost(x->D, x->h) > blk_cost(y->D, y->h); });
             int max_stride = 0;
-            for (const BlockBucket* b : pick) max_stride = std::max(max_stride, blk_stride(b->D, b->h));
+            for (int k = 0; k < n_pick; ++k) max_stride = std::max(max_stride, blk_stride(pick[k]->D, pick[k]->h));
             // tiles of phi: one per warp while that leaves two thread blocks per SM,
             // then a shared one with atomics.  Blocks staged at a time: the most
             // that keeps four thread blocks per SM (a staged sub-chunk ends on a
@@ -290,19 +298,6 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
             a.M = M;
             a.phi = phi;
             a.status = e->d_status;
-            auto flush = [&]() -> cudaError_t {
-                if (a.n_seg == 0) return cudaSuccess;
-                if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-                cudaError_t r = cudaErrorInvalidValue;
-#define QTS_GO(C, N) \
-    if (cls == C && np == N) r = launch_fb<C, N>(a, ctas, smem, st);
-                QTS_GO(0, 8) QTS_GO(0, 4) QTS_GO(0, 2) QTS_GO(1, 4) QTS_GO(1, 2) QTS_GO(2, 2)
-                QTS_GO(3, 2) QTS_GO(4, 2)
-#undef QTS_GO
-                a.n_seg = 0;
-                ctas = 0;
-                return r;
-            };
             // work per thread block: about eight rounds of the whole chip, and what
             // keeps the tiles' set-up and flush small beside it as far as that leaves
             // two rounds of the thread blocks that fit
@@ -311,11 +306,8 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
             const double share = e->tune[0].bpaths > 0
                                      ? kBlkUnit * e->tune[0].bpaths
                                      : std::min(400e3, std::max({4e3, wide, total / (8.0 * num_sms() * 4)}));
-            for (const BlockBucket* b : pick) {
-                if (a.n_seg == kFbSegs) {
-                    const cudaError_t r = flush();
-                    if (r != cudaSuccess) return r;
-                }
+            for (int k = 0; k < n_pick; ++k) {
+                const BlockBucket* b = pick[k];
                 FbSeg& sg = a.seg[a.n_seg++];
                 sg.rec = e->blkdev.rec + b->rec_off;
                 sg.n = b->n;
@@ -326,7 +318,13 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
                 sg.per_cta = (int32_t)((per + kFbWarps - 1) / kFbWarps * kFbWarps);
                 ctas += (b->n + sg.per_cta - 1) / sg.per_cta * tiles;
             }
-            const cudaError_t r = flush();
+            if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+            cudaError_t r = cudaErrorInvalidValue;
+#define QTS_GO(C, N) \
+    if (cls == C && np == N) r = launch_fb<C, N>(a, ctas, smem, st);
+            QTS_GO(0, 8) QTS_GO(0, 4) QTS_GO(0, 2) QTS_GO(1, 4) QTS_GO(1, 2) QTS_GO(2, 2)
+            QTS_GO(3, 2) QTS_GO(4, 2)
+#undef QTS_GO
             if (r != cudaSuccess) return r;
         }
     }

@@ -198,3 +198,33 @@ def test_adjoint_in_slabs_of_samples(qts):
     for got, p, q in ((dl, a[0], b[0]), (dz, a[1], b[1])):
         assert _rel(got.cpu().numpy(), (p + q).cpu().numpy()) <= 1e-11
     E.close()
+
+
+@pytest.mark.parametrize("T,depth,F,M", [(1, 1, 1, 20000), (1, 2, 3, 19999), (3, 6, 12, 20001), (1, 10, 40, 40033),
+                                         (2, 14, 9, 40000), (0, 41, 50, 40031)])
+@pytest.mark.parametrize("missing", [False, True])
+def test_small_ensemble_many_samples(qts, T, depth, F, M, missing):
+    """A warp walks all blocks for its samples (every class of widths, whole and
+    ragged tiles, clean tiles beside tiles with NaN and +inf); 0 trees: a chain."""
+    import torch
+
+    from helpers import caterpillar_ensemble
+
+    ens = (synth.grow(9850 + depth, T, depth, F, 3000, 0.5, min_rows=3) if T else
+           caterpillar_ensemble(9850, [depth, 20, 9], F))
+    X = synth.normal(9850 + depth, synth.STREAM_X, (M, F))
+    r = np.random.default_rng(9850)
+    rows = np.unique(np.concatenate([np.arange(40), M - 1 - np.arange(40), r.integers(0, M, 60)]))
+    if missing:
+        X[::3][r.random(X[::3].shape) < 0.2] = np.nan
+        X[64:96] = np.abs(X[64:96])
+    ref = oracle.shap_exact(ens, np.ascontiguousarray(X[rows]))
+    E = qts.Ensemble.from_arrays(ens)
+    Xd = torch.from_numpy(X).cuda()
+    few = qts.shap_values(E, Xd[:16], qts.EXACT_NODES)  # another kernel
+    for n_quad in (qts.EXACT_NODES,) + ((8, 11) if T else (21,)):
+        phi = qts.shap_values(E, Xd, n_quad)
+        E.sync_status()
+        assert rel_err_rows(phi[torch.from_numpy(rows).cuda()].cpu().numpy(), ref).max() <= TOL32, n_quad
+        assert rel_err_rows(phi[:16].cpu().numpy(), few.cpu().numpy()).max() <= TOL32
+    E.close()
