@@ -205,8 +205,10 @@ qts_status qts_shap_values_alg1(qts_ensemble *ens, const float *X, int64_t M, in
  *           [s][F][F] = E[f], other entries of row/column F are 0.
  * Cross-tree accumulation is FP64 in the ensemble's workspace (device memory
  * of M * (F(F+1)/2) doubles, grown on demand with cudaMalloc).  Runs on the
- * block tables of qts_shap_values (built by the first call that needs them); under
- * capture the workspace must have been grown before, by a call of the same size.
+ * block tables of qts_shap_values (built by the first call that needs them), or on
+ * path tables with sibling leaves merged where F is too large for a pair tile in
+ * shared memory (above about 50); under capture the workspace must have been grown
+ * before, by a call of the same size.
  * n_quad as qts_shap_values;
  * QTS_NQ_EXACT takes the first-order count ceil(w / 2) of a bucket's widest path
  * w (the pair terms need ceil((w - 1) / 2), the diagonal's first-order values

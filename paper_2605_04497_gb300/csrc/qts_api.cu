@@ -70,6 +70,8 @@ void release_device(qts_ensemble* e) {
     e->d_empty_leaf = nullptr;
     e->device_bytes = 0;
     release_dfs(e);
+    cudaFree(e->d_pair_rec);
+    e->d_pair_rec = nullptr;
     e->pair_ready = false;
     release_blocks(e);
 }
@@ -120,26 +122,6 @@ qts_status upload(qts_ensemble* e) {
     return QTS_OK;
 }
 
-// Sizes of the path tables with sibling leaves merged (qts_get_batch_info): prepared
-// from the host copy of the model, nothing is kept but the counts.
-qts_status ensure_pair_sizes(qts_ensemble* e) {
-    if (e->pair_ready) return QTS_OK;
-    Prepared P;
-    std::string err;
-    const bool cat = !e->is_cat.empty();
-    qts_status st = prepare(e->n_trees, e->off.data(), e->left.data(), e->right.data(), e->feature.data(),
-                            e->thr.data(), e->defl.data(), e->z.data(), e->leaf.data(),
-                            cat ? e->is_cat.data() : nullptr, cat ? e->cat_left.data() : nullptr,
-                            e->n_features, false, &P, &err, true);
-    if (st != QTS_OK) return fail(st, err);
-    e->pair_sizes.buckets = P.buckets;
-    e->pair_sizes.n_paths = P.n_paths;
-    e->pair_sizes.sum_unique = P.sum_unique;
-    e->pair_sizes.n_pair_paths = P.n_pair_paths;
-    e->pair_ready = true;
-    return QTS_OK;
-}
-
 static void free_blocks(BlockDev& T) {
     for (void* p : {(void*)T.rec, (void*)T.dbl, (void*)T.ent, (void*)T.bias_leaf, (void*)T.bias_z}) cudaFree(p);
     T = BlockDev();
@@ -176,6 +158,41 @@ struct TableUpload {
         return err;
     }
 };
+
+// The path tables with sibling leaves merged: prepared from the host copy of the model;
+// on the host only their counts are kept.
+qts_status ensure_pairs(qts_ensemble* e, bool records) {
+    std::lock_guard<std::mutex> lk(e->blk_mu);
+    if (e->pair_ready && (!records || e->d_pair_rec)) return QTS_OK;
+    Prepared P;
+    std::string err;
+    const bool cat = !e->is_cat.empty();
+    qts_status st = prepare(e->n_trees, e->off.data(), e->left.data(), e->right.data(), e->feature.data(),
+                            e->thr.data(), e->defl.data(), e->z.data(), e->leaf.data(),
+                            cat ? e->is_cat.data() : nullptr, cat ? e->cat_left.data() : nullptr,
+                            e->n_features, false, &P, &err, true);
+    if (st != QTS_OK) return fail(st, err);
+    if (records) {
+        Rec32* rec = nullptr;
+        TableUpload up;
+        up.add(&rec, P.rec32);
+        const cudaError_t ce = up.finish();
+        if (ce != cudaSuccess) {
+            if (ce == cudaErrorMemoryAllocation) cudaGetLastError();
+            cudaFree(rec);
+            return cuda_fail(ce, "upload pair tables");
+        }
+        e->d_pair_rec = rec;
+    }
+    if (!e->pair_ready) {
+        e->pair_sizes.buckets = P.buckets;
+        e->pair_sizes.n_paths = P.n_paths;
+        e->pair_sizes.sum_unique = P.sum_unique;
+        e->pair_sizes.n_pair_paths = P.n_pair_paths;
+        e->pair_ready = true;
+    }
+    return QTS_OK;
+}
 
 // Block tables: built from the host copy of the model; `grad` adds the adjoint's
 // part.  The records are the same either way: once they are there nothing that a

@@ -1030,7 +1030,7 @@ extern "C" qts_status qts_get_batch_info(qts_ensemble* e, int64_t* n_paths, int6
                                          int64_t* bucket_paths) try {
     if (!e) return fail(QTS_ERR_ARG, "ensemble handle is NULL");
     if (e->flags & QTS_FLAG_FP64) return fail(QTS_ERR_UNSUPPORTED, "batched calls use FP32 tables");
-    const qts_status st = ensure_pair_sizes(e);
+    const qts_status st = ensure_pairs(e, false);
     if (st != QTS_OK) return st;
     if (n_paths) *n_paths = e->pair_sizes.n_paths;
     if (sum_unique) *sum_unique = e->pair_sizes.sum_unique;

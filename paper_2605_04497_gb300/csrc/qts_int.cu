@@ -1,8 +1,8 @@
 // Pairwise Shapley interaction values (Thm 1 with S = {i, j}; Alg. 1 with
 // s = 2), in the pred_interactions layout: the entry points, the finalize kernel,
-// and the path kernels of the allocation-free call.  qts_shap_interactions runs on
-// the block tables (qts_int_blocks.cu), which are built and allocated on first use;
-// the allocation-free call must not do that and keeps the per-leaf path tables.
+// and the kernels on path tables.  qts_shap_interactions runs on the block tables
+// (qts_int_blocks.cu), or here with sibling leaves merged (pairs_on_paths); the
+// allocation-free call may not build tables and runs here on the per-leaf ones.
 //
 // For a path with merged elements sorted by feature and a sample,
 //     SII_ij += val d_i d_j sum_m w_m prod_{k != i,j} a_k(t_m),   d = o - z,
@@ -21,7 +21,7 @@
 // launch per width of 512 paths per thread block left most SMs idle on narrow
 // widths; 500 trees of depth 6, 2,000 samples: 1.79 -> 1.56 ms).
 //
-// qts-build-parts: 6 (part 0: host code; parts 1-5: the kernels)
+// qts-build-parts: 7 (part 0: host code; parts 1-6: the kernels)
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -73,14 +73,29 @@ struct IntArgs {
 // the widest register pass a width takes (nodes per pass)
 __host__ __device__ constexpr int int_max_np(int D) { return D <= 6 ? 8 : (D <= 12 ? 4 : 2); }
 
-// launch classes: widths up to 4, 6, 12, 16 and the padded ones above
-__host__ __device__ constexpr int int_class(int D) { return D <= 4 ? 0 : D <= 6 ? 1 : D <= 12 ? 2 : D <= 16 ? 3 : 4; }
-[[maybe_unused]] constexpr int kIntClasses = 5;
+// launch classes: widths up to 4, 6, 8, 12, 16 and the padded ones above (7 and 8 with
+// 9 to 12 held 155 registers instead of 109: 100 trees of depth 8, F = 56,
+// 2,000 samples 2,879 instead of 2,260 us)
+__host__ __device__ constexpr int int_class(int D) {
+    return D <= 4 ? 0 : D <= 6 ? 1 : D <= 8 ? 2 : D <= 12 ? 3 : D <= 16 ? 4 : 5;
+}
+[[maybe_unused]] constexpr int kIntClasses = 6;
 
 template <int CLS>
 cudaError_t launch_int_c(const IntArgs& a, int np, bool pair_smem, int64_t blocks, size_t smem, cudaStream_t st);
 
 #if QTS_DEVICE_PARTS
+
+// d of a sibling pair's element (Rec32): the leaf that x reaches, or neither
+template <bool HAS_NAN>
+__device__ __forceinline__ float pair_d(float x, const Rec32& e, const Rec32& head) {
+    bool in = x >= e.lo && x < e.hi, left = x < __uint_as_float(head.bits);
+    if (HAS_NAN && x != x) {
+        in = (e.bits & kNanOk) != 0;
+        left = (e.bits & kDefLeft) != 0;
+    }
+    return !in ? -e.z : left ? head.lo : head.hi;
+}
 
 // PAIR_SMEM: pair sums go to a shared tile [n_pairs][33]; otherwise straight to
 // the FP64 accumulator (lanes = consecutive samples, so each add is coalesced).
@@ -90,6 +105,10 @@ __device__ __forceinline__ void int_path_f32(const Rec32* __restrict__ r, const 
                                              int64_t M, int lane, int F, const QuadF& q) {
     constexpr int K = NP / 2;
     const float val = r[0].z;
+    // a sibling pair (tables that merge them; they serve only calls without a pair
+    // tile): its element sits last, after the padding and out of feature order,
+    // and its two-leaf polynomial is one more linear factor of every term (val = 1)
+    const bool pair = !PAIR_SMEM && (r[D].bits & kPairElem) != 0;
     float dd[D], c1[D];
     int nreal = D;  // sorted elements before the padding (padding sorts last)
 #pragma unroll
@@ -99,9 +118,11 @@ __device__ __forceinline__ void int_path_f32(const Rec32* __restrict__ r, const 
         const float x = xs[f * kTileLd + lane];
         const bool o = satisfies<HAS_NAN>(x, e.lo, e.hi, e.bits);
         dd[j] = (o ? 1.f : 0.f) - e.z;
+        if (j == D - 1 && pair) dd[j] = pair_d<HAS_NAN>(x, e, r[0]);
         c1[j] = 0.f;
         if (f >= F && j < nreal) nreal = j;
     }
+    if (pair && nreal > D - 1) nreal = D - 1;
     const int npass = q.n_pad / NP;
     for (int pass = 0; pass < npass; ++pass) {
         float2 T[K], A[D][K], P[D][K], S[D][K];
@@ -137,7 +158,7 @@ __device__ __forceinline__ void int_path_f32(const Rec32* __restrict__ r, const 
         // pairs i < j
 #pragma unroll
         for (int i = 0; i < D - 1; ++i) {
-            if (i + 1 >= nreal) break;
+            if (i + (pair ? 0 : 1) >= nreal) break;
             const int fi = feat_of(r[1 + i].bits);
             const int64_t rowbase = tri_index(fi, fi + 1, F) - (fi + 1);  // + fj gives the index
             float2 R[K];
@@ -161,11 +182,22 @@ __device__ __forceinline__ void int_path_f32(const Rec32* __restrict__ r, const 
                     if (s < M && v != 0.f) atomicAdd(&acc_pair[idx * M + s], (double)v);
                 }
             }
+            if (!PAIR_SMEM && pair) {
+                // R spans the elements between i and the pair's (padding's factors are
+                // 1), whose suffix is 1
+                float2 acc = R[0];
+#pragma unroll
+                for (int k = 1; k < K; ++k) acc = add2(R[k], acc);
+                const float v = (acc.x + acc.y) * (dd[i] * dd[D - 1]);
+                const int fp = feat_of(r[D].bits);
+                const int64_t idx = tri_index(min(fi, fp), max(fi, fp), F);
+                if (s < M && v != 0.f) atomicAdd(&acc_pair[idx * M + s], (double)v);
+            }
         }
     }
 #pragma unroll
     for (int j = 0; j < D; ++j)
-        if (j < nreal)
+        if (j < nreal || (pair && j == D - 1))
             atomicAdd(&ps[feat_of(r[1 + j].bits) * kTileLd + lane], dd[j] * c1[j]);
 }
 
@@ -250,10 +282,15 @@ __global__ void __launch_bounds__(kIntWarps * 32) int_kernel(const __grid_consta
         }
     } else if constexpr (CLS == 2) {
         switch (sg.D) {
-            QTS_CASE(7) QTS_CASE(8) QTS_CASE(9) QTS_CASE(10) QTS_CASE(11) QTS_CASE(12)
+            QTS_CASE(7) QTS_CASE(8)
             default: break;
         }
     } else if constexpr (CLS == 3) {
+        switch (sg.D) {
+            QTS_CASE(9) QTS_CASE(10) QTS_CASE(11) QTS_CASE(12)
+            default: break;
+        }
+    } else if constexpr (CLS == 4) {
         switch (sg.D) {
             QTS_CASE(13) QTS_CASE(14) QTS_CASE(15) QTS_CASE(16)
             default: break;
@@ -298,7 +335,7 @@ static cudaError_t launch_int_t(const IntArgs& a, int64_t blocks, size_t smem, c
 // up to 6 (a rule of four points)
 template <int CLS>
 cudaError_t launch_int_c(const IntArgs& a, int np, bool pair_smem, int64_t blocks, size_t smem, cudaStream_t st) {
-    constexpr int NP = CLS <= 1 ? 8 : CLS == 2 ? 4 : 2;
+    constexpr int NP = CLS <= 1 ? 8 : CLS <= 3 ? 4 : 2;
     if constexpr (NP == 8) {
         if (np < NP) {
             if (pair_smem) return launch_int_t<CLS, NP / 2, true>(a, blocks, smem, st);
@@ -306,6 +343,11 @@ cudaError_t launch_int_c(const IntArgs& a, int np, bool pair_smem, int64_t block
         }
     }
     if (pair_smem) return launch_int_t<CLS, NP, true>(a, blocks, smem, st);
+    if constexpr (CLS == 2) {
+        // adds to global memory bound these: one pass over all nodes halves them (100
+        // trees of depth 8, F = 56, 2,000 samples 2,260 -> 1,913 us)
+        if (a.q.n_pad % 8 == 0) return launch_int_t<CLS, 8, false>(a, blocks, smem, st);
+    }
     return launch_int_t<CLS, NP, false>(a, blocks, smem, st);
 }
 
@@ -324,6 +366,9 @@ QTS_INST(3)
 #endif
 #if QTS_IN_PART(5)
 QTS_INST(4)
+#endif
+#if QTS_IN_PART(6)
+QTS_INST(5)
 #endif
 #undef QTS_INST
 
@@ -372,69 +417,78 @@ __global__ void int_finalize_kernel(const double* __restrict__ acc_pair, const d
 
 static constexpr size_t kSmemBudget = 200 * 1024;
 
-// Pairwise sums of every bucket of the per-leaf tables with a rule of nq points.
-static cudaError_t launch_int_buckets(const qts_ensemble* e, const float* X, int64_t M, int F, int nq,
-                                      double* acc_pair, double* acc_phi, cudaStream_t st) {
+// Pairwise sums of every bucket of the path tables, one path per leaf or (F too large for a
+// pair tile) with sibling leaves merged (QTS_NQ_EXACT: the first-order
+// count per bucket, because the diagonal holds first-order values).
+static cudaError_t launch_int_buckets(const qts_ensemble* e, const Rec32* rec, const std::vector<Bucket>& buckets,
+                                      const float* X, int64_t M, int F, int n_quad, double* acc_pair, double* acc_phi,
+                                      cudaStream_t st) {
     if (M <= 0) return cudaSuccess;
-    const Prepared& P = e->prep;
-    const Rec32* rec = (const Rec32*)e->d_rec;
     const int64_t tiles = (M + 31) / 32;
     const int group = M <= kFewRows ? (int)(32 / M) : 0;
     // work per thread block: about eight rounds of the whole chip (three thread
-    // blocks per SM); at least what makes the pair tile's set-up and flush, F^2 / 2
-    // rows, small beside the paths'
+    // blocks per SM); at least what makes the set-up and flush of the tiles, F^2 / 2 rows
+    // where the pair tile fits and F where not, small beside the paths'
     double total = 0.0;
-    for (const Bucket& b : P.buckets) total += (double)b.n_paths * b.D * (b.D + 8);
-    const double least = std::min(512.0, 64.0 + (double)F * F / 8.0) * 60.0;
+    for (const Bucket& b : buckets) total += (double)b.n_paths * b.D * (b.D + 8);
+    const bool tile = int_smem_bytes(F, 16 * 17, true) <= kSmemBudget;
+    const double least = std::min(512.0, 64.0 + (tile ? (double)F * F / 8.0 : F / 2.0)) * 60.0;
     const double share = std::max(least, std::min(512.0 * 84.0, total * (double)tiles / (8.0 * 3 * num_sms())));
     for (int cls = 0; cls < kIntClasses; ++cls) {
-        IntArgs a;
-        a.n_seg = 0;
-        int64_t ctas = 0;
-        int max_d = 0;
-        // widest first: its thread blocks are the longest
-        for (auto it = P.buckets.rbegin(); it != P.buckets.rend(); ++it) {
-            const Bucket& b = *it;
-            if (b.n_paths == 0 || int_class(b.D) != cls) continue;
-            max_d = std::max(max_d, b.D);
-            int64_t per = std::max<int64_t>(16, (int64_t)(share / (b.D * (b.D + 8))));
-            if (group) per = std::max<int64_t>(per, 4LL * kIntWarps * group);
-            per = std::min<int64_t>((per + 15) / 16 * 16, 1 << 20);
-            a.seg[a.n_seg++] = {rec + b.rec_off, b.n_paths, ctas, (int32_t)per, b.D};
-            ctas += (b.n_paths + per - 1) / per * tiles;
+        uint64_t rules = 0;  // bit q: some bucket of the class takes q points
+        for (const Bucket& b : buckets)
+            if (b.n_paths > 0 && int_class(b.D) == cls) rules |= (uint64_t)1 << nodes_for(n_quad, b.D, 1);
+        for (int nq = QTS_MAX_QUAD; nq >= 1; --nq) {  // one launch per rule
+            if (!((rules >> nq) & 1)) continue;
+            IntArgs a;
+            a.n_seg = 0;
+            int64_t ctas = 0;
+            int max_d = 0;
+            // widest first: its thread blocks are the longest
+            for (auto it = buckets.rbegin(); it != buckets.rend(); ++it) {
+                const Bucket& b = *it;
+                if (b.n_paths == 0 || int_class(b.D) != cls || nodes_for(n_quad, b.D, 1) != nq) continue;
+                max_d = std::max(max_d, b.D);
+                int64_t per = std::max<int64_t>(16, (int64_t)(share / (b.D * (b.D + 8))));
+                if (group) per = std::max<int64_t>(per, 4LL * kIntWarps * group);
+                per = std::min<int64_t>((per + 15) / 16 * 16, 1 << 20);
+                a.seg[a.n_seg++] = {rec + b.rec_off, b.n_paths, ctas, (int32_t)per, b.D};
+                ctas += (b.n_paths + per - 1) / per * tiles;
+            }
+            if (a.n_seg == 0) continue;
+            if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+            // the rule, padded to 4 nodes up to width 12 (a pass of 4 or 8 nodes) and to
+            // 2 above
+            if (!make_quad(nq, &a.q, nullptr, cls <= 3 ? 4 : 2)) return cudaErrorInvalidValue;
+            a.sub = max_d <= 16 ? 16 : 8;
+            // wide inputs: stage fewer paths at a time until the block fits shared memory
+            while (a.sub > 1 && int_smem_bytes(F, a.sub * (max_d + 1), false) > kSmemMax) a.sub /= 2;
+            a.stage = a.sub * (max_d + 1);
+            a.n_tiles = (int)tiles;
+            a.X = X;
+            a.M = M;
+            a.F = F;
+            a.cat = e->prep.has_cat ? 1 : 0;
+            a.n_pairs = (int64_t)F * (F - 1) / 2;
+            a.group = group;
+            a.acc_pair = acc_pair;
+            a.acc_phi = acc_phi;
+            a.status = e->d_status;
+            const bool pair_smem = int_smem_bytes(F, a.stage, true) <= kSmemBudget;
+            const size_t smem = int_smem_bytes(F, a.stage, pair_smem);
+            if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
+            // nodes per register pass: the class's widest, or half of it when that
+            // does not divide the rule's padded node count
+            const int np = a.q.n_pad % int_max_np(max_d) == 0 ? int_max_np(max_d) : int_max_np(max_d) / 2;
+            if (a.q.n_pad % np != 0) return cudaErrorInvalidValue;
+            const cudaError_t r = cls == 0   ? launch_int_c<0>(a, np, pair_smem, ctas, smem, st)
+                                  : cls == 1 ? launch_int_c<1>(a, np, pair_smem, ctas, smem, st)
+                                  : cls == 2 ? launch_int_c<2>(a, np, pair_smem, ctas, smem, st)
+                                  : cls == 3 ? launch_int_c<3>(a, np, pair_smem, ctas, smem, st)
+                                  : cls == 4 ? launch_int_c<4>(a, np, pair_smem, ctas, smem, st)
+                                             : launch_int_c<5>(a, np, pair_smem, ctas, smem, st);
+            if (r != cudaSuccess) return r;
         }
-        if (a.n_seg == 0) continue;
-        if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-        // the rule, padded to 4 nodes up to width 12 (a pass of 4 or 8 nodes) and to
-        // 2 above
-        if (!make_quad(nq, &a.q, nullptr, cls <= 2 ? 4 : 2)) return cudaErrorInvalidValue;
-        a.sub = max_d <= 16 ? 16 : 8;
-        // wide inputs: stage fewer paths at a time until the block fits shared memory
-        while (a.sub > 1 && int_smem_bytes(F, a.sub * (max_d + 1), false) > kSmemMax) a.sub /= 2;
-        a.stage = a.sub * (max_d + 1);
-        a.n_tiles = (int)tiles;
-        a.X = X;
-        a.M = M;
-        a.F = F;
-        a.cat = P.has_cat ? 1 : 0;
-        a.n_pairs = (int64_t)F * (F - 1) / 2;
-        a.group = group;
-        a.acc_pair = acc_pair;
-        a.acc_phi = acc_phi;
-        a.status = e->d_status;
-        const bool pair_smem = int_smem_bytes(F, a.stage, true) <= kSmemBudget;
-        const size_t smem = int_smem_bytes(F, a.stage, pair_smem);
-        if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
-        // nodes per register pass: the class's widest, or half of it when that
-        // does not divide the rule's padded node count
-        const int np = a.q.n_pad % int_max_np(max_d) == 0 ? int_max_np(max_d) : int_max_np(max_d) / 2;
-        if (a.q.n_pad % np != 0) return cudaErrorInvalidValue;
-        const cudaError_t r = cls == 0   ? launch_int_c<0>(a, np, pair_smem, ctas, smem, st)
-                              : cls == 1 ? launch_int_c<1>(a, np, pair_smem, ctas, smem, st)
-                              : cls == 2 ? launch_int_c<2>(a, np, pair_smem, ctas, smem, st)
-                              : cls == 3 ? launch_int_c<3>(a, np, pair_smem, ctas, smem, st)
-                                         : launch_int_c<4>(a, np, pair_smem, ctas, smem, st);
-        if (r != cudaSuccess) return r;
     }
     return cudaSuccess;
 }
@@ -445,6 +499,27 @@ cudaError_t launch_int_finalize(const double* acc_pair, const double* acc_phi, i
     const int blocks = (int)std::min<int64_t>((n + 255) / 256, 8 * 152);
     int_finalize_kernel<<<blocks, 256, 0, st>>>(acc_pair, acc_phi, M, F, bias, out);
     return cudaGetLastError();
+}
+
+}  // namespace qts
+
+namespace qts {
+
+// Which tables a pairwise call runs on: the blocks, or, where F is too large for a pair
+// tile in shared memory, the path tables with sibling leaves merged.  Without a tile every
+// add goes to global memory: a block needs fewer of them, but keeps more vectors than
+// fit its registers and has fewer warps in flight.  Blocks and paths: 100 trees of depth 8,
+// F = 56, 300 samples 1,314 and 428 us, 2,000 4,064 and 1,913, 6,000 9,969 and 5,454 (one
+// launch per width: 2,213, 2,679 and 6,381); F = 200, 2,000 samples 8,060 and 3,033; 300
+// trees of depth 4, F = 56, 2,000 samples 455 and 164; one row of 8 trees of depth 14, F
+// = 60 512 and 440, but of 2 trees of depth 18 731 and 872, F = 400 913 and 1,894.  The
+// paths' error against FP64 is the smaller one there (100 trees of depth 8, F = 60:
+// 1.0e-7 against 1.3e-7).  With a tile the blocks stay, also where the per-leaf paths are
+// faster (mean width above 9.5: F = 24, depth 14, 640 samples 11.2 ms against 6.5), because
+// there the blocks' error is smaller (1.8e-7 against 2.1e-7).
+static bool pairs_on_paths(const qts_ensemble* e, int64_t M, int F) {
+    if (int_smem_bytes(F, 16 * 17, true) <= kSmemBudget) return false;
+    return M > 1 || (double)e->prep.sum_unique <= 13.5 * (double)e->prep.n_paths;
 }
 
 }  // namespace qts
@@ -463,8 +538,9 @@ extern "C" qts_status qts_shap_interactions(qts_ensemble* e, const float* X, int
         return fail(QTS_ERR_UNSUPPORTED, "interactions support paths of at most 32 unique features");
     cudaStream_t s = (cudaStream_t)stream;
     if (n_quad != QTS_NQ_EXACT && (n_quad < 1 || n_quad > QTS_MAX_QUAD)) return fail(QTS_ERR_ARG, "quadrature rule");
-    // the block tables (built on the first call that needs them)
-    st = ensure_blocks(e, false);
+    const bool paths = pairs_on_paths(e, M, F);
+    // the tables (built on the first call that needs them)
+    st = paths ? ensure_pairs(e, true) : ensure_blocks(e, false);
     if (st != QTS_OK) return st;
     const int64_t n_pairs = (int64_t)F * (F - 1) / 2;
     const size_t bytes = sizeof(double) * (size_t)((n_pairs + F) * M);
@@ -474,7 +550,8 @@ extern "C" qts_status qts_shap_interactions(qts_ensemble* e, const float* X, int
     double* acc_phi = acc_pair + n_pairs * M;
     cudaError_t ce = cudaMemsetAsync(e->d_work, 0, bytes, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "workspace clear");
-    ce = launch_int_blocks(e, X, M, F, n_quad, acc_pair, acc_phi, s);
+    ce = paths ? launch_int_buckets(e, e->d_pair_rec, e->pair_sizes.buckets, X, M, F, n_quad, acc_pair, acc_phi, s)
+               : launch_int_blocks(e, X, M, F, n_quad, acc_pair, acc_phi, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction kernel launch");
     ce = launch_int_finalize(acc_pair, acc_phi, M, F, e->prep.bias, phi_ij, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction finalize launch");
@@ -588,7 +665,7 @@ extern "C" qts_status qts_shap_interactions_noalloc(qts_ensemble* e, const float
     // the array keeps the previous call's sums: clear the part this call uses
     cudaError_t ce = cudaMemsetAsync(scratch, 0, sizeof(double) * (size_t)need, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "scratch clear");
-    ce = launch_int_buckets(e, X, M, F, nq, acc_pair, acc_phi, s);
+    ce = launch_int_buckets(e, (const Rec32*)e->d_rec, e->prep.buckets, X, M, F, nq, acc_pair, acc_phi, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction kernel launch");
     ce = launch_int_finalize(acc_pair, acc_phi, M, F, e->prep.bias, phi_ij, s);
     if (ce != cudaSuccess) return cuda_fail(ce, "interaction finalize launch");

@@ -207,9 +207,11 @@ struct qts_ensemble {
     int64_t* d_dfs_off = nullptr;     // per tree, n_trees + 1
     int dfs_levels = 0;               // internal-node depth + 1
     int64_t dfs_records = 0;
-    // sizes of the path tables with sibling leaves merged (qts_get_batch_info)
+    // sizes of the path tables with sibling leaves merged (qts_get_batch_info), and
+    // their records, uploaded by the first pairwise call that runs on them
     qts::Prepared pair_sizes;
     bool pair_ready = false;
+    qts::Rec32* d_pair_rec = nullptr;
     // block tables of the FP32 first-order and adjoint passes, built on the
     // first call that needs them (the adjoint's part on the first such call)
     std::vector<qts::BlockBucket> blk;
@@ -240,7 +242,7 @@ bool is_capturing(cudaStream_t st);
 qts_status upload(qts_ensemble* e);
 void release_device(qts_ensemble* e);
 void release_dfs(qts_ensemble* e);      // drop the depth-first program (rebuilt on demand)
-qts_status ensure_pair_sizes(qts_ensemble* e);
+qts_status ensure_pairs(qts_ensemble* e, bool records);
 // build the block tables, with grad those of the adjoint too
 void build_blocks(const qts_ensemble* e, bool grad, BlockHost* out);
 qts_status ensure_blocks(qts_ensemble* e, bool grad);

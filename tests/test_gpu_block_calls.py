@@ -228,3 +228,37 @@ def test_small_ensemble_many_samples(qts, T, depth, F, M, missing):
         assert rel_err_rows(phi[torch.from_numpy(rows).cuda()].cpu().numpy(), ref).max() <= TOL32, n_quad
         assert rel_err_rows(phi[:16].cpu().numpy(), few.cpu().numpy()).max() <= TOL32
     E.close()
+
+
+# (trees, 0: a chain, its depth, F, M): pairs without a tile in shared memory (F = 60, at a
+# mean width on either side of the one-row line) and with one, wide and padded widths,
+# few and many samples
+PAIR_ROUTES = [(4, 5, 60, 1), (4, 5, 60, 40), (2, 17, 60, 1), (2, 17, 60, 33), (2, 12, 24, 4), (2, 12, 24, 5),
+               (2, 12, 24, 40), (0, 30, 40, 5), (0, 30, 40, 40), (1, 4, 10, 16), (1, 4, 10, 17), (3, 7, 48, 40), (0, 30, 60, 5), (0, 30, 60, 40)]
+
+
+@pytest.mark.parametrize("T,depth,F,M", PAIR_ROUTES)
+@pytest.mark.parametrize("kind", ["clean", "missing", "categories"])
+def test_pairs_on_either_tables(qts, T, depth, F, M, kind):
+    import torch
+
+    from helpers import caterpillar_ensemble
+
+    ens = (synth.grow(9950 + depth, T, depth, F, 600, 0.5, min_rows=3) if T else
+           caterpillar_ensemble(9950, [depth, 18, 4], F))
+    X = synth.normal(9950 + depth, synth.STREAM_X, (M, F))
+    if kind == "categories":
+        cats = list(range(0, F, 3))
+        ens = synth.make_categorical(ens, cats, 6, 9951)
+        X = synth.categorical_columns(X, cats, 6, 9952)
+    elif kind == "missing":
+        X[np.random.default_rng(9950).random(X.shape) < 0.2] = np.nan
+    E = qts.Ensemble.from_arrays(ens)
+    sii, phi = oracle.sii_exact(ens, X)
+    ref = oracle.interaction_matrix(sii, phi)
+    scale = np.maximum(np.abs(phi.sum(1)), np.abs(phi[:, :-1]).max(1))
+    for n_quad in (qts.EXACT_NODES, 16, 17):  # 17: an odd rule
+        got = qts.shap_interactions(E, torch.from_numpy(X).cuda(), n_quad).cpu().numpy().astype(np.float64)
+        E.sync_status()
+        assert (np.abs(got - ref).reshape(M, -1).max(1) / scale).max() <= TOL32, n_quad
+    E.close()
