@@ -314,8 +314,10 @@ typedef struct qts_request {
  * cost is consumed through an atomic counter, and one pass over each (sample,
  * block) produces both phi and the adjoint (the forward product terms are a subset
  * of the adjoint's).  The whole call (one preparation kernel, the persistent
- * kernels as parallel branches, the adjoint epilogue) is captured once into a CUDA graph keyed by the request set and
- * replayed on later calls with the same requests.  Each ensemble may appear in
+ * kernels as parallel branches, the adjoint epilogue) is captured once into a CUDA
+ * graph keyed by the request set and replayed on later calls with the same
+ * requests.  A forward-only request that fills the chip by itself runs
+ * qts_shap_values' kernels as a branch of the graph instead of items.  Each ensemble may appear in
  * at most one request of a call.  FP32 ensembles only.  n_quad as
  * qts_shap_values; the graph holds one persistent launch per (register class,
  * accumulator-tile size, rule).

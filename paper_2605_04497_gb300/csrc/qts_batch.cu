@@ -647,6 +647,18 @@ static void request_segments(const qts_request& R, char* base, int req, int n_qu
     }
 }
 
+// A forward-only request that fills the chip by itself: the forward's own kernels, with
+// phi tiles of the warps' own and a variant without NaN tests, in place of items.  8 trees of
+// depth 18, F = 24, 2,000 samples: 6,934 us as items, 3,021 here (5,782 on the path
+// tables); four of 100 trees of depth 8, F = 30, 2,000 samples 1,606 -> 755.  Below about 25 us
+// of work its launches would weigh: small requests share the persistent kernels.
+static bool forward_alone(const qts_request& R) {
+    if (R.grad_phi || R.M <= 0) return false;
+    double work = 0.0;
+    for (const BlockBucket& b : R.ens->blk) work += (double)b.n * blk_cost(b.D, b.h);
+    return work * (double)((R.M + 31) / 32) >= 2e7;
+}
+
 struct LaunchHost {
     int cls, nq, npad, pad;
     bool sp;
@@ -724,6 +736,7 @@ static qts_status build_plan(int n, const qts_request* reqs, int n_quad, BatchPl
     std::vector<SegHost> segs;
     std::vector<ReqDev> rd(n);
     std::vector<ReqWork> rw(n);
+    std::vector<int> alone;  // requests that run the forward's own kernels
     WorkBlocks nb;
     const size_t flag_bytes = 256 * ((sizeof(int) * (size_t)n + 255) / 256);
     const size_t gb_bytes = 256 * ((sizeof(double) * (size_t)n + 255) / 256);
@@ -731,8 +744,13 @@ static qts_status build_plan(int n, const qts_request* reqs, int n_quad, BatchPl
         const qts_request& R = reqs[r];
         char* ws = (char*)R.ens->d_work;
         rw[r] = request_work(R, ws);
+        if (forward_alone(R)) {
+            rw[r].Mpad = 0;  // no transposed copy
+            if (!ov) alone.push_back(r);
+        } else if (R.M > 0) {
+            request_segments(R, ws, r, n_quad, ov, &segs);
+        }
         number_work(rw[r], &nb);
-        if (R.M > 0) request_segments(R, ws, r, n_quad, ov, &segs);
     }
     const std::vector<LaunchHost> launches = order_segments(segs, (size_t)1 << 30);
     auto pad = [](size_t v) { return (v + 255) / 256 * 256; };
@@ -766,7 +784,7 @@ static qts_status build_plan(int n, const qts_request* reqs, int n_quad, BatchPl
     // capture: preparation, persistent kernels, epilogue.  The persistent kernels
     // (and the gradients' start values) are branches of the graph, so one class's
     // last items run beside the next one's first.
-    std::vector<cudaStream_t> side(std::min<size_t>(launches.size(), kBatchBranches), nullptr);
+    std::vector<cudaStream_t> side(std::min<size_t>(launches.size() + alone.size(), kBatchBranches), nullptr);
     std::vector<cudaEvent_t> done(side.size() + 1, nullptr);
     for (auto& x : side)
         if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
@@ -810,6 +828,10 @@ static qts_status build_plan(int n, const qts_request* reqs, int n_quad, BatchPl
         a.reqs = d_reqs;
         err = launch_ordered(launches[c], a, d_cnt + c, side[c % side.size()]);
         ++kernels;
+    }
+    for (size_t i = 0; i < alone.size() && err == cudaSuccess; ++i) {
+        const qts_request& R = reqs[alone[i]];
+        err = launch_fwd_blocks(R.ens, R.X, R.M, R.F, n_quad, R.phi, side[(launches.size() + i) % side.size()], &kernels);
     }
     work(batch_bias_kernel, nb.bias, cap);
     for (size_t b = 0; b < side.size(); ++b) {
@@ -966,7 +988,7 @@ extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, i
     std::vector<double> work(kMaxD + 1, 0.0);
     std::vector<char> packed(kMaxD + 1, 0);
     for (const auto& R : sub) {
-        if (R.M <= 0) continue;
+        if (R.M <= 0 || forward_alone(R)) continue;
         for (const BlockBucket& b : R.ens->blk) {
             work[b.D] += (double)R.M * (double)b.n * blk_cost(b.D, b.h);
             if (R.grad_phi && b.D <= 16) packed[b.D] = 1;

@@ -246,7 +246,7 @@ cudaError_t launch_phi_init(double* phi, int64_t M, int F, double bias, cudaStre
 static double fb_least(int F) { return 200.0 * (F + 40); }
 
 cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* phi,
-                              cudaStream_t st) {
+                              cudaStream_t st, int* kernels) {
     if (M <= 0) return cudaSuccess;
     const int64_t tiles = (M + 31) / 32;
     double total = 0.0;
@@ -267,6 +267,7 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
                     pick[n_pick++] = &b;
                 }
             if (n_pick == 0) continue;
+            if (kernels) ++*kernels;
             if (!make_quad(nq, &a.q, nullptr, 2)) return cudaErrorInvalidValue;
             const int np = fb_np(cls, a.q.n_pad);
             if (fwd_own_wins(pick, n_pick, M, F)) {

@@ -262,3 +262,39 @@ def test_pairs_on_either_tables(qts, T, depth, F, M, kind):
         E.sync_status()
         assert (np.abs(got - ref).reshape(M, -1).max(1) / scale).max() <= TOL32, n_quad
     E.close()
+
+
+def test_large_forward_only_requests_in_a_batch(qts):
+    """Forward-only requests that fill the chip run the forward's own kernels inside the
+    batch's graph, beside small ones and one with gradients; replays start from
+    new inputs."""
+    import torch
+
+    sizes = [(60, 8, 20, 3000), (5, 4, 6, 40), (30, 13, 130, 1500), (20, 6, 12, 200)]
+    items, hosts = [], []
+    for i, (T, depth, F, M) in enumerate(sizes):
+        ens = synth.grow(9960 + i, T, depth, F, 5000, 0.5, min_rows=3)
+        X = synth.normal(9960 + i, synth.STREAM_X, (M, F))
+        X[::7, 0] = np.nan
+        G = torch.from_numpy(synth.normal(9960, synth.STREAM_GRAD, (M, F + 1))).cuda() if i == 3 else None
+        items.append(_request(qts, qts.Ensemble.from_arrays(ens), torch.from_numpy(X).cuda(), G))
+        hosts.append(ens)
+    reqs = qts.make_requests(items)
+    rows = np.arange(0, 40)
+    for n_quad in (8, qts.EXACT_NODES):
+        for _ in range(2):
+            qts.batched_fwd_bwd(reqs, n_quad)
+            assert qts.batched_kernel_count() > 4
+            for ens, it in zip(hosts, items):
+                it["ens"].sync_status()
+                ref = oracle.shap_exact(ens, it["X"].cpu().numpy()[rows])
+                assert rel_err_rows(it["phi"][:40].cpu().numpy(), ref).max() <= TOL32
+                last = qts.shap_values(it["ens"], it["X"][-16:].contiguous(), n_quad)
+                assert rel_err_rows(it["phi"][-16:].cpu().numpy(), last.cpu().numpy()).max() <= TOL32
+                it["X"].mul_(-1.0)
+    assert qts.batched_autotune(reqs, 8, max_samples=0)
+    qts.batched_fwd_bwd(reqs)
+    for ens, it in zip(hosts, items):
+        ref = oracle.shap_exact(ens, it["X"].cpu().numpy()[rows])
+        assert rel_err_rows(it["phi"][:40].cpu().numpy(), ref).max() <= TOL32
+        it["ens"].close()
