@@ -330,10 +330,10 @@ qts_status qts_batched_fwd_bwd(int32_t n_requests, const qts_request *reqs, int3
  * set of requests by timing its persistent kernel on the requests' own data (the
  * autotuner of the batched form; the paper has no batching).  For every block
  * width (shared elements) that carries at least 1% of the batch's work it times,
- * with that width's work items alone in the launch, 64, 256, 1,024 and 2,048 blocks
- * per work item and, where the pass holds two samples per lane, the sample mapping
- * (each warp its own 64 samples, or the thread block's warps sharing 64 samples and
- * splitting the blocks), and keeps the fastest.  The
+ * with that width's work items alone in the launch, the blocks per work item (the
+ * default rule, 64, 256, 1,024 and 2,048) and, where the pass holds two samples per
+ * lane, the sample mapping (each warp its own 64 samples, or the thread block's
+ * warps sharing 64 samples and splitting the blocks), and keeps the fastest.  The
  * choices are stored in each request's ensemble and used by later batched
  * calls that include it (their cached graphs are rebuilt).
  *   reqs, n, n_quad  as qts_batched_fwd_bwd; the requests' outputs are
@@ -341,7 +341,8 @@ qts_status qts_batched_fwd_bwd(int32_t n_requests, const qts_request *reqs, int3
  *   max_samples      time on the first min(M, max_samples) samples of each
  *                    request (0: all)
  *   chosen           host, 3 * (QTS_MAX_UNIQUE_FEATURES_PER_PATH + 1) int32 or
- *                    NULL: for width D, [3D] blocks per item, [3D + 1] mapping
+ *                    NULL: for width D, [3D] blocks per item (the rule's for these
+ *                    requests where it stays), [3D + 1] mapping
  *                    (2 or 3, 0 where one sample per lane), [3D + 2] 0 (all
  *                    thread blocks that fit an SM); 0 for untuned widths
  * Synchronous on `stream`.  Errors as qts_batched_fwd_bwd.
@@ -384,9 +385,11 @@ qts_status qts_batched_last_kernel_ms(float *ms);
 
 /*
  * qts_autotune - time candidate launch configurations (work per thread block of
- * the forward) for this ensemble and sample count on `stream`,
- * keep the fastest in the ensemble, and, if cache_path is not NULL, merge the
- * result into that JSON file keyed by (bucket width, F range, M range).
+ * the forward, the default rule among them) for this ensemble and sample count on
+ * `stream`, keep the fastest in the ensemble, and, if cache_path is not NULL, merge
+ * the result into that JSON file keyed by (bucket width, range of the ensemble's
+ * work, F range, M range).  Entries that earlier versions wrote are kept in the file
+ * and not used.
  * X: device M x F.  Synchronous.  Scratch output is allocated internally.
  */
 qts_status qts_autotune(qts_ensemble *ens, const float *X, int64_t M, int32_t F,

@@ -562,9 +562,9 @@ static ReqDev request_dev(const ReqWork& w, const qts_ensemble* e) {
     return {w.XT, w.G ? w.GT : nullptr, w.phi, w.M, w.Mpad, w.F, e->prep.has_cat ? 1 : 0, w.flag, e->d_status};
 }
 
-// Per-width launch choices that override the ensembles' own while tuning:
-// blocks per work item and packed sample mapping (0: keep), and optionally only
-// the buckets of one width.
+// Per-width launch choices that override the ensembles' own while tuning: blocks per
+// work item (0: the default rule), packed sample mapping (0: keep), and optionally
+// only the buckets of one width.
 struct BatchOverride {
     int paths[kMaxD + 1];
     int mode[kMaxD + 1];
@@ -607,7 +607,6 @@ static void request_segments(const qts_request& R, char* base, int req, int n_qu
     const bool grad = R.grad_phi != nullptr;
     double* g = grad ? (double*)base + kGradHead : nullptr;
     for (const BlockBucket& b : e->blk) {
-        if (ov && ov->only_width > 0 && b.D != ov->only_width) continue;
         const Tune& tn = e->tune[b.D];
         SegHost s;
         s.cls = batch_class(b.D, b.h);
@@ -626,7 +625,7 @@ static void request_segments(const qts_request& R, char* base, int req, int n_qu
         s.d.item_begin = 0;
         s.d.D = b.D;
         s.d.h = b.h;
-        s.d.per_item = ov && ov->paths[b.D] ? ov->paths[b.D] : tn.bt_paths;
+        s.d.per_item = ov ? ov->paths[b.D] : tn.bt_paths;
         s.d.n_tiles = (int)((R.M + per - 1) / per);
         s.d.req = req;
         s.d.mode = mode;
@@ -752,6 +751,10 @@ static qts_status build_plan(int n, const qts_request* reqs, int n_quad, BatchPl
         }
         number_work(rw[r], &nb);
     }
+    default_items(segs);  // from the whole launch, also where one width of it is timed
+    if (ov && ov->only_width > 0)
+        segs.erase(std::remove_if(segs.begin(), segs.end(), [&](const SegHost& s) { return s.d.D != ov->only_width; }),
+                   segs.end());
     const std::vector<LaunchHost> launches = order_segments(segs, (size_t)1 << 30);
     auto pad = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t seg_bytes = pad(sizeof(SegDev) * std::max<size_t>(segs.size(), 1));
@@ -958,15 +961,21 @@ extern "C" qts_status qts_batched_fwd_bwd(int32_t n, const qts_request* reqs, in
 namespace qts {
 
 // Device time of the persistent kernels of one plan built for `reqs` with the
-// override `ov` (second of two launches); the plan is destroyed afterwards.
+// override `ov` (the faster of two launches after a first); the plan is destroyed
+// afterwards.
 static qts_status time_plan(int n, const qts_request* reqs, int n_quad, const BatchOverride& ov,
                             cudaStream_t cap, cudaStream_t st, float* ms) {
     auto* plan = new BatchPlan();
     qts_status s = build_plan(n, reqs, n_quad, plan, cap, &ov);
     cudaError_t ce = cudaSuccess;
-    for (int k = 0; k < 2 && s == QTS_OK && ce == cudaSuccess; ++k) ce = cudaGraphLaunch(plan->exec, st);
-    if (s == QTS_OK && ce == cudaSuccess) ce = cudaEventSynchronize(plan->ev1);
-    if (s == QTS_OK && ce == cudaSuccess) ce = cudaEventElapsedTime(ms, plan->ev0, plan->ev1);
+    *ms = 1e30f;
+    for (int k = 0; k < 3 && s == QTS_OK && ce == cudaSuccess; ++k) {
+        float t = 0.f;
+        ce = cudaGraphLaunch(plan->exec, st);
+        if (ce == cudaSuccess) ce = cudaEventSynchronize(plan->ev1);
+        if (ce == cudaSuccess) ce = cudaEventElapsedTime(&t, plan->ev0, plan->ev1);
+        if (k > 0) *ms = std::min(*ms, t);
+    }
     if (s == QTS_OK && ce != cudaSuccess) s = cuda_fail(ce, "batched tuning run");
     cudaStreamSynchronize(st);
     destroy_plan(plan);
@@ -1008,10 +1017,11 @@ extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, i
         BatchOverride ov;
         std::memset(&ov, 0, sizeof(ov));
         ov.only_width = D;
+        // the defaults first: they stay unless another choice is faster
         float best = 1e30f;
-        for (int mode : {2, 3}) {
-            if (mode == 3 && !packed[D]) continue;
-            for (int paths : {64, 256, 1024, 2048}) {
+        for (int mode : {3, 2}) {
+            if (mode == 2 && !packed[D]) continue;
+            for (int paths : {0, 64, 256, 1024, 2048}) {
                 ov.paths[D] = paths;
                 ov.mode[D] = packed[D] ? mode : 0;
                 float ms = 0.f;
@@ -1038,12 +1048,23 @@ extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, i
         ++e->tune_gen;
         batch_forget(e);
     }
-    if (chosen)
+    if (chosen) {
+        // widths that keep the default rule report what it gives for these requests
+        std::vector<SegHost> segs;
+        BatchOverride rule;
+        std::memset(&rule, 0, sizeof(rule));
+        for (const auto& R : sub)
+            if (R.M > 0 && !forward_alone(R)) request_segments(R, (char*)R.ens->d_work, 0, n_quad, &rule, &segs);
+        default_items(segs);
+        for (int D : widths)
+            for (const SegHost& s : segs)
+                if (best_paths[D] == 0 && s.d.D == D) best_paths[D] = s.d.per_item;
         for (int D = 0; D <= kMaxD; ++D) {
             chosen[3 * D] = best_paths[D];
             chosen[3 * D + 1] = best_mode[D];
             chosen[3 * D + 2] = 0;
         }
+    }
     return QTS_OK;
 } QTS_ENTRY_END
 

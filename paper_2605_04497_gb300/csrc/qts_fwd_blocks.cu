@@ -303,10 +303,11 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
             // keeps the tiles' set-up and flush small beside it as far as that leaves
             // two rounds of the thread blocks that fit
             const int resident = std::min(cls <= 3 ? 4 : 2, std::max(1, (int)(kSmemMax / (smem + 1024))));
-            const double wide = std::min(fb_least(F), total / (2.0 * num_sms() * resident));
-            const double share = e->tune[0].bpaths > 0
-                                     ? kBlkUnit * e->tune[0].bpaths
-                                     : std::min(400e3, std::max({4e3, wide, total / (8.0 * num_sms() * 4)}));
+            const double two_rounds = total / (2.0 * num_sms() * resident);
+            // a tuned share (of another call's samples, maybe) leaves two rounds too
+            const double share = e->bpaths > 0 ? std::min(kBlkUnit * e->bpaths, std::max(4e3, two_rounds))
+                                               : std::min(400e3, std::max({4e3, std::min(fb_least(F), two_rounds),
+                                                                           total / (8.0 * num_sms() * 4)}));
             for (int k = 0; k < n_pick; ++k) {
                 const BlockBucket* b = pick[k];
                 FbSeg& sg = a.seg[a.n_seg++];

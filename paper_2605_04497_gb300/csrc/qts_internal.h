@@ -150,17 +150,12 @@ struct BlockDev {
     double *bias_leaf = nullptr, *bias_z = nullptr;
 };
 
-// Launch tuning of one bucket width.
+// Launch parameters of one bucket width.
 struct Tune {
+    // path kernels of the FP64 adjoint
     int warps = 4;        // warps per block (samples are shared, paths split)
     int paths = 128;      // paths per block (chunk)
     int sub = 32;         // paths per staged sub-chunk
-    int np = 8;           // nodes per register pass (8, 4 or 2)
-    int bpaths = 0;       // block-table forward: work per thread block in units of an
-                          // average block (kBlkUnit); 0: chosen from the call's work
-    int priv = 1;         // forward: 1 each warp owns a sample tile (when it fits), 2 the
-                          // warps share one and split the paths with a phi tile each,
-                          // 0 they share one phi tile (shared-memory atomics)
     // choices of the batched-launch tuner (0: not tuned, the launch's default)
     int bt_paths = 0;     // blocks per work item of the persistent batched kernel
     int bt_mode = 0;      // sample mapping of the packed fused pass: 2 (64 samples
@@ -221,7 +216,8 @@ struct qts_ensemble {
     std::mutex blk_mu;                // one thread builds them
     // per-width launch tuning (index = bucket width)
     qts::Tune tune[qts::kMaxD + 1];
-    bool tuned = false;
+    int bpaths = 0;                   // the forward's work per thread block in units of an average
+                                      // block (kBlkUnit); 0: chosen from the call's work
     uint32_t tune_gen = 0;            // bumped by every tuning call (cached batched graphs key on it)
 };
 

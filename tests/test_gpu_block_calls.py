@@ -298,3 +298,34 @@ def test_large_forward_only_requests_in_a_batch(qts):
         ref = oracle.shap_exact(ens, it["X"].cpu().numpy()[rows])
         assert rel_err_rows(it["phi"][:40].cpu().numpy(), ref).max() <= TOL32
         it["ens"].close()
+
+
+def test_tuning_cache_of_an_earlier_format(qts, tmp_path):
+    """Entries of another meaning are kept in the file and not used; a fitting entry is
+    taken only with a value that the tuner writes."""
+    import json
+    import math
+
+    import torch
+
+    ens = synth.grow(9970, 12, 5, 9, 2000, 0.5, min_rows=3)
+    E = qts.Ensemble.from_arrays(ens)
+    Xh = synth.normal(9970, synth.STREAM_X, (300, 9))
+    X = torch.from_numpy(Xh).cuda()
+    path = tmp_path / "tune.json"
+    old = {f"{D}|{int(math.log2(9))}|{int(math.log2(300))}": [8, 2048, 32, 8, 2147483647, 0]
+           for D, _ in E.info()["buckets"]}
+    path.write_text(json.dumps(old))
+    qts.autotune(E, X, str(path))
+    data = json.loads(path.read_text())
+    new = {k: v for k, v in data.items() if k not in old}
+    assert {k: v for k, v in data.items() if k in old} == old
+    assert len(new) == len(old) and all(v in ([0], [128], [256], [512], [1024], [2048]) for v in new.values())
+    # a spoiled entry under the current key is timed anew
+    path.write_text(json.dumps({k: [2147483647] for k in new}))
+    qts.autotune(E, X, str(path))
+    assert all(v[0] <= 2048 for v in json.loads(path.read_text()).values())
+    phi = qts.shap_values(E, X)
+    E.sync_status()
+    assert rel_err_rows(phi.cpu().numpy(), oracle.shap_exact(ens, Xh)).max() <= TOL32
+    E.close()
