@@ -196,6 +196,8 @@ qts_status ensure_pairs(qts_ensemble* e, bool records) {
 qts_status ensure_blocks(qts_ensemble* e, bool grad) {
     std::lock_guard<std::mutex> lk(e->blk_mu);
     if (e->blk_ready && (!grad || e->blk_grad_ready)) return QTS_OK;
+    grad = grad || e->wants_grad;  // (!blk_ready: a refit step's forward comes first)
+    e->wants_grad = grad;
     if (grad && e->n_nodes >= ((int64_t)1 << 31)) return fail(QTS_ERR_UNSUPPORTED, "gradients of 2^31 nodes or more");
     BlockHost H;
     build_blocks(e, grad, &H);

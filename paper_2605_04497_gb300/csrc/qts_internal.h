@@ -213,6 +213,8 @@ struct qts_ensemble {
     qts::BlockDev blkdev;
     int64_t n_blocks = 0, n_blk_slots = 0;
     bool blk_ready = false, blk_grad_ready = false;
+    bool wants_grad = false;          // an adjoint call has been made: build its part at once
+                                      // with the next tables (after qts_update_params)
     std::mutex blk_mu;                // one thread builds them
     // per-width launch tuning (index = bucket width)
     qts::Tune tune[qts::kMaxD + 1];

@@ -480,7 +480,7 @@ qts_status prepare(int32_t n_trees, const int64_t* off, const int32_t* left, con
         run_threads(nth, [&](int k) {
             extract_trees(cut[k], cut[k + 1], off, left, right, feature, thr, defl, z, leaf, is_cat, cat_left, pairs,
                           &outs[k]);
-        });
+        }, nth > 1 ? 0 : 1);
     }
     for (auto& o : outs)
         if (o.st != QTS_OK) { *err = o.err; return o.st; }
