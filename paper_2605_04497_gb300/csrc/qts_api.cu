@@ -256,7 +256,7 @@ bool is_capturing(cudaStream_t st) {
 // A captured call leaves the workspace's address in the caller's graph, which may be
 // replayed after any later call: such a workspace is never freed before the
 // ensemble, a call that outgrows it gets a new one beside it.
-qts_status ensure_workspace(qts_ensemble* e, size_t bytes, cudaStream_t st) {
+qts_status ensure_workspace_uncaptured(qts_ensemble* e, size_t bytes) {
     if (bytes > e->work_bytes) {
         if (e->d_work) {
             batch_forget(e);
@@ -277,8 +277,13 @@ qts_status ensure_workspace(qts_ensemble* e, size_t bytes, cudaStream_t st) {
         }
         e->work_bytes = want;
     }
-    if (!e->work_captured && is_capturing(st)) e->work_captured = true;
     return QTS_OK;
+}
+
+qts_status ensure_workspace(qts_ensemble* e, size_t bytes, cudaStream_t st) {
+    const qts_status r = ensure_workspace_uncaptured(e, bytes);
+    if (r == QTS_OK && !e->work_captured && is_capturing(st)) e->work_captured = true;
+    return r;
 }
 
 // The device failure path on demand: one block waits, bounded, on an mbarrier

@@ -870,7 +870,7 @@ namespace qts {
 
 // Argument checks shared by the batched call and its tuner; grows every
 // request's workspace to what the batched launch needs.
-static qts_status check_batch(int32_t n, const qts_request* reqs, int32_t n_quad, cudaStream_t stream) {
+static qts_status check_batch(int32_t n, const qts_request* reqs, int32_t n_quad) {
     if (n < 1 || !reqs) return fail(QTS_ERR_ARG, "no requests");
     for (int r = 0; r < n; ++r) {
         const qts_request& R = reqs[r];
@@ -889,7 +889,8 @@ static qts_status check_batch(int32_t n, const qts_request* reqs, int32_t n_quad
         const qts_request& R = reqs[r];
         qts_status st = ensure_blocks(R.ens, R.grad_phi != nullptr);
         if (st != QTS_OK) return st;
-        st = ensure_workspace(R.ens, batch_work(R.ens, R.M, R.F, R.grad_phi != nullptr).total, stream);
+        // (a graph launch cannot be captured, so the workspace stays the library's)
+        st = ensure_workspace_uncaptured(R.ens, batch_work(R.ens, R.M, R.F, R.grad_phi != nullptr).total);
         if (st != QTS_OK) return st;
     }
     return QTS_OK;
@@ -900,7 +901,7 @@ static qts_status check_batch(int32_t n, const qts_request* reqs, int32_t n_quad
 extern "C" qts_status qts_batched_fwd_bwd(int32_t n, const qts_request* reqs, int32_t n_quad,
                                           qts_stream_t stream) try {
     {
-        const qts_status st = check_batch(n, reqs, n_quad, (cudaStream_t)stream);
+        const qts_status st = check_batch(n, reqs, n_quad);
         if (st != QTS_OK) return st;
     }
     std::vector<uint64_t> key;
@@ -986,7 +987,7 @@ static qts_status time_plan(int n, const qts_request* reqs, int n_quad, const Ba
 
 extern "C" qts_status qts_batched_autotune(int32_t n, const qts_request* reqs, int32_t n_quad, int64_t max_samples,
                                            int32_t* chosen, qts_stream_t stream) try {
-    qts_status st = check_batch(n, reqs, n_quad, (cudaStream_t)stream);
+    qts_status st = check_batch(n, reqs, n_quad);
     if (st != QTS_OK) return st;
     if (max_samples < 0) return fail(QTS_ERR_ARG, "max_samples must be >= 0");
     std::vector<qts_request> sub(reqs, reqs + n);

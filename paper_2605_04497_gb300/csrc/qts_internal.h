@@ -234,6 +234,7 @@ namespace qts {
 void set_error(const std::string& msg);
 qts_status fail(qts_status st, const std::string& msg);
 qts_status cuda_fail(cudaError_t e, const char* what);
+qts_status ensure_workspace_uncaptured(qts_ensemble* e, size_t bytes);
 // At least `bytes` of workspace for a call on `st`.
 qts_status ensure_workspace(qts_ensemble* e, size_t bytes, cudaStream_t st);
 bool is_capturing(cudaStream_t st);
