@@ -159,8 +159,10 @@ qts_status qts_update_params(qts_ensemble *ens, const float *z, const float *lea
  *           (the bias, so that sum_f phi[s][f] = f(x_s))
  * Per-path arithmetic is FP32 (FP64 with QTS_FLAG_FP64); contributions are
  * accumulated in FP32 (FP64) within a thread block, then in FP64 across thread
- * blocks.  With M <= 16 lanes are (block, sample) pairs instead of one sample per
- * lane.
+ * blocks.  A thread block's FP32 sums cover at most 8,192 subtrees of up to eight
+ * leaves (2,048 in a batched or adjoint call), a quarter of them in each warp's own
+ * sums as far as these fit shared memory.  With M <= 16 lanes are (block, sample)
+ * pairs instead of one sample per lane.
  * Runs on a second set of tables in which a small subtree's leaves (up to
  * eight) are evaluated together against the merged elements they share; it is
  * built by the first call that needs it (host preparation, cudaMalloc and copies

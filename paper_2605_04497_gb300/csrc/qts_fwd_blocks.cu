@@ -316,7 +316,8 @@ cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, 
                 sg.D = b->D;
                 sg.h = b->h;
                 sg.cta_begin = ctas;
-                const int64_t per = std::max<int64_t>(kFbWarps, (int64_t)(share / blk_cost(b->D, b->h)));
+                const int64_t per = std::min<int64_t>(
+                    kMostBlocks, std::max<int64_t>(kFbWarps, (int64_t)(share / blk_cost(b->D, b->h))));
                 sg.per_cta = (int32_t)((per + kFbWarps - 1) / kFbWarps * kFbWarps);
                 ctas += (b->n + sg.per_cta - 1) / sg.per_cta * tiles;
             }

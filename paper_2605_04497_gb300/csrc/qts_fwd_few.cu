@@ -188,9 +188,10 @@ cudaError_t launch_fwd_few(const qts_ensemble* e, const float* X, int64_t M, int
                 // one round of the thread block's lanes, or, for large
                 // ensembles, what makes about four thread blocks per SM
                 const int64_t round = (int64_t)kFewWarps * group;
-                const int64_t rounds = std::max<int64_t>(1, b.n / (round * 4 * num_sms()));
+                const int64_t rounds =
+                    std::min<int64_t>(kMostBlocks / round, std::max<int64_t>(1, b.n / (round * 4 * num_sms())));
                 FewSeg& sg = a.seg[a.n_seg++];
-                sg = {e->blkdev.rec + b.rec_off, b.n, ctas, (int32_t)std::min<int64_t>(round * rounds, 1 << 30), b.D,
+                sg = {e->blkdev.rec + b.rec_off, b.n, ctas, (int32_t)(round * rounds), b.D,
                       b.h};
                 ctas += (b.n + sg.per_cta - 1) / sg.per_cta;
             }

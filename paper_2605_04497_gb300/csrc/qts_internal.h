@@ -287,6 +287,7 @@ cudaError_t launch_wait_selftest(int* status, cudaStream_t st);
 // first-order values on the block tables: FP32 (any M), FP32 for M <= kFewRows, FP64
 cudaError_t launch_fwd_blocks(const qts_ensemble* e, const float* X, int64_t M, int F, int n_quad, double* phi,
                               cudaStream_t st, int* kernels = nullptr);  // kernels: += launches
+constexpr int64_t kMostBlocks = 8192;  // whose contributions a thread block sums in FP32
 // the same for small ensembles and many samples (qts_fwd_own.cu): the buckets of one
 // class `cls` of qts_fwd_blocks.cu that take a rule of nq points, np of them per pass
 constexpr int kFbSegs = 24;  // buckets of a class: at most six widths of four heights
