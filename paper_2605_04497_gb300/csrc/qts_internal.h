@@ -104,10 +104,6 @@ struct Prepared {
     // sibling leaves of a numerical split as one path (kPairElem)
     bool pairs = false;
     int64_t n_pair_paths = 0;
-    std::vector<int64_t> pair_leaf2;   // per path: leaf B of a pair, -1 otherwise (path_leaf is A)
-    std::vector<double> pair_zprod2;   // per path: prod of leaf B's merged z (path_zprod is A's)
-    std::vector<double> pair_z;        // per path: z_A, z_B of the pair element
-    std::vector<int64_t> pair_gslot;   // per path: slot of the pair element, -1 otherwise
 };
 
 // Prepare the path tables (host, multi-threaded).  Returns QTS_OK or an error

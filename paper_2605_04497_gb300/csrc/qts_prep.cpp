@@ -524,12 +524,6 @@ qts_status prepare(int32_t n_trees, const int64_t* off, const int32_t* left, con
     P->slot_edge_begin.assign((size_t)slot_total + 1, 0);
     P->slot_zexcl.assign((size_t)slot_total, 0.0);
     P->pairs = pairs;
-    if (pairs) {
-        P->pair_leaf2.assign((size_t)path_total, -1);
-        P->pair_zprod2.assign((size_t)path_total, 0.0);
-        P->pair_z.assign(2 * (size_t)path_total, 0.0);
-        P->pair_gslot.assign((size_t)path_total, -1);
-    }
 
     // fill, bucket by bucket in tree order; first count edges per slot
     std::vector<int64_t> cursor(P->buckets.size());
@@ -554,11 +548,6 @@ qts_status prepare(int32_t n_trees, const int64_t* off, const int32_t* left, con
             if (pr) {
                 P->bias += p.val_a * zprod * p.z_a + p.val_b * zprod * p.z_b;
                 P->path_zprod[gp] = zprod * p.z_a;
-                P->pair_leaf2[gp] = p.leaf2;
-                P->pair_zprod2[gp] = zprod * p.z_b;
-                P->pair_z[2 * gp] = p.z_a;
-                P->pair_z[2 * gp + 1] = p.z_b;
-                P->pair_gslot[gp] = b.slot_base + lp * D + D - 1;
                 ++P->n_pair_paths;
             } else {
                 P->bias += p.val * zprod;
