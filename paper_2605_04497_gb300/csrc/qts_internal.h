@@ -230,9 +230,11 @@ namespace qts {
 void set_error(const std::string& msg);
 qts_status fail(qts_status st, const std::string& msg);
 qts_status cuda_fail(cudaError_t e, const char* what);
-qts_status ensure_workspace_uncaptured(qts_ensemble* e, size_t bytes);
-// At least `bytes` of workspace for a call on `st`.
+// At least `bytes` of workspace for a call that may be under capture on `st`, or
+// for a plan of the library's own (asking a stream is a driver call, which every
+// request of a batched call would make).
 qts_status ensure_workspace(qts_ensemble* e, size_t bytes, cudaStream_t st);
+qts_status ensure_workspace_uncaptured(qts_ensemble* e, size_t bytes);
 bool is_capturing(cudaStream_t st);
 qts_status upload(qts_ensemble* e);
 void release_device(qts_ensemble* e);
